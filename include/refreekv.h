@@ -234,10 +234,8 @@ refree_status refree_compress_layer_inplace(const refree_params *p, const void *
  * while the kept rows of an earlier one are copied.  On the tensor-core path
  * and with a single query row several layers share a launch (as many as the run's
  * length, their size and the workspace suggest), all on the caller's stream; other
- * shapes use two internal streams.  Budgets and rows are those of num_layers calls of
- * refree_compress_layer, up to the rounding of the scores: layers that share a
- * launch are cut over the SMs differently, so a row's sum may be added in another
- * order.
+ * shapes use two internal streams.  Results are bit-identical to num_layers calls of
+ * refree_compress_layer, whatever shares a launch.
  *   q_win, k, v, k_out, v_out, lengths, offsets  HOST arrays of `num_layers`
  *            DEVICE pointers, one per layer, each as in refree_compress_layer;
  *            the arrays themselves are read before the call returns

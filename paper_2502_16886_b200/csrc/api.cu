@@ -49,9 +49,9 @@ Workspace workspace_layout(const refree_params &p, int64_t total_tokens)
     const int64_t rows = G * wc;
     const int64_t tiles = total_tokens / kTile + p.num_seqs;
     size_t off = 0;
-    // partials: per (64 positions, head, row) for the generic path, per (CTA + unit, padded row) for the tensor-core path
+    // partials: per (64 positions, head, row) for the generic path, per (range + unit, column half, padded row) for the tensor-core path
     const int64_t rows_pad = (rows + kTile - 1) / kTile * kTile;
-    const int64_t part_items = std::max<int64_t>((total_tokens / 64 + p.num_seqs) * p.num_kv_heads * rows, (256 + U) * rows_pad);
+    const int64_t part_items = std::max<int64_t>((total_tokens / 64 + p.num_seqs) * p.num_kv_heads * rows, 2 * (256 + U) * rows_pad);
     size_t part_bytes = (size_t)part_items * sizeof(float2);
     if (score_w1_supported(p)) part_bytes = std::max(part_bytes, score_w1_scratch_bytes(p, total_tokens));
     w.part_off = off;   w.part_bytes = align256(part_bytes);                                               off += w.part_bytes;
@@ -561,7 +561,7 @@ BatchLayout batch_layout(const refree_params &p, int64_t total_tokens, int layer
     const int64_t heads = (int64_t)p.num_kv_heads * layers, U = p.num_seqs * heads, tiles = total_tokens / kTile + p.num_seqs;
     const int64_t rows_pad = ((int64_t)(p.num_q_heads / p.num_kv_heads) * p.window + kTile - 1) / kTile * kTile;
     size_t off = 0;
-    b.part_off = off;    b.part_bytes = align256((size_t)((256 + U) * rows_pad) * sizeof(float2)); off += b.part_bytes;
+    b.part_off = off;    b.part_bytes = align256((size_t)(2 * (256 * layers + U) * rows_pad) * sizeof(float2)); off += b.part_bytes;
     b.grp_off = off;     off += align256((size_t)(tiles * heads * 4) * sizeof(GroupPartial));
     b.tickets_off = off; off += align256((size_t)(2 * U) * sizeof(uint32_t));
     b.cut_off = off;     off += align256((size_t)U * sizeof(Cut));
@@ -600,8 +600,9 @@ int w1_batch(const refree_params &p, int64_t total_tokens, int num_layers, size_
 // Layers of a run that one launch scores together.  A launch costs about 22 us beyond its tiles (setup, the first loads,
 // normalisers, the stopping rule, the last CTA of the chain), paid once per group; a group's rows, 2.7 us per layer and
 // item (128 positions of a KV head) of an SM, are moved without scoring beside them at the end of the run.  The sum is
-// smallest at sqrt(8 layers / items per SM) layers.  Measured, 8 KV heads of 256 rows: 16 layers of 8K positions 633 us
-// one by one, 469 in twos, 407 in fours; of 2K positions 343, 313 and 184, 150 in eights; 8 layers of 32K 703 and 673.
+// smallest at sqrt(8 layers / items per SM) layers.  Measured, 8 KV heads of 256 rows: 16 layers of 8K positions 707 us
+// one by one, 527 in twos, 444 in fours, 418 in eights; of 2K positions 390, 341, 247 and 180; 8 layers of 32K 728 one by
+// one, 679 in twos, 716 in fours.
 int run_batch(const refree_params &p, int64_t total_tokens, int num_layers, size_t workspace_bytes, bool copy)
 {
     const double items = (double)(total_tokens / kTile + p.num_seqs) * p.num_kv_heads / sm_count();

@@ -249,12 +249,12 @@ cudaError_t launch_score_tc(const refree_params &p, const void *q_win, const voi
                             int32_t *dev_status, Stream st, GroupPartial *groups = nullptr,
                             int32_t *sel_lengths = nullptr);
 
-// A group of consecutive layers of a run that the same launches score: a unit of the group is (sequence, layer, KV head),
-// and what a launch keeps per unit or per head is laid out with layers x KV heads for the heads.
+// A group of consecutive layers of a run that the same launches score.  What a launch keeps of a layer follows what it
+// keeps of the layer before.
 struct TcGroup {
     int layers;
     const void *q_win[kMaxBatch], *k[kMaxBatch];
-    float2 *part;           // [256 + units, padded rows]: partials between the two passes
+    float2 *part;           // layers x [256 + units of a layer, column half, padded rows]: partials between the two passes
     float *scores;          // [layers x Hkv, total_tokens]
     GroupPartial *groups;   // nullable: records for the stopping rule (position ranking per head)
     // nullable: the launch that finishes the group evaluates the rule too

@@ -6,27 +6,30 @@
 // all of the row, and the column sums need every row's normaliser, so the logits are
 // formed twice (storing them would cost more HBM traffic than K itself):
 //
-//   pass 1  D[row, position] = Q_blk K^T (M = 128 rows, N = 256 positions, two tiles): Z[row] = sum over positions of
-//           2^(y - c[row]) per (CTA, unit); the pairs (c, Z) go to the workspace
+//   pass 1  D[row, position] = Q_blk K_tile^T (M = 128 rows, N = 128 positions): Z[row] = sum over the positions of a
+//           run of tiles of 2^(y - c[row]), per half of a tile's columns; the pairs (c, Z) go to the workspace
 //   pass 2  on entering a unit, L[row] = log2 sum_i 2^(y_i) is merged from those pairs; then D[position, row] =
 //           K_tile Q^T (M = 128 positions, N = up to 256 rows) and
 //           a'[i] = sum over the rows that see i of 2^(y - L[row])  (Eq. 2)
 //
 // Both passes use the same shared-memory images of Q and K (K-major, so either can be the A or the B operand); only
-// the roles swap, which puts each pass's reduction inside a lane.  Every product goes to one of two accumulators of
-// 256 tensor-memory columns, and all sixteen epilogue warps share every product: a warp takes a quarter of the lanes
-// and a quarter of the columns.
+// the roles swap, which puts each pass's reduction inside a lane.
 //
-// Why this form.  N = 256 products take 128 cycles per k-step here (N = 128: 109-116, and twice as many), and the warp
-// that issues them waits about 300 cycles at every barrier, because its loads queue behind the exponentials of the
-// epilogue warps: half as many, wider products keep it ahead of them.  Everything waits like that beside sixteen warps
-// that use the exponential unit, so the epilogue waits as rarely as it can: one barrier per 64 logits of a lane,
-// passed while the last logits of the product before are still being summed.
-// Scoring one layer, measured on one GPU against the form before (pass 1 in N = 128 products on four accumulators, pass
-// 2 in two groups of eight warps): 32K positions, 8 units of 256 rows 72 -> 66 us; 74K positions, 4 heads of 448 rows
-// 134 -> 127; 20K positions, 8 units of 512 rows 84 -> 78.  The exponentials alone take 29, 59 and 38 us.  The rest: the
-// sixteen warps run in step, and between two products all of them do at once what is not exponentials (800 of some 3000
-// cycles); taking the exponentials out, or seven of eight products, changes these times by less than 6 %.
+// Order of the sums.  A budget follows from fp32 scores, and about one unit in 10^4 lies so near a tie that the last bits
+// of a score decide it (two units of 19200: criterion within 4e-9 of the threshold).  So every sum here has one order,
+// whatever else is in the launch: a row's terms inside a run in the order of the tiles, the runs cut at the ranges of a
+// single layer (see Split), records merged in their order, a position's terms by halves of a product's columns.  A layer
+// gets the same bits from every entry point, in every group of layers, with every workspace.
+//
+// Why this form.  The epilogue (a multiply-add, an exponential and an addition per logit and pass) takes longer than the
+// products; the two groups of eight epilogue warps take products in turn and run out of step, so that one sums while the
+// other waits for its next accumulator.  An accumulator is handed back as soon as its last values sit in registers.  In
+// pass 1 a group has two accumulators of 128 columns: pairs of tiles as one N = 256 product per group are held until the
+// second tile's logits are read, and the product that follows comes late (us a pass: four layers of the ragged batch of
+// eight, 448 rows, 757 and 725 as here; eight of 20K positions, 512 rows, 783 and 769; 16 of 8K, 256 rows, 443 and 437).
+// All sixteen warps sharing every product is faster where runs are short (16 layers of 8K 396, of 2K 154 and here 180;
+// eight of 32K 671 and here 681; the ragged batch 738), but takes a row's or position's terms in another order, and
+// layers that share a launch then round differently from the same layers one by one.
 //
 // Persistent CTAs (one per SM) take contiguous ranges of (unit, tile) items; warp 16 issues TMA, warp 17 issues MMA,
 // warps 0-15 are the epilogue, warp 18 moves rows of another layer, warp 19 adds the warps' shares of a column sum,
@@ -54,7 +57,7 @@ constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kMaxRowsTc = 512;
 constexpr int kMaxCtas = 256;
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kZLimit = 1.3292280e36f;         // 2^120: a row sum above this is formed again with a reference of its own
+constexpr float kZLimit = 1.2676506e30f;         // 2^100: a tile sum above this is redone with a fresh reference
 
 // ------------------------------------------------------------------ PTX ------
 __device__ inline uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -146,23 +149,27 @@ __device__ inline void umma_commit(uint64_t *bar)
 // Tensor-memory loads are split into issue and wait so that the next chunk can be
 // in flight while the current one is consumed.  The wait names the destination
 // registers as in/out operands: the compiler must not read them before it.
-#define RF_OUT16(r) "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), \
-                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-#define RF_IO16(r) "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), \
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+#define RF_OUT16(r, o) "=r"(r[o+0]), "=r"(r[o+1]), "=r"(r[o+2]), "=r"(r[o+3]), "=r"(r[o+4]), "=r"(r[o+5]), "=r"(r[o+6]), "=r"(r[o+7]), \
+                       "=r"(r[o+8]), "=r"(r[o+9]), "=r"(r[o+10]), "=r"(r[o+11]), "=r"(r[o+12]), "=r"(r[o+13]), "=r"(r[o+14]), "=r"(r[o+15])
+#define RF_IO16(r, o) "+r"(r[o+0]), "+r"(r[o+1]), "+r"(r[o+2]), "+r"(r[o+3]), "+r"(r[o+4]), "+r"(r[o+5]), "+r"(r[o+6]), "+r"(r[o+7]), \
+                      "+r"(r[o+8]), "+r"(r[o+9]), "+r"(r[o+10]), "+r"(r[o+11]), "+r"(r[o+12]), "+r"(r[o+13]), "+r"(r[o+14]), "+r"(r[o+15])
 __device__ inline void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
                  "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : RF_OUT16(r) : "r"(taddr) : "memory");
+                 : RF_OUT16(r, 0) : "r"(taddr) : "memory");
 }
-__device__ inline void tmem_ld_wait(uint32_t (&r)[16]) { asm volatile("tcgen05.wait::ld.sync.aligned;" : RF_IO16(r) :: "memory"); }
-// Largest value over the lanes of the warp (NaN is skipped).
-__device__ inline float warp_max(float x)
+__device__ inline void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[32])
 {
-    float y;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
-    return y;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : RF_OUT16(r, 0), RF_OUT16(r, 16) : "r"(taddr) : "memory");
+}
+__device__ inline void tmem_ld_wait(uint32_t (&r)[16]) { asm volatile("tcgen05.wait::ld.sync.aligned;" : RF_IO16(r, 0) :: "memory"); }
+__device__ inline void tmem_ld_wait(uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : RF_IO16(r, 0), RF_IO16(r, 16) :: "memory");
 }
 __device__ inline float ex2(float x)
 {
@@ -189,7 +196,7 @@ __host__ __device__ inline uint32_t make_idesc(int n)
 struct TcShape {
     int R;        // query rows per unit: G * window
     int Rpad;     // rows of the shared-memory Q image (multiple of 128)
-    int rblocks;  // 128-row blocks: pass-1 products per pair of tiles (A operands)
+    int rblocks;  // 128-row blocks: pass-1 products per tile (A operands)
     int cblocks;  // pass-2 products per tile: 1 up to 256 rows, else 2
     int ncol;     // pass-2 columns (rows of Q) per product: a multiple of 32, cblocks * ncol >= R
     int stages;   // K tile ring depth
@@ -202,34 +209,33 @@ struct TcShape {
 // requested; the MMA thread and the epilogue warps read it after the barriers that order them behind
 // that request, instead of each walking the item list in registers.
 struct ItemInfo {
-    int32_t u;        // unit = sequence * heads + head; a head is (layer of the group, KV head)
-    int32_t g;        // head
+    int32_t u;        // unit = (layer of the group * sequences + sequence) * KV heads + KV head
+    int32_t g;        // row of the score array: layer * KV heads + KV head
     int32_t n;        // length of the sequence
     int32_t tile;     // tile index inside the sequence
     int32_t ntiles;   // tiles of the sequence
     int32_t pack;     // positions before the sequence in the packed score array
-    int32_t ib;       // index of the unit's first item
+    int32_t ib;       // pass 2: index of the unit's first item; pass 1: index of the run's record
     int32_t flags;    // kNewUnit .. below
 };
-// kNewUnit: first item of its unit in this pass of the CTA (Q is loaded again); kRunFirst / kRunLast: first / last of
-// the CTA's items of the unit; kPassLast: nothing more is loaded in this pass; kTwoTiles: pass 1, a pair of tiles
-// (else the odd last one of a run).
-constexpr int32_t kNewUnit = 1, kRunFirst = 2, kRunLast = 4, kPassLast = 8, kTwoTiles = 16;
+// kNewUnit: first item of its unit in this pass of the CTA (Q is loaded again); kRunLast: the last of a run (pass 1: the
+// tiles of one unit in one range, see Ranges); kPassLast: nothing more is loaded in this pass.
+constexpr int32_t kNewUnit = 1, kRunLast = 2, kPassLast = 4;
 constexpr int kInfoRing = 16;   // the TMA thread runs at most ring stages + accumulators in flight ahead of the epilogue
 // Pass 2: tiles whose column sums wait for the finishing warp.  That warp is slower per tile than the sixteen
 // epilogue warps together while rows are being copied beside them, and catches up under the row pass that follows:
 // the ring is deep enough to let it fall behind instead of holding the epilogue back.
 constexpr int kStageSlots = 8;
 constexpr int kRuleList = 16;   // units whose stopping rule a CTA evaluates when it has left its passes
-constexpr int kCombRows = 256;  // pass 1: rows whose quarters are put together at a time
 struct StageSlot {
     ItemInfo info;                            // the staged tile's record, copied beside its sums
-    float sum[4][kTile];                      // partial column sums, one share per quarter of the rows
+    float sum[4][kTile];                      // partial column sums (share = product * 2 + half of its columns)
 };
 
 struct TcSmemTail {
     uint64_t k_full[4], k_empty[4], q_full, q_empty, epi_bar;
-    uint64_t acc_full[2], acc_empty[2];       // accumulators of 256 tensor-memory columns, taken in turn
+    uint64_t p1_full[4], p1_empty[4];         // pass 1: accumulator (group * 2 + slot), 128 tensor-memory columns each
+    uint64_t p2_full[2], p2_empty[2];         // pass 2: accumulators of 256 columns, one per group of eight warps
     uint64_t chunk_ready[kStageSlots];        // pass 2: every share of a tile has been staged
     uint64_t stage_free[kStageSlots];         // pass 2: the finishing warp has read the slot
     uint64_t c_full[kMaxCopySlots];           // row copy: a piece has landed in its slot
@@ -241,7 +247,6 @@ struct TcSmemTail {
     BlockRuleShared<kThreadsTc> rule;
     alignas(16) ItemInfo info[kInfoRing];
     alignas(16) float lse[kMaxRowsTc];        // pass 2: log2-sum-exp of the unit's rows
-    alignas(16) float2 comb[4][kCombRows];    // pass 1: (c, Z) of the four quarters of the positions at the end of a run
 };
 
 // Per-sequence tables of the CTA behind the tail, sized by the number of sequences:
@@ -252,20 +257,11 @@ struct SeqView {
 };
 
 struct ItemTc {
-    int u, s, g, n, tile_start, tok0, pack;
+    int s, g, n, tok0, pack;
     int tile, ntiles;      // tile index inside the sequence, tiles of the sequence
 };
 
-__device__ inline void fill_seq_fields(ItemTc &it, const SeqView &sv, int Hkv)
-{
-    it.u = it.s * Hkv + it.g;
-    it.n = sv.len[it.s];
-    it.tok0 = sv.start[it.s];
-    it.pack = sv.pack[it.s];
-    it.tile_start = it.tile * kTile;
-}
-
-// Items are ordered (sequence, head, tile): a CTA's consecutive items mostly share a unit.
+// Item of one layer: ordered (sequence, KV head, tile), so consecutive items mostly share a unit.
 __device__ inline ItemTc decode_item_tc(const SeqView &sv, int B, int Hkv, int item)
 {
     int lo = 0, hi = B;
@@ -279,18 +275,23 @@ __device__ inline ItemTc decode_item_tc(const SeqView &sv, int B, int Hkv, int i
     const int rem = item - sv.tiles[lo] * Hkv;
     it.g = rem / it.ntiles;
     it.tile = rem % it.ntiles;
-    fill_seq_fields(it, sv, Hkv);
+    it.n = sv.len[lo];
+    it.tok0 = sv.start[lo];
+    it.pack = sv.pack[lo];
     return it;
 }
 
-// Split of the items over the CTAs.  A change of unit inside a CTA's range costs about as much as a few tiles (the
-// accumulators drain, the new unit's normalisers are merged from the partials, Q is reloaded), so what the CTAs
-// get equal shares of is  items + pen * (changes of unit): item i of the o-th non-empty unit sits at
-// v = i + pen * o, and CTA c takes the items with v in [c V / ctas, (c + 1) V / ctas).  `pen` stays below the
-// share of a CTA, so no CTA's range is empty.
+// Ranges: the split of one layer's items over `ctas` CTAs.  A change of unit inside a range costs about as much as a few
+// tiles (the accumulators drain, the new unit's normalisers are merged from the partials, Q is reloaded), so what the
+// ranges get equal shares of is  items + pen * (changes of unit): item i of the o-th non-empty unit sits at
+// v = i + pen * o, and range c takes the items with v in [c V / ctas, (c + 1) V / ctas).  `pen` stays below the
+// share of a range, so none is empty.
+// A launch over one layer gives every CTA one range.  The layers of a group are cut into the same ranges, and a CTA takes
+// several that follow one another: the sums of pass 1 begin and end with the ranges, so that a layer's scores are the same
+// bits whatever other layers share its launch.
 constexpr int kUnitChangeTiles = 3;
 struct Split {
-    int items, ctas, pen, Hkv;
+    int items, ctas, pen, Hkv;      // of one layer
     int64_t V;
 };
 
@@ -311,10 +312,10 @@ __device__ inline Split make_split(const SeqView &sv, int B, int Hkv, int grid)
     return sp;
 }
 
-// first item of CTA c (c == ctas: one past the last item)
+// first item of range c (c == ctas: one past the last item)
 __device__ inline int range_begin(const Split &sp, const SeqView &sv, int B, int c)
 {
-    const int64_t t = div_nonneg((int64_t)c * sp.V + sp.ctas - 1, sp.ctas);      // smallest v of the CTA's share
+    const int64_t t = div_nonneg((int64_t)c * sp.V + sp.ctas - 1, sp.ctas);      // smallest v of the range's share
     if (t >= sp.V) return sp.items;
     const int Hkv = sp.Hkv;
     auto key = [&](int q) { return (int64_t)sv.tiles[q] * Hkv + (int64_t)sp.pen * sv.ne[q] * Hkv; };   // v of a sequence's first item
@@ -331,25 +332,47 @@ __device__ inline int range_begin(const Split &sp, const SeqView &sv, int B, int
     return sv.tiles[lo] * Hkv + g * nt + (int)min(r, (int64_t)nt);
 }
 
-// CTA that owns item x of unit u
-__device__ inline int cta_of_item(const Split &sp, const SeqView &sv, int x, int u)
+// Range that holds item x of unit u (of one layer).
+__device__ inline int range_of_item(const Split &sp, const SeqView &sv, int x, int u)
 {
     const int ord = sv.ne[u / sp.Hkv] * sp.Hkv + u % sp.Hkv;
     const int64_t v = (int64_t)x + (int64_t)sp.pen * ord;
     return (int)min((int64_t)(sp.ctas - 1), div_nonneg(v * sp.ctas, sp.V));
 }
 
+// Items of a group are numbered layer after layer.  First item of range q, counted over the layers of the group.
+__device__ inline int group_range_begin(const Split &sp, const SeqView &sv, int B, int q)
+{
+    const int l = q / sp.ctas;
+    return l * sp.items + range_begin(sp, sv, B, q - l * sp.ctas);
+}
+// The ranges and items of this CTA in a pass over a group: items [first, first + count), ranges from `q` on.
+struct Share { int q, first, count; };
+__device__ inline Share cta_share(const Split &sp, const SeqView &sv, int B, int layers)
+{
+    Share sh = {0, 0, 0};
+    const int Q = layers * sp.ctas, ctas = min((int)gridDim.x, Q);
+    if ((int)blockIdx.x < ctas && sp.items > 0) {
+        sh.q = (int)((int64_t)blockIdx.x * Q / ctas);
+        sh.first = group_range_begin(sp, sv, B, sh.q);
+        sh.count = group_range_begin(sp, sv, B, (int)((int64_t)(blockIdx.x + 1) * Q / ctas)) - sh.first;
+    }
+    return sh;
+}
+// Pass 1 leaves one record per (range, unit, half of a tile's columns); record of range c and unit u of layer l.
+__device__ inline int record_index(int l, int c, int u, int U) { return l * (kMaxCtas + U) + c + u; }
+
 struct TcArgs {
     refree_params p;
     TcShape sh;
     const int32_t *seq_start, *seq_len;
+    int split_ctas;      // ranges of a layer, at most
     // Pass 1 writes the partials of group `a`, pass 2 reads those of group `b` and writes its scores.
-    int heads_a, heads_b;      // layers x KV heads of the group that pass 1 / pass 2 works on
-    float2 *part_a;      // [ctas + units][Rpad]: one (c, Z) per (CTA, unit) and row
+    int layers_a, layers_b;
+    float2 *part_a;      // [layers (kMaxCtas + units)][2][Rpad]: one (c, Z) per (range, unit, half of the columns) and row
     const float2 *part_b;
     GroupPartial *groups; // nullable: per 32 positions, exact sum of squared scores for the stopping rule
     float *scores;
-    const __nv_bfloat16 *q_a[kMaxBatch], *k_a[kMaxBatch];   // pass 1 as the tensor maps see it, for the rows that are formed again
     int64_t total_tokens;
     int32_t *dev_status;
     // Stopping rule inside the launch (position ranking per head): the finishing warp that completes a unit's
@@ -365,11 +388,11 @@ struct TcMaps {
     CUtensorMap q[kMaxBatch], k[kMaxBatch];
 };
 
-// budget and record of unit u of the group that pass 2 works on
+// budget of unit u of the group that pass 2 works on
 __device__ inline int32_t *unit_length(const TcArgs &a, int u)
 {
-    const int Hkv = a.p.num_kv_heads, s = u / a.heads_b, g = u - s * a.heads_b, l = g / Hkv;
-    return a.sel_lengths[l] + s * Hkv + (g - l * Hkv);
+    const int U = a.p.num_seqs * a.p.num_kv_heads, l = u / U;
+    return a.sel_lengths[l] + (u - l * U);
 }
 
 // Barrier among the epilogue warps, built on an mbarrier so that it is bounded like
@@ -384,80 +407,74 @@ __device__ inline bool epi_sync(TcSmemTail &tl, uint32_t &phase)
 }
 
 // Loop state that survives from one pass to the other when both run in one launch.  `icount` numbers the
-// items a role has gone through in this launch (both passes): its low bits index the info ring.  `cnt` numbers the
-// products: its low bit is the accumulator.
+// items a role has gone through in this launch (both passes): its low bits index the info ring.  `p2` counts the products
+// of pass 2.
 struct RingState { int stage = 0; uint32_t kphase = 0, qphase = 0, icount = 0; };
-struct MmaState : RingState { uint32_t cnt = 0; bool first = true; };
-struct EpiState { uint32_t ephase = 0, icount = 0, cnt = 0; };
+struct MmaState : RingState { uint32_t p2 = 0; bool first = true; };
+struct EpiState { uint32_t ephase = 0, icount = 0; };
 
 // --------------------------------------------------------- producer / MMA -----
-// Loads one pass's tiles, run by run (a run: the CTA's tiles of one unit).
-//   pass 2  a stage holds one tile: its two 64-column halves, 16 KB each
-//   pass 1  a stage holds one 64-column half of two tiles, 256 rows one after the other (the B operand of a wide
-//           product); a pair of tiles takes two stages, and the odd last tile of a run two half-filled ones
+// Loads one pass's tiles, run by run (a run: the CTA's tiles of one unit, in pass 1 those of one range).
 // The column pass walks a CTA's items backwards: the row pass before it (at the end of the launch before) left its last K tiles in L2, and those are asked for first.
 template <bool PASS1>
 __device__ inline void producer_loop(const TcArgs &a, const TcMaps &maps,
                                      unsigned char *smem_q, unsigned char *smem_k, TcSmemTail &tl, const SeqView &sv,
-                                     int item0, int item1, RingState &rs)
+                                     const Split &sp, const Share &share, RingState &rs)
 {
     const TcShape &sh = a.sh;
-    const int Hkv = a.p.num_kv_heads, G = a.p.num_q_heads / Hkv, heads = PASS1 ? a.heads_a : a.heads_b;
+    const int B = a.p.num_seqs, Hkv = a.p.num_kv_heads, G = a.p.num_q_heads / Hkv, U = B * Hkv;
+    const int item0 = share.first, item1 = share.first + share.count;
     uint64_t pol;
     if (PASS1) asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
     else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    constexpr int kStep = PASS1 ? 2 : 1;                     // tiles per record
     bool ok = true;
+    int q = share.q - 1, range_end = item0, last_u = -1;     // pass 1: the range of item x, and the item it ends at
     for (int x = PASS1 ? item0 : item1 - 1; ok && x >= item0 && x < item1;) {
-        const ItemTc it = decode_item_tc(sv, a.p.num_seqs, heads, x);
-        const int layer = it.g / Hkv, g = it.g - layer * Hkv;
+        const int layer = x / sp.items;
+        const ItemTc it = decode_item_tc(sv, B, Hkv, x - layer * sp.items);
+        if (PASS1 && x >= range_end) range_end = group_range_begin(sp, sv, B, ++q + 1);      // (no range is empty)
+        const int g = it.g, u = layer * U + it.s * Hkv + g;
         const CUtensorMap *const mapq = &maps.q[layer], *const mapk = &maps.k[layer];
-        const int run = PASS1 ? min(it.ntiles - it.tile, item1 - x) : min(it.tile + 1, x - item0 + 1);
+        const int run = PASS1 ? min(it.ntiles - it.tile, range_end - x) : min(it.tile + 1, x - item0 + 1);
         const bool last_run = PASS1 ? x + run >= item1 : x - run < item0;
-        const int ib = sv.tiles[it.s] * heads + it.g * it.ntiles;
+        const int ib = PASS1 ? record_index(layer, q - layer * sp.ctas, it.s * Hkv + g, U)
+                             : layer * sp.items + sv.tiles[it.s] * Hkv + g * it.ntiles;
+        const bool new_unit = u != last_u;
+        last_u = u;
         auto load = [&](unsigned char *dst, int half, int tile) {
             if (sh.rank4)
                 tma_load_4d(dst, mapk, &tl.k_full[rs.stage], half * 64, it.tok0 + tile * kTile, g, it.s, pol);
             else
                 tma_load_3d(dst, mapk, &tl.k_full[rs.stage], half * 64, it.tok0 + tile * kTile, g, pol);
         };
-        for (int j = 0; j < run && ok; j += kStep) {
+        for (int j = 0; j < run && ok; ++j) {
             const int tile = PASS1 ? it.tile + j : it.tile - j;
-            const bool two = PASS1 && j + 1 < run, last = j + kStep >= run;
+            const bool last = j + 1 == run;
             // the ring entry was last used sixteen items ago, which every consumer has long left behind
             ItemInfo &inf = tl.info[rs.icount++ & (kInfoRing - 1)];
-            inf.u = it.u; inf.g = it.g; inf.n = it.n; inf.tile = tile; inf.ntiles = it.ntiles; inf.pack = it.pack;
+            inf.u = u; inf.g = layer * Hkv + g; inf.n = it.n; inf.tile = tile; inf.ntiles = it.ntiles; inf.pack = it.pack;
             inf.ib = ib;
-            inf.flags = (j == 0 ? kNewUnit | kRunFirst : 0) | (last ? kRunLast : 0) | (two ? kTwoTiles : 0) |
-                        (last && last_run ? kPassLast : 0);
-            for (int st = 0; st < kStep; ++st) {
-                // The K tile first: the MMA thread learns of a unit change from the record, which it reads once
-                // the tile has landed, and only then gives the Q image back.
-                ok = mbar_wait(&tl.k_empty[rs.stage], rs.kphase ^ 1, &tl.abort_flag);
+            inf.flags = (j == 0 && new_unit ? kNewUnit : 0) | (last ? kRunLast : 0) | (last && last_run ? kPassLast : 0);
+            // The K tile first: the MMA thread learns of a unit change from the record, which it reads once
+            // the tile has landed, and only then gives the Q image back.
+            ok = mbar_wait(&tl.k_empty[rs.stage], rs.kphase ^ 1, &tl.abort_flag);
+            if (!ok) break;
+            mbar_expect_tx(&tl.k_full[rs.stage], (uint32_t)kTileBytes);      // (release) orders the record before the tile
+            unsigned char *dst = smem_k + (size_t)rs.stage * kTileBytes;
+            load(dst, 0, tile);
+            load(dst + kHalfBytes, 1, tile);
+            if (new_unit && j == 0) {
+                ok = mbar_wait(&tl.q_empty, rs.qphase ^ 1, &tl.abort_flag);
                 if (!ok) break;
-                // (release) orders the record before the tile
-                mbar_expect_tx(&tl.k_full[rs.stage], (uint32_t)(PASS1 && !two ? kHalfBytes : kTileBytes));
-                unsigned char *dst = smem_k + (size_t)rs.stage * kTileBytes;
-                if (PASS1) {
-                    load(dst, st, tile);
-                    if (two) load(dst + kHalfBytes, st, tile + 1);
-                } else {
-                    load(dst, 0, tile);
-                    load(dst + kHalfBytes, 1, tile);
-                }
-                if (j == 0 && st == 0) {
-                    ok = mbar_wait(&tl.q_empty, rs.qphase ^ 1, &tl.abort_flag);
-                    if (!ok) break;
-                    mbar_expect_tx(&tl.q_full, (uint32_t)sh.Rpad * 256u);
-                    const int row0 = (it.s * a.p.num_q_heads + g * G) * a.p.window;
-                    for (int h = 0; h < 2; ++h)
-                        for (int b = 0; b < sh.rblocks; ++b)
-                            tma_load_2d(smem_q + (size_t)h * sh.Rpad * 128 + (size_t)b * kHalfBytes, mapq, &tl.q_full,
-                                        h * 64, row0 + b * kTile);
-                    rs.qphase ^= 1;
-                }
-                if (++rs.stage == sh.stages) { rs.stage = 0; rs.kphase ^= 1; }
+                mbar_expect_tx(&tl.q_full, (uint32_t)sh.Rpad * 256u);
+                const int row0 = (it.s * a.p.num_q_heads + g * G) * a.p.window;
+                for (int h = 0; h < 2; ++h)
+                    for (int b = 0; b < sh.rblocks; ++b)
+                        tma_load_2d(smem_q + (size_t)h * sh.Rpad * 128 + (size_t)b * kHalfBytes, mapq, &tl.q_full,
+                                    h * 64, row0 + b * kTile);
+                rs.qphase ^= 1;
             }
+            if (++rs.stage == sh.stages) { rs.stage = 0; rs.kphase ^= 1; }
         }
         x += PASS1 ? run : -run;
     }
@@ -483,44 +500,41 @@ __device__ inline bool mma_new_unit(TcSmemTail &tl, MmaState &ms)
     return true;
 }
 
-// Pass 1: D[row, position] = Q_blk K^T, one product per pair of tiles and row block.
+// Pass 1: D[row, position] = Q_blk K_tile^T.  Row block rb goes to accumulator pair rb & 1 (the group of epilogue warps
+// that takes it), which alternates between its two accumulators of 128 columns: the product of a pair's next block runs
+// while the epilogue reads the current one.
 __device__ inline void mma_loop_pass1(const TcArgs &a, unsigned char *smem_q, unsigned char *smem_k, TcSmemTail &tl,
                                       uint32_t tmem_base, MmaState &ms)
 {
     const TcShape &sh = a.sh;
     const uint32_t q_lo = desc_lo(smem_u32(smem_q)), k_lo = desc_lo(smem_u32(smem_k));
     const uint32_t q_half = (uint32_t)(sh.Rpad * 128) >> 4;      // distance between the two 64-column halves of Q
+    const uint32_t idesc = make_idesc(kTile);
+    uint32_t cnt0 = 0, cnt1 = 0;                                 // products per pair
     for (;;) {
-        int st[2];
         if (!mbar_wait(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
         tc_fence_after();
         const int flags = tl.info[ms.icount++ & (kInfoRing - 1)].flags;
-        const uint32_t idesc = make_idesc(flags & kTwoTiles ? 2 * kTile : kTile);
         if ((flags & kNewUnit) && !mma_new_unit(tl, ms)) return;
+        const uint32_t kt = k_lo + (uint32_t)ms.stage * (kTileBytes >> 4);
         for (int rb = 0; rb < sh.rblocks; ++rb) {
-            const uint32_t buf = ms.cnt & 1u;
-            if (!mbar_wait(&tl.acc_empty[buf], ((ms.cnt >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
+            const uint32_t pair = (uint32_t)(rb & 1), cnt = pair ? cnt1 : cnt0, acc = 2u * pair + (cnt & 1u);
+            // a pair covers the columns of an accumulator of pass 2: the last product left there must have been handed back
+            const uint32_t before = (ms.p2 + 1u - pair) >> 1;
+            if (cnt == 0 && before > 0 && !mbar_wait(&tl.p2_empty[pair], (before - 1u) & 1u, &tl.abort_flag)) return;
+            if (!mbar_wait(&tl.p1_empty[acc], ((cnt >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
             tc_fence_after();
+            const uint32_t qa = q_lo + (uint32_t)rb * (kHalfBytes >> 4);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (rb == 0) {
-                    if (h == 1) {
-                        if (!mbar_wait(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
-                        tc_fence_after();
-                    }
-                    st[h] = ms.stage;
-                    if (++ms.stage == sh.stages) { ms.stage = 0; ms.kphase ^= 1; }
-                }
-                const uint32_t kb = k_lo + (uint32_t)st[h] * (kTileBytes >> 4);
-                const uint32_t qa = q_lo + (uint32_t)rb * (kHalfBytes >> 4) + (uint32_t)h * q_half;
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)                          // 32 bytes per K step of 16
-                    umma_bf16(tmem_base + buf * 256u, qa + kk * 2, kb + kk * 2, kDescHi, idesc, h + kk > 0);
-                if (rb == sh.rblocks - 1) umma_commit(&tl.k_empty[st[h]]);
+            for (int kk = 0; kk < 8; ++kk) {
+                const uint32_t h = kk >> 2, ko = (kk & 3) * 2;          // 32 bytes per K step of 16
+                umma_bf16(tmem_base + acc * 128u, qa + h * q_half + ko, kt + h * (kHalfBytes >> 4) + ko, kDescHi, idesc, kk > 0);
             }
-            umma_commit(&tl.acc_full[buf]);
-            ++ms.cnt;
+            umma_commit(&tl.p1_full[acc]);
+            if (pair) ++cnt1; else ++cnt0;
         }
+        umma_commit(&tl.k_empty[ms.stage]);
+        if (++ms.stage == sh.stages) { ms.stage = 0; ms.kphase ^= 1; }
         if (flags & kPassLast) break;
     }
 }
@@ -541,8 +555,8 @@ __device__ inline void mma_loop_pass2(const TcArgs &a, unsigned char *smem_q, un
         if ((flags & kNewUnit) && !mma_new_unit(tl, ms)) return;
         const uint32_t ka = k_lo + (uint32_t)ms.stage * (kTileBytes >> 4);
         for (int cb = 0; cb < sh.cblocks; ++cb) {
-            const uint32_t buf = ms.cnt & 1u;
-            if (!mbar_wait(&tl.acc_empty[buf], ((ms.cnt >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
+            const uint32_t buf = ms.p2 & 1u;
+            if (!mbar_wait(&tl.p2_empty[buf], ((ms.p2 >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
             tc_fence_after();
             const uint32_t qb = q_lo + (uint32_t)cb * (uint32_t)(sh.ncol * 128 >> 4);
 #pragma unroll
@@ -550,8 +564,8 @@ __device__ inline void mma_loop_pass2(const TcArgs &a, unsigned char *smem_q, un
                 const uint32_t h = kk >> 2, ko = (kk & 3) * 2;
                 umma_bf16(tmem_base + buf * 256u, ka + h * (kHalfBytes >> 4) + ko, qb + h * q_half + ko, kDescHi, idesc, kk > 0);
             }
-            umma_commit(&tl.acc_full[buf]);
-            ++ms.cnt;
+            umma_commit(&tl.p2_full[buf]);
+            ++ms.p2;
         }
         umma_commit(&tl.k_empty[ms.stage]);
         if (++ms.stage == sh.stages) { ms.stage = 0; ms.kphase ^= 1; }
@@ -561,19 +575,6 @@ __device__ inline void mma_loop_pass2(const TcArgs &a, unsigned char *smem_q, un
 }
 
 // ------------------------------------------------------------- epilogues -----
-// Pass 2: the rows (columns of a product) of a warp: `np` pairs of 16 from column `col0` on.  The pairs of the product
-// go to the four warps that share a quarter of the positions; those four sit on one SM sub-partition, so an uneven
-// split loads the sub-partitions evenly all the same.
-struct WarpColumns { int np, col0; };
-__device__ inline WarpColumns warp_columns(int ncol, int cq)
-{
-    const int pairs = ncol >> 5, base = pairs >> 2, extra = pairs & 3;
-    WarpColumns c;
-    c.np = base + (cq < extra ? 1 : 0);
-    c.col0 = 32 * (cq * base + min(cq, extra));
-    return c;
-}
-
 // Give an accumulator back: every load of this warp from it has landed.
 __device__ inline void release_acc(uint64_t *bar, int lane)
 {
@@ -582,189 +583,119 @@ __device__ inline void release_acc(uint64_t *bar, int lane)
     if (lane == 0) mbar_arrive(bar);
 }
 
-// Pass 1: one row's sum over a warp's positions of a run (64 of every 256 from tile `tile0` on), formed again from
-// global memory with fp32 multiply-adds: the row's largest logit lies so far above the reference (the largest of the
-// run's first tiles) that the sum left the range of fp32.  Slow and rare: it takes logits that grow by more than 83
-// (natural units) within a run.
-__device__ __noinline__ float2 row_sum_again(const TcArgs &a, const SeqView &sv, int u, int row, int cq, int tile0, int tile1)
-{
-    const int lane = threadIdx.x & 31;
-    const int Hkv = a.p.num_kv_heads, G = a.p.num_q_heads / Hkv, w = a.p.window;
-    const int s = u / a.heads_a, gl = u - s * a.heads_a, layer = gl / Hkv, g = gl - layer * Hkv, n = sv.len[s];
-    const int head = row / w, rloc = row - head * w;
-    const float scale = kLog2e * rsqrtf((float)kD);
-    const __nv_bfloat16 *q = a.q_a[layer] + (((int64_t)s * a.p.num_q_heads + (int64_t)g * G + head) * w + rloc) * kD;
-    const __nv_bfloat16 *k = a.k_a[layer] + (int64_t)s * a.p.k_stride_seq + (int64_t)g * a.p.k_stride_head +
-                             (int64_t)sv.start[s] * a.p.k_stride_tok;
-    const int end = min(min(n, n - w + rloc + 1), (tile1 + 1) * kTile);
-    float m = -INFINITY, z = 0.f;
-    for (int p0 = tile0 * kTile + cq * 64; p0 < end; p0 += 256)
-        for (int pos = p0 + lane; pos < min(p0 + 64, end); pos += 32) {
-            const uint4 *kr = reinterpret_cast<const uint4 *>(k + (int64_t)pos * a.p.k_stride_tok);
-            float acc = 0.f;
-            for (int c = 0; c < kD / 8; ++c) {
-                const uint4 kv = __ldg(kr + c);
-                const uint4 qv = __ldg(reinterpret_cast<const uint4 *>(q) + c);
-                const uint32_t kw[4] = {kv.x, kv.y, kv.z, kv.w}, qw[4] = {qv.x, qv.y, qv.z, qv.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc = fmaf(__uint_as_float(kw[e] << 16), __uint_as_float(qw[e] << 16), acc);
-                    acc = fmaf(__uint_as_float(kw[e] & 0xffff0000u), __uint_as_float(qw[e] & 0xffff0000u), acc);
-                }
-            }
-            const float y = acc * scale;
-            if (y > m) { z = z * ex2(m - y) + 1.f; m = y; }
-            else z += ex2(y - m);
-        }
-    const float M = warp_max(m);
-    z = M > -INFINITY ? z * ex2(m - M) : 0.f;
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    return make_float2(M > -INFINITY ? M : 0.f, z);
-}
-
-// Pass 1: lane = query row, 64 logits of the row per product, 16 at a time with the next 16 in flight.  The accumulator
-// goes back once the last of them have landed, and then the first 16 of the next product are asked for if it is there
-// already (`have`: they are in flight in b0).  limit: positions of the 64 that the row sees.
+// Pass 1: lane = query row, 64 logits of the row in registers.
 template <bool MASKED>
-__device__ inline float row_product(uint32_t taddr, uint64_t *empty_bar, int lane, float scale, float nc, int limit,
-                                    uint32_t (&b0)[16], uint32_t (&b1)[16], uint64_t *next_bar, uint32_t next_parity,
-                                    uint32_t next_taddr, bool &have)
+__device__ inline float row_sum_regs(const uint32_t (&ra)[32], const uint32_t (&rb)[32], float scale, float cref, int limit)
 {
-    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    float z0 = 0.f, z1 = 0.f;
+    const float nc = -cref;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        uint32_t (&cur)[16] = (c & 1) ? b1 : b0;
-        uint32_t (&nxt)[16] = (c & 1) ? b0 : b1;
-        tmem_ld_wait(cur);
-        if (c < 3) {
-            tmem_ld_issue(taddr + 16 * (c + 1), nxt);
-        } else {
-            release_acc(empty_bar, lane);
-            have = next_bar && __all_sync(0xffffffffu, mbar_try(next_bar, next_parity));
-            if (have) { tc_fence_after(); tmem_ld_issue(next_taddr, nxt); }
-        }
+    for (int c = 0; c < 2; ++c) {
+        const uint32_t (&cur)[32] = c ? rb : ra;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            float e = ex2(fmaf(__uint_as_float(cur[i]), scale, nc));
-            if (MASKED) e = 16 * c + i < limit ? e : 0.f;
-            z[i & 3] += e;
+        for (int i = 0; i < 32; i += 2) {
+            float e0 = ex2(fmaf(__uint_as_float(cur[i]), scale, nc));
+            float e1 = ex2(fmaf(__uint_as_float(cur[i + 1]), scale, nc));
+            if (MASKED) {
+                e0 = (c * 32 + i < limit) ? e0 : 0.f;
+                e1 = (c * 32 + i + 1 < limit) ? e1 : 0.f;
+            }
+            z0 += e0;
+            z1 += e1;
         }
     }
-    return (z[0] + z[1]) + (z[2] + z[3]);
+    return z0 + z1;
+}
+__device__ inline float row_max_regs(const uint32_t (&ra)[32], const uint32_t (&rb)[32], float scale, int limit)
+{
+    float m = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const uint32_t (&cur)[32] = c ? rb : ra;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (c * 32 + i < limit) m = fmaxf(m, __uint_as_float(cur[i]) * scale);
+    }
+    return m;
 }
 
-__device__ inline void epilogue_pass1(const TcArgs &a, TcSmemTail &tl, const SeqView &sv, uint32_t tmem_base, EpiState &es)
+// Two groups of eight warps take the row blocks in turn (block rb goes to group rb & 1); inside a group a warp is
+// (lane quarter) x (half of each tile's columns), and adds its half of tile after tile of a run in their order.
+__device__ inline void epilogue_pass1(const TcArgs &a, TcSmemTail &tl, uint32_t tmem_base, EpiState &es)
 {
     const TcShape &sh = a.sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quarter = warp & 3, cq = warp >> 2;
+    const int group = (warp >> 2) & 1, half = warp >> 3, lane_base = (warp & 3) * 32;
+    if (group >= sh.rblocks) return;             // a single row block: all of it is the first group's
     const float scale = kLog2e * rsqrtf((float)kD);
     const int w = a.p.window;
-    const uint32_t tlane = tmem_base + (uint32_t)(cq * 64) + ((uint32_t)(quarter * 32) << 16);
-    float nc[4] = {0.f, 0.f, 0.f, 0.f}, z[4] = {0.f, 0.f, 0.f, 0.f};     // per row block: minus the reference, the sum
-    uint32_t b0[16], b1[16];
-    bool have = false;
-    int tile0 = 0;
+    uint32_t cnt = 0;                            // products this group has taken
+    // running reference and sum of this lane's rows (row blocks group and group + 2) over its half of the columns
+    float cref[2] = {-INFINITY, -INFINITY}, zsum[2] = {0.f, 0.f};
+    int rmod[2];
+    bool rvalid[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int row = (group + 2 * j) * kTile + lane_base + lane;
+        rmod[j] = row % w;                       // offset of the row's query inside the window
+        rvalid[j] = row < sh.R;
+    }
     for (;;) {
         const ItemInfo *inf = &tl.info[es.icount++ & (kInfoRing - 1)];
-        int flags = 0, tile = 0, n = 0;
-        for (int rb = 0; rb < sh.rblocks; ++rb) {
-            const uint32_t buf = es.cnt & 1u, parity = (es.cnt >> 1) & 1u;
-            const uint32_t taddr = tlane + buf * 256u;
-            if (!have) {
-                if (!mbar_wait(&tl.acc_full[buf], parity, &tl.abort_flag)) return;
-                tc_fence_after();
-                tmem_ld_issue(taddr, b0);
-            }
-            ++es.cnt;
-            if (rb == 0) {                                       // the record is valid once the item's first product is
-                flags = inf->flags; tile = inf->tile; n = inf->n;
-                if (flags & kRunFirst) tile0 = tile;
-            }
-            const int row = rb * kTile + quarter * 32 + lane;
-            const int first = tile * kTile + cq * 64;            // first position of this warp's columns
-            const bool in_pair = cq < 2 || (flags & kTwoTiles);
-            int limit = 64;
-            bool full = true, none = false;                      // the whole warp sees all / nothing of its columns
-            if (!in_pair || tile * kTile + 2 * kTile > n - w + 1) {
-                limit = in_pair && row < sh.R ? max(0, min(64, n - w + row % w + 1 - first)) : 0;
-                full = __all_sync(0xffffffffu, limit == 64);
-                none = __all_sync(0xffffffffu, limit == 0);
-            }
-            float c = rb == 0 ? nc[0] : rb == 1 ? nc[1] : rb == 2 ? nc[2] : nc[3];
-            if (flags & kRunFirst) {
-                // the run's reference: the row's largest logit among these 64 (0 where it sees none of them: it then
-                // sees none of the run's)
-                c = 0.f;
-                if (!none) {
-                    float m = -INFINITY;
-                    for (int k = 0; k < 4; ++k) {
-                        tmem_ld_issue(taddr + 16 * k, b1);
-                        tmem_ld_wait(b1);
+        int flags = 0, tile_start = 0, n = 0, rec = 0;
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) m = 16 * k + i < limit ? fmaxf(m, __uint_as_float(b1[i])) : m;
-                    }
-                    if (m > -INFINITY) c = -(m * scale);
-                }
+        for (int j = 0; j < 2; ++j) {
+            const int rb = group + 2 * j;
+            if (rb >= sh.rblocks) continue;
+            const uint32_t acc = 2u * (uint32_t)group + (cnt & 1u);
+            if (!mbar_wait(&tl.p1_full[acc], (cnt >> 1) & 1u, &tl.abort_flag)) return;
+            ++cnt;
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + acc * 128u + (uint32_t)(half * 64) + ((uint32_t)lane_base << 16);
+            uint32_t ra[32], rb2[32];
+            tmem_ld_issue(taddr, ra);
+            tmem_ld_issue(taddr + 32, rb2);
+            tmem_ld_wait(ra);
+            tmem_ld_wait(rb2);
+            // the logits are in registers: the accumulator goes back to the MMA warp before any arithmetic
+            release_acc(&tl.p1_empty[acc], lane);
+            if (j == 0) { flags = inf->flags; tile_start = inf->tile * kTile; n = inf->n; rec = inf->ib; }   // valid once a product of the item is
+            const bool full = tile_start + kTile <= n - w + 1;      // tile wholly before the window
+            int limit = kTile;                                  // visible positions of the tile: [0, limit)
+            if (!full) {
+                limit = n - w + rmod[j] - tile_start + 1;           // up to this row's own position
+                limit = rvalid[j] ? max(0, min(kTile, limit)) : 0;
+            } else if (!rvalid[j]) {
+                limit = 0;
             }
-            const bool end = (flags & kPassLast) && rb + 1 == sh.rblocks;
-            uint64_t *next_bar = end ? nullptr : &tl.acc_full[buf ^ 1u];
-            const uint32_t next_parity = (es.cnt >> 1) & 1u, next_taddr = tlane + (buf ^ 1u) * 256u;
+            limit = max(0, min(64, limit - half * 64));         // inside this warp's columns
+            const bool uniform = __all_sync(0xffffffffu, limit == 64);
+            bool need_max = (cref[j] == -INFINITY) && limit > 0;
             float zt = 0.f;
-            if (none) {
-                tmem_ld_wait(b0);
-                release_acc(&tl.acc_empty[buf], lane);
-                have = false;
-            } else if (full) {
-                zt = row_product<false>(taddr, &tl.acc_empty[buf], lane, scale, c, 64, b0, b1, next_bar, next_parity, next_taddr, have);
-            } else {
-                zt = row_product<true>(taddr, &tl.acc_empty[buf], lane, scale, c, limit, b0, b1, next_bar, next_parity, next_taddr, have);
+            for (int attempt = 0; attempt < 2; ++attempt) {
+                if (__any_sync(0xffffffffu, need_max)) {
+                    const float m = row_max_regs(ra, rb2, scale, limit);
+                    if (need_max && m > cref[j]) {
+                        zsum[j] = (cref[j] == -INFINITY) ? 0.f : zsum[j] * ex2(cref[j] - m);
+                        cref[j] = m;
+                    }
+                }
+                zt = uniform ? row_sum_regs<false>(ra, rb2, scale, cref[j], limit)
+                             : row_sum_regs<true>(ra, rb2, scale, cref[j], limit);
+                need_max = !(zt <= kZLimit) && limit > 0;       // overflow against a stale reference
+                if (attempt == 1 || !__any_sync(0xffffffffu, need_max)) break;
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (j == rb) { nc[j] = c; z[j] += zt; }
+            if (limit > 0) zsum[j] += zt;
         }
         if (flags & kRunLast) {
-            const int u = inf->u;
-            const int tile1 = tile + (flags & kTwoTiles ? 1 : 0);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (j >= sh.rblocks) break;
-                const int row = j * kTile + quarter * 32 + lane;
-                unsigned over = __ballot_sync(0xffffffffu, row < sh.R && !(z[j] <= kZLimit));
-                while (over) {
-                    const int l = __ffs(over) - 1;
-                    over &= over - 1;
-                    const float2 r = row_sum_again(a, sv, u, row - lane + l, cq, tile0, tile1);
-                    if (lane == l) { nc[j] = -r.x; z[j] = r.y; }
-                }
+            for (int j = 0; j < 2; ++j) {
+                const int row = (group + 2 * j) * kTile + lane_base + lane;
+                if (group + 2 * j < sh.rblocks && row < sh.R)
+                    a.part_a[((int64_t)rec * 2 + half) * sh.Rpad + row] = make_float2(cref[j], zsum[j]);
+                cref[j] = -INFINITY;
+                zsum[j] = 0.f;
             }
-            // the four quarters of the positions come together, kCombRows rows at a time
-            for (int r0 = 0; r0 < sh.R; r0 += kCombRows) {
-                if (!epi_sync(tl, es.ephase)) return;            // what was there before has been read
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int row = j * kTile + quarter * 32 + lane - r0;
-                    if (j < sh.rblocks && row >= 0 && row < kCombRows) tl.comb[cq][row] = make_float2(-nc[j], z[j]);
-                }
-                if (!epi_sync(tl, es.ephase)) return;
-                const int row = (int)threadIdx.x;
-                if (row < kCombRows && r0 + row < sh.R) {
-                    float2 r[4];
-                    float M = -INFINITY, Z = 0.f;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        r[k] = tl.comb[k][row];
-                        if (r[k].y > 0.f) M = fmaxf(M, r[k].x);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (r[k].y > 0.f) Z = fmaf(r[k].y, ex2(r[k].x - M), Z);
-                    a.part_a[(int64_t)(blockIdx.x + u) * sh.Rpad + r0 + row] = make_float2(M, Z);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) z[j] = 0.f;
         }
         if (flags & kPassLast) break;
     }
@@ -797,82 +728,79 @@ __device__ inline void col_sum16(const uint32_t (&cur)[16], float scale, const f
     }
 }
 
-// One product's share of a warp in pass 2: pairs of 16 rows, one chunk of 16 in flight while the other is summed; the
-// accumulator goes back as soon as the last load has landed, and then the first chunk of the next product is asked for
-// if it is there already (`have`: it is in flight in b0).
+// One product's share of a warp: `nch` chunks of 16 columns (rows of Q) come from tensor memory one chunk at a
+// time, the next in flight while 2^(y - L[row]) is summed over the current one; the accumulator is handed back
+// as soon as the last load has landed.
 template <bool MASKED>
-__device__ inline float col_product(int np, uint32_t taddr, uint64_t *empty_bar, int lane, float scale, const float *lse,
-                                    int r0, int R, int w, int pos_gap, uint32_t (&b0)[16], uint32_t (&b1)[16],
-                                    uint64_t *next_bar, uint32_t next_parity, uint32_t next_taddr, bool &have)
+__device__ inline float col_product(int nch, uint32_t taddr, uint64_t *empty_bar, int lane, float scale, const float *lse,
+                                    int r0, int R, int w, int pos_gap)
 {
+    uint32_t b0[16], b1[16];
     float s0 = 0.f, s1 = 0.f;
-    have = false;
-    if (np == 0) { release_acc(empty_bar, lane); return 0.f; }
-    for (int p = 0; p < np; ++p, r0 += 32, taddr += 32) {
-        tmem_ld_wait(b0);
-        tmem_ld_issue(taddr + 16, b1);
-        col_sum16<MASKED>(b0, scale, lse, r0, R, w, pos_gap, s0, s1);
-        tmem_ld_wait(b1);
-        if (p + 1 < np) {
-            tmem_ld_issue(taddr + 32, b0);
-        } else {
-            release_acc(empty_bar, lane);
-            have = next_bar && __all_sync(0xffffffffu, mbar_try(next_bar, next_parity));
-            if (have) { tc_fence_after(); tmem_ld_issue(next_taddr, b0); }
+    tmem_ld_issue(taddr, b0);
+    tmem_ld_wait(b0);
+    for (int c = 0; c < nch; c += 2) {
+        if (c + 1 < nch) tmem_ld_issue(taddr + 16 * (c + 1), b1); else release_acc(empty_bar, lane);
+        col_sum16<MASKED>(b0, scale, lse, r0 + 16 * c, R, w, pos_gap, s0, s1);
+        if (c + 1 < nch) {
+            tmem_ld_wait(b1);
+            if (c + 2 < nch) tmem_ld_issue(taddr + 16 * (c + 2), b0); else release_acc(empty_bar, lane);
+            col_sum16<MASKED>(b1, scale, lse, r0 + 16 * (c + 1), R, w, pos_gap, s0, s1);
+            if (c + 2 < nch) tmem_ld_wait(b0);
         }
-        col_sum16<MASKED>(b1, scale, lse, r0 + 16, R, w, pos_gap, s0, s1);
     }
     return s0 + s1;
 }
 
-// L[row] = log2 sum over the row of 2^y for the rows of unit u, merged from the (reference, sum) pairs that pass 1
-// left per (CTA, unit), the same way in every CTA that needs the unit.
-// Called by all epilogue threads; `ib` = index of the unit's first item, `ts` = its tiles.
-__device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, const SeqView &sv, const Split &sp, int u, int ib,
+// L[row] = log2 sum over the row of 2^y for the rows of unit u of a layer, merged from the (reference, sum) pairs that
+// pass 1 left per (range, unit, column half), in ascending record order (the same in every CTA that needs the unit).
+// Called by all epilogue threads; `ib` = index of the unit's first item in its layer, `ts` = its tiles.
+__device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, const SeqView &sv, const Split &sp, int layer, int u, int ib,
                                       int ts, uint32_t &ephase)
 {
     const TcShape &sh = a.sh;
     const int tid = threadIdx.x;
-    const int c_lo = cta_of_item(sp, sv, ib, u), c_hi = cta_of_item(sp, sv, ib + ts - 1, u);
-    // Several threads per row (a power of two), each taking every per_row-th record: the largest reference of a batch
-    // first, then terms that do not wait for one another, so a batch costs one round trip to L2.
-    int per_row = 1;
-    while (per_row < 8 && 2 * per_row * sh.R <= kEpiWarps * 32) per_row *= 2;
-    const int r = tid / per_row, sub = tid & (per_row - 1);
+    const int c_lo = range_of_item(sp, sv, ib, u), c_hi = range_of_item(sp, sv, ib + ts - 1, u);
+    // two threads per row when there are enough threads: even and odd records, then one exchange
+    const int per_row = 2 * sh.R <= kEpiWarps * 32 ? 2 : 1;
+    const int r = tid / per_row, sub = tid % per_row;
     float M = -INFINITY, Z = 0.f;
     if (r < sh.R) {
-        const float2 *rec = a.part_b + (int64_t)(c_lo + u) * sh.Rpad + r;
-        const int nrec = c_hi - c_lo + 1;
+        const float2 *rec = a.part_b + (int64_t)record_index(layer, c_lo, u, a.p.num_seqs * a.p.num_kv_heads) * 2 * sh.Rpad + r;
+        const int nrec = 2 * (c_hi - c_lo + 1);             // records: (range, column half)
         constexpr int kBatch = 12;                          // independent loads in flight per thread
         for (int s0 = sub; s0 < nrec; s0 += kBatch * per_row) {
             float2 pr[kBatch];
 #pragma unroll
             for (int q = 0; q < kBatch; ++q)
                 pr[q] = s0 + q * per_row < nrec ? __ldcg(rec + (int64_t)(s0 + q * per_row) * sh.Rpad) : make_float2(0.f, 0.f);
-            float m = M;
+            // Z 2^M + y 2^x, record after record, at the larger of the two references.  What a step scales by depends on
+            // the references alone, so the exponentials do not wait for the sums.
+            float f[kBatch];
+            unsigned grows = 0;
 #pragma unroll
-            for (int q = 0; q < kBatch; ++q) if (pr[q].y > 0.f) m = fmaxf(m, pr[q].x);
-            if (m == -INFINITY) continue;                   // records of a row that sees nothing
-            float z0 = Z * ex2(M - m), z1 = 0.f;
-#pragma unroll
-            for (int q = 0; q < kBatch; q += 2) {
-                if (pr[q].y > 0.f) z0 = fmaf(pr[q].y, ex2(pr[q].x - m), z0);
-                if (pr[q + 1].y > 0.f) z1 = fmaf(pr[q + 1].y, ex2(pr[q + 1].x - m), z1);
+            for (int q = 0; q < kBatch; ++q) {
+                const bool up = pr[q].y > 0.f && pr[q].x > M;
+                f[q] = ex2(up ? M - pr[q].x : pr[q].x - M);
+                if (up) { M = pr[q].x; grows |= 1u << q; }
             }
-            Z = z0 + z1;
-            M = m;
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q) {
+                const bool up = (grows >> q) & 1u;
+                if (pr[q].y > 0.f) Z = fmaf(up ? Z : pr[q].y, f[q], up ? pr[q].y : Z);
+            }
         }
     }
-    // the lanes of a row combine in a fixed pattern: every lane, and every CTA, gets the same bits
-    for (int o = 1; o < per_row; o <<= 1) {
-        const float M2 = __shfl_xor_sync(0xffffffffu, M, o), Z2 = __shfl_xor_sync(0xffffffffu, Z, o);
-        const float m = fmaxf(M, M2);
-        if (m > -INFINITY) {
-            const bool low = (sub & o) == 0;                // (lower lane's share) + (upper lane's share) on both
-            const float za = (low ? Z : Z2) * ex2((low ? M : M2) - m), zb = (low ? Z2 : Z) * ex2((low ? M2 : M) - m);
-            Z = za + zb;
-            M = m;
-        }
+    if (per_row == 2) {
+        const float M2 = __shfl_xor_sync(0xffffffffu, M, 1), Z2 = __shfl_xor_sync(0xffffffffu, Z, 1);
+        // (even records) then (odd records), in that order on both lanes
+        const float Ma = sub ? M2 : M, Za = sub ? Z2 : Z, Mb = sub ? M : M2, Zb = sub ? Z : Z2;
+        if (Zb > 0.f) {
+            if (Za > 0.f) {
+                if (Mb > Ma) { Z = Za * ex2(Ma - Mb) + Zb; M = Mb; }
+                else { Z = Za + Zb * ex2(Mb - Ma); M = Ma; }
+            } else { Z = Zb; M = Mb; }
+        } else { Z = Za; M = Ma; }
     }
     // a row that sees nothing adds 2^(-inf) = 0
     if (r < sh.R && sub == 0) tl.lse[r] = Z > 0.f ? M + log2f(Z) : INFINITY;
@@ -881,66 +809,65 @@ __device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, const Seq
     return epi_sync(tl, ephase);
 }
 
-// Pass 2, the sixteen epilogue warps: every warp leaves its share of a tile's column sums (one quarter of the rows, all
-// row blocks) in a staging slot, and the finishing warp adds the shares.
+// Pass 2, the sixteen epilogue warps.  Two groups of eight warps take the products in turn (product j goes to
+// group j & 1 and to accumulator j & 1), so the groups run out of step: while one waits for its next accumulator,
+// stages a tile or refills its pipeline, the other keeps the exponential units busy.  Inside a group a warp is
+// (lane quarter) x (half of the product's columns); it leaves its share of the tile's column sums in a staging
+// slot, and the finishing warp adds the shares.
 __device__ inline void epilogue_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot *stage, const SeqView &sv, uint32_t tmem_base,
                                       int item0, int nitems, const Split &sp, EpiState &es)
 {
     const TcShape &sh = a.sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quarter = warp & 3, cq = warp >> 2;
-    const WarpColumns wc = warp_columns(sh.ncol, cq);
+    const int group = (warp >> 2) & 1, half = warp >> 3, lane_base = (warp & 3) * 32;
     const float scale = kLog2e * rsqrtf((float)kD);
-    const int w = a.p.window;
-    const int pos_in_tile = quarter * 32 + lane;
+    const int w = a.p.window, Hkv = a.p.num_kv_heads;
+    const int pos_in_tile = lane_base + lane;
+    const int c_width = sh.ncol >> 1, c_begin = half * c_width;     // this warp's columns of a product
     const bool exact = sh.cblocks * sh.ncol == sh.R;               // no padding columns in the products
-    const uint32_t tlane = tmem_base + (uint32_t)wc.col0 + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t taddr = tmem_base + (uint32_t)group * 256u + (uint32_t)c_begin + ((uint32_t)lane_base << 16);
     const int slot_shift = 31 - __clz(sh.slots);
-    uint32_t b0[16], b1[16];
-    bool have = false;
+    uint32_t gcnt = 0;                                             // products this group has taken
     int next_change = 0;                                           // item (relative) at which the next unit begins
     for (int item = 0; item < nitems; ++item) {
         const ItemInfo *inf = &tl.info[es.icount++ & (kInfoRing - 1)];
         if (item == next_change) {   // `item` counts the pass's items in the order they come: from the CTA's last one backwards
-            // A unit begins.  It is looked up in the sequence tables, not in the item's record: the normalisers do
-            // not wait for the tile (the partials come from the row pass, not from anything this pass loads).
-            const ItemTc it = decode_item_tc(sv, a.p.num_seqs, a.heads_b, item0 + (nitems - 1 - item));
+            // A unit begins: all sixteen warps meet (the two groups share L), whichever group takes the item's
+            // products.  The unit is looked up in the sequence tables, not in the item's record, which a warp
+            // that takes none of the item's products has no barrier to wait for.  The normalisers do not wait
+            // for the tile either: the partials come from the row pass, not from anything this pass loads.
+            const int x = item0 + (nitems - 1 - item), layer = x / sp.items;
+            const ItemTc it = decode_item_tc(sv, a.p.num_seqs, Hkv, x - layer * sp.items);
             if (item > 0 && !epi_sync(tl, es.ephase)) return;      // nobody still reads the previous unit's L
-            if (!merge_unit_lse(a, tl, sv, sp, it.u, sv.tiles[it.s] * a.heads_b + it.g * it.ntiles, it.ntiles, es.ephase))
+            if (!merge_unit_lse(a, tl, sv, sp, layer, it.s * Hkv + it.g, sv.tiles[it.s] * Hkv + it.g * it.ntiles, it.ntiles, es.ephase))
                 return;
             next_change = item + it.tile + 1;                      // the unit's earlier tiles follow
         }
-        float part = 0.f;
         for (int cb = 0; cb < sh.cblocks; ++cb) {
-            const uint32_t buf = es.cnt & 1u, parity = (es.cnt >> 1) & 1u;
-            const uint32_t taddr = tlane + buf * 256u;
-            if (!have) {
-                if (!mbar_wait(&tl.acc_full[buf], parity, &tl.abort_flag)) return;
-                tc_fence_after();
-                if (wc.np) tmem_ld_issue(taddr, b0);
-            }
-            ++es.cnt;
+            const uint32_t j = (uint32_t)item * (uint32_t)sh.cblocks + (uint32_t)cb;      // product index in this pass
+            if ((int)(j & 1u) != group) continue;
+            if (!mbar_wait(&tl.p2_full[group], gcnt & 1u, &tl.abort_flag)) return;
+            ++gcnt;
+            tc_fence_after();
             // the item's record is valid once one of its products is
             const int tile_start = inf->tile * kTile, n = inf->n;
             const int pos_gap = tile_start + pos_in_tile - (n - w);
             // tile wholly before the window and wholly inside the sequence: every row sees every position
             const bool full = tile_start + kTile <= n - w + 1 && exact;
-            uint64_t *next_bar = item + 1 < nitems || cb + 1 < sh.cblocks ? &tl.acc_full[buf ^ 1u] : nullptr;
-            const uint32_t next_parity = (es.cnt >> 1) & 1u, next_taddr = tlane + (buf ^ 1u) * 256u;
-            part += full ? col_product<false>(wc.np, taddr, &tl.acc_empty[buf], lane, scale, tl.lse, cb * sh.ncol + wc.col0, sh.R, w,
-                                              pos_gap, b0, b1, next_bar, next_parity, next_taddr, have)
-                         : col_product<true>(wc.np, taddr, &tl.acc_empty[buf], lane, scale, tl.lse, cb * sh.ncol + wc.col0, sh.R, w,
-                                             pos_gap, b0, b1, next_bar, next_parity, next_taddr, have);
+            const float part = full ? col_product<false>(c_width >> 4, taddr, &tl.p2_empty[group], lane, scale, tl.lse,
+                                                         cb * sh.ncol + c_begin, sh.R, w, pos_gap)
+                                    : col_product<true>(c_width >> 4, taddr, &tl.p2_empty[group], lane, scale, tl.lse,
+                                                        cb * sh.ncol + c_begin, sh.R, w, pos_gap);
+            // the slot's previous tile has been read by the finishing warp
+            const uint32_t slot = (uint32_t)item & (uint32_t)(sh.slots - 1);
+            if (!mbar_wait(&tl.stage_free[slot], (((uint32_t)item >> slot_shift) & 1u) ^ 1u, &tl.abort_flag)) return;
+            stage[slot].sum[cb * 2 + half][pos_in_tile] = part;
+            // the tile's record travels with its sums (the ring it came from may be reused before the tile is finished)
+            if (cb == 0 && half == 0 && lane_base == 0 && lane < 8)
+                reinterpret_cast<uint32_t *>(&stage[slot].info)[lane] = reinterpret_cast<const uint32_t *>(inf)[lane];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tl.chunk_ready[slot]);
         }
-        // the slot's previous tile has been read by the finishing warp
-        const uint32_t slot = (uint32_t)item & (uint32_t)(sh.slots - 1);
-        if (!mbar_wait(&tl.stage_free[slot], (((uint32_t)item >> slot_shift) & 1u) ^ 1u, &tl.abort_flag)) return;
-        stage[slot].sum[cq][pos_in_tile] = part;
-        // the tile's record travels with its sums (the ring it came from may be reused before the tile is finished)
-        if (warp == 0 && lane < 8)
-            reinterpret_cast<uint32_t *>(&stage[slot].info)[lane] = reinterpret_cast<const uint32_t *>(inf)[lane];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tl.chunk_ready[slot]);
     }
 }
 
@@ -959,7 +886,8 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
     // it took one warp 28 us, which ended the launch.
     int run_u = -1, run_ntiles = 0, run_ib = 0, run_tiles = 0;
     uint32_t run_max = 0;                       // largest score of the run (bit pattern)
-    const int U = a.p.num_seqs * a.heads_b;
+    const int Hkv = a.p.num_kv_heads, U1 = a.p.num_seqs * Hkv, U = U1 * a.layers_b;
+    const bool two_products = a.sh.cblocks > 1;
     auto close_run = [&]() {
         if (run_u < 0 || run_tiles == 0) return;
         if (lane == 0) atomicMax(&a.tickets[U + run_u], run_max);      // the unit's largest score, beside its count
@@ -979,9 +907,9 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
                 if (lane == 0) { tl.rule_unit[k] = run_u; tl.rule_max[k] = umax; tl.rule_n = k + 1; }
                 __syncwarp();
             } else {
-                const int s = run_u / a.heads_b, g = run_u - s * a.heads_b;
-                const Cut cut = select_unit_from_groups_warp(a.p, a.scores + (int64_t)g * a.total_tokens + sv.pack[s], sv.len[s],
-                                                             a.groups + (int64_t)run_ib * 4, umax);
+                const int l = run_u / U1, u = run_u - l * U1, s = u / Hkv, g = u - s * Hkv;
+                const Cut cut = select_unit_from_groups_warp(a.p, a.scores + (int64_t)(l * Hkv + g) * a.total_tokens + sv.pack[s],
+                                                             sv.len[s], a.groups + (int64_t)run_ib * 4, umax);
                 if (lane == 0) {
                     *unit_length(a, run_u) = cut.b;
                     if (a.sel_cuts) a.sel_cuts[run_u] = cut;
@@ -1008,10 +936,13 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
             {
                 const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[0][p0]);
                 const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[1][p0]);
-                const float4 u = *reinterpret_cast<const float4 *>(&stage[slot].sum[2][p0]);
-                const float4 v = *reinterpret_cast<const float4 *>(&stage[slot].sum[3][p0]);
-                tot[0] = (x.x + y.x) + (u.x + v.x); tot[1] = (x.y + y.y) + (u.y + v.y);
-                tot[2] = (x.z + y.z) + (u.z + v.z); tot[3] = (x.w + y.w) + (u.w + v.w);
+                tot[0] = x.x + y.x; tot[1] = x.y + y.y; tot[2] = x.z + y.z; tot[3] = x.w + y.w;
+            }
+            if (two_products) {
+                const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[2][p0]);
+                const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[3][p0]);
+                tot[0] += x.x; tot[1] += x.y; tot[2] += x.z; tot[3] += x.w;
+                tot[0] += y.x; tot[1] += y.y; tot[2] += y.z; tot[3] += y.w;
             }
             float sc[4];
             uint32_t bits[4];
@@ -1047,7 +978,8 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int pos = q * 32 + lane, i = tile * kTile + pos;
-            const float tot = (stage[slot].sum[0][pos] + stage[slot].sum[1][pos]) + (stage[slot].sum[2][pos] + stage[slot].sum[3][pos]);
+            float tot = stage[slot].sum[0][pos] + stage[slot].sum[1][pos];
+            if (two_products) { tot += stage[slot].sum[2][pos]; tot += stage[slot].sum[3][pos]; }
             const int cnt_i = max(1, min(min(w, n), n - i));
             float sc = 0.f;
             if (i < n) {
@@ -1200,11 +1132,12 @@ __device__ inline void copy_loop(const TcArgs &a, TcSmemTail &tl, const SeqView 
 // The stopping rule of the units on the CTA's list, by all threads of the CTA.
 __device__ inline void evaluate_rules(const TcArgs &a, TcSmemTail &tl, const SeqView &sv)
 {
+    const int Hkv = a.p.num_kv_heads, U1 = a.p.num_seqs * Hkv, items = sv.tiles[a.p.num_seqs] * Hkv;
     for (int k = 0; k < tl.rule_n; ++k) {
-        const int u = tl.rule_unit[k], s = u / a.heads_b, g = u - s * a.heads_b;
+        const int u = tl.rule_unit[k], l = u / U1, s = (u - l * U1) / Hkv, g = (u - l * U1) - s * Hkv;
         const int nt = sv.tiles[s + 1] - sv.tiles[s];
-        const UnitRule ur(a.p, a.scores + (int64_t)g * a.total_tokens + sv.pack[s], sv.len[s],
-                          a.groups + ((int64_t)sv.tiles[s] * a.heads_b + (int64_t)g * nt) * 4, tl.rule_max[k]);
+        const UnitRule ur(a.p, a.scores + (int64_t)(l * Hkv + g) * a.total_tokens + sv.pack[s], sv.len[s],
+                          a.groups + ((int64_t)l * items + (int64_t)sv.tiles[s] * Hkv + (int64_t)g * nt) * 4, tl.rule_max[k]);
         block_unit_rule<kThreadsTc>(ur, tl.rule, unit_length(a, u), a.sel_cuts ? a.sel_cuts + u : nullptr);
     }
 }
@@ -1232,11 +1165,11 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == kEpiWarps * 32) {
-        for (int l = 0; P1 && l * a.p.num_kv_heads < a.heads_a; ++l) {
+        for (int l = 0; P1 && l < a.layers_a; ++l) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps_a.q[l]) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps_a.k[l]) : "memory");
         }
-        for (int l = 0; P2 && l * a.p.num_kv_heads < a.heads_b; ++l) {
+        for (int l = 0; P2 && l < a.layers_b; ++l) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps_b.q[l]) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps_b.k[l]) : "memory");
         }
@@ -1245,8 +1178,13 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
         for (int s = 0; s < 4; ++s) { mbar_init(&tl.k_full[s], 1); mbar_init(&tl.k_empty[s], 1); }
         mbar_init(&tl.q_full, 1);
         mbar_init(&tl.q_empty, 1);
-        for (int b = 0; b < 2; ++b) { mbar_init(&tl.acc_full[b], 1); mbar_init(&tl.acc_empty[b], kEpiWarps); }
-        for (int b = 0; b < kStageSlots; ++b) { mbar_init(&tl.chunk_ready[b], kEpiWarps); mbar_init(&tl.stage_free[b], 1); }
+        // a group of eight warps hands an accumulator back
+        for (int b = 0; b < 4; ++b) { mbar_init(&tl.p1_full[b], 1); mbar_init(&tl.p1_empty[b], kEpiWarps / 2); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&tl.p2_full[b], 1); mbar_init(&tl.p2_empty[b], kEpiWarps / 2); }
+        for (int b = 0; b < kStageSlots; ++b) {
+            mbar_init(&tl.chunk_ready[b], sh.cblocks * (kEpiWarps / 2));
+            mbar_init(&tl.stage_free[b], 1);
+        }
         mbar_init(&tl.epi_bar, kEpiWarps);
         for (int b = 0; b < kMaxCopySlots; ++b) mbar_init(&tl.c_full[b], 1);
         tl.abort_flag = 0;
@@ -1281,26 +1219,12 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
     SeqView sv;
     sv.pack = t_pack; sv.tiles = t_tiles; sv.len = t_len; sv.start = t_start; sv.ne = t_ne;
 
-    // ranges over min(grid, items) CTAs, so that every CTA that has a range has a non-empty one
-    Split sp_b;                                  // pass 2
-    int a0 = 0, na = 0, b0 = 0, nb = 0;          // items of pass 1 and of pass 2: the first, how many
-    if (P2) {
-        sp_b = make_split(sv, B, a.heads_b, (int)gridDim.x);
-        if ((int)blockIdx.x < sp_b.ctas && sp_b.items > 0) {
-            b0 = range_begin(sp_b, sv, B, blockIdx.x);
-            nb = range_begin(sp_b, sv, B, blockIdx.x + 1) - b0;
-        }
-    }
-    if (P1 && (!P2 || a.heads_a != a.heads_b)) {
-        const Split sp_a = make_split(sv, B, a.heads_a, (int)gridDim.x);
-        if ((int)blockIdx.x < sp_a.ctas && sp_a.items > 0) {
-            a0 = range_begin(sp_a, sv, B, blockIdx.x);
-            na = range_begin(sp_a, sv, B, blockIdx.x + 1) - a0;
-        }
-    } else if (P1) {
-        a0 = b0;
-        na = nb;
-    }
+    // the layer's items in min(SMs, items) ranges, so that no range is empty
+    const Split sp = make_split(sv, B, a.p.num_kv_heads, a.split_ctas);
+    Share sh_a = {0, 0, 0}, sh_b = {0, 0, 0};    // pass 1, pass 2
+    if (P2) sh_b = cta_share(sp, sv, B, a.layers_b);
+    if (P1) sh_a = P2 && a.layers_a == a.layers_b ? sh_b : cta_share(sp, sv, B, a.layers_a);
+    const int na = sh_a.count, b0 = sh_b.first, nb = sh_b.count;
 
     // A run of layers: the launch that follows may put a CTA on an SM as soon as this one's has left it (programmatic
     // dependent launch; 8K positions: 41 us a layer against 45 without).  What such an early CTA does before griddepcontrol.wait must not need this launch's results:
@@ -1311,10 +1235,10 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
     if (blockIdx.x == 0 && !inputs_only) {
         const int t0 = threadIdx.x < kEpiWarps * 32 ? threadIdx.x : threadIdx.x - 64;
         if (P1 && a.tickets_next)
-            for (int t = t0; t < 2 * B * a.heads_a; t += kThreadsTc - 64) a.tickets_next[t] = 0u;
+            for (int t = t0; t < 2 * B * a.p.num_kv_heads * a.layers_a; t += kThreadsTc - 64) a.tickets_next[t] = 0u;
         if (P2 && a.tickets)                      // an empty sequence has no tile to finish: it keeps nothing
-            for (int t = t0; t < B * a.heads_b; t += kThreadsTc - 64)
-                if (t_len[t / a.heads_b] == 0) {
+            for (int t = t0; t < B * a.p.num_kv_heads * a.layers_b; t += kThreadsTc - 64)
+                if (t_len[t / a.p.num_kv_heads % B] == 0) {
                     Cut cut;
                     cut.b = 0; cut.ties = 0; cut.tau = 0; cut.prot_kept = 0; cut.sbias = 0;
                     *unit_length(a, t) = 0;
@@ -1324,22 +1248,19 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
 
     if (warp < kEpiWarps) {
         EpiState es;
-        if (MODE == 3) epilogue_pass2(a, tl, stage, sv, tmem_base, b0, nb, sp_b, es);
-        if (P1 && na > 0) epilogue_pass1(a, tl, sv, tmem_base, es);
-        if (MODE == 2) epilogue_pass2(a, tl, stage, sv, tmem_base, b0, nb, sp_b, es);
+        if (P2) epilogue_pass2(a, tl, stage, sv, tmem_base, b0, nb, sp, es);
+        if (P1 && na > 0 && !tl.abort_flag) epilogue_pass1(a, tl, tmem_base, es);
     } else if (warp == kEpiWarps) {
         if (lane == 0) {
             RingState rs;
-            if (MODE == 3) producer_loop<false>(a, maps_b, smem_q, smem_k, tl, sv, b0, b0 + nb, rs);
-            if (P1) producer_loop<true>(a, maps_a, smem_q, smem_k, tl, sv, a0, a0 + na, rs);
-            if (MODE == 2) producer_loop<false>(a, maps_b, smem_q, smem_k, tl, sv, b0, b0 + nb, rs);
+            if (P2) producer_loop<false>(a, maps_b, smem_q, smem_k, tl, sv, sp, sh_b, rs);
+            if (P1) producer_loop<true>(a, maps_a, smem_q, smem_k, tl, sv, sp, sh_a, rs);
         }
     } else if (warp == kEpiWarps + 1) {
         if (lane == 0) {
             MmaState ms;
-            if (MODE == 3 && nb > 0) mma_loop_pass2(a, smem_q, smem_k, tl, tmem_base, ms, true);
+            if (P2 && nb > 0) mma_loop_pass2(a, smem_q, smem_k, tl, tmem_base, ms, P1);
             if (P1 && na > 0 && !tl.abort_flag) mma_loop_pass1(a, smem_q, smem_k, tl, tmem_base, ms);
-            if (MODE == 2 && nb > 0 && !tl.abort_flag) mma_loop_pass2(a, smem_q, smem_k, tl, tmem_base, ms, false);
         }
     } else if (warp == kEpiWarps + 2) {
         if (a.cj.nslots > 0) copy_loop(a, tl, sv, smem_c, coff);
@@ -1545,17 +1466,14 @@ cudaError_t launch_score_tc_pipe(const refree_params &p, const TcGroup *begin, c
     a.seq_len = seq_len;
     a.total_tokens = total_tokens;
     a.dev_status = dev_status;
+    a.split_ctas = di.sms;
     if (begin) {
-        a.heads_a = begin->layers * p.num_kv_heads;
+        a.layers_a = begin->layers;
         a.part_a = begin->part;
-        for (int l = 0; l < begin->layers; ++l) {
-            a.q_a[l] = static_cast<const __nv_bfloat16 *>(begin->q_win[l]);
-            a.k_a[l] = static_cast<const __nv_bfloat16 *>(begin->k[l]);
-        }
         a.tickets_next = begin->tickets;
     }
     if (finish) {
-        a.heads_b = finish->layers * p.num_kv_heads;
+        a.layers_b = finish->layers;
         a.part_b = finish->part;
         a.scores = finish->scores;
         a.groups = finish->groups;
@@ -1581,8 +1499,8 @@ cudaError_t launch_score_tc_pipe(const refree_params &p, const TcGroup *begin, c
 }
 
 // Both passes of one layer: a run of one, two launches of which the second starts while the first drains.  (One
-// cooperative launch for both, which waited on flags between the passes, was slower: four layers of 8 units of 256 rows,
-// us, 8K positions 260 -> 252, 32K 522 -> 508; 8 units of 512 rows, 8K 315 -> 287; 2 units of 371 positions 144 -> 138.)
+// cooperative launch for both, which waited on flags between the passes, was slower: score, selection and copy of a
+// layer of 8 units of 256 rows, us, 8K positions 72.1 -> 68.1, 32K 154.0 -> 152.1.)
 cudaError_t launch_score_tc(const refree_params &p, const void *q_win, const void *k,
                             const int32_t *seq_start, const int32_t *seq_len,
                             int64_t total_tokens, float *scores, char *ws, const Workspace &lay,

@@ -1,5 +1,6 @@
 """GPU parity of the tensor-core scoring path (bf16, head_dim 128) and of the
 fused pass on bf16 caches, against the CPU oracle."""
+import math
 import dataclasses
 
 import numpy as np
@@ -132,3 +133,36 @@ def test_tc_few_query_rows_are_padded(hq, hkv, w):
     cfg = cfg_with(num_q_heads=hq, num_kv_heads=hkv, window=w)
     lay = workloads.make_layer(cfg, 2, seq_lens=[700, 3, 129])
     parity.run_fused_and_check(cfg, lay)
+
+
+@pytest.mark.parametrize("hq,hkv,w,lens,layers", [(32, 8, 64, [16384], 6), (28, 4, 64, [9877, 4096, 640], 4), (8, 2, 16, [2000, 77], 11),
+                                                  (48, 4, 32, [5000], 5)])
+@pytest.mark.parametrize("small_workspace", [False, True])
+@pytest.mark.parametrize("rank_mode", [0, 1])
+def test_run_of_layers_scores_a_layer_as_alone(hq, hkv, w, lens, layers, small_workspace, rank_mode):
+    """A layer's scores are the same bits whatever shares its launch (a budget on a near-tie would else depend on the length
+    of the run and on the workspace).  A run does not return scores; those of its last layers are still in the workspace."""
+    d, total = 128, sum(lens)
+    gen = torch.Generator(device=DEV).manual_seed(11)
+    mu = torch.randn(layers, 1, hkv, 1, 1, d, generator=gen, device=DEV)
+    q = torch.randn(layers, len(lens), hkv, hq // hkv, w, d, generator=gen, device=DEV)
+    q = list(((q + mu) / math.sqrt(2)).view(layers, len(lens), hq, w, d).to(torch.bfloat16))
+    k = list(torch.randn(layers, hkv, total, d, generator=gen, device=DEV).to(torch.bfloat16))
+    sl = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    ss = torch.tensor([sum(lens[:i]) for i in range(len(lens))], dtype=torch.int32, device=DEV)
+    p = binding.Params(num_seqs=len(lens), num_q_heads=hq, num_kv_heads=hkv, head_dim=d, window=w, kv_tokens=total,
+                       rank_mode=rank_mode, k_strides=(0, d, total * d), v_strides=(0, d, total * d))
+    ko, vo = [list(torch.empty(layers, hkv * total, d, dtype=torch.bfloat16, device=DEV)) for _ in range(2)]
+    lengths = list(torch.zeros(layers, len(lens) * hkv, dtype=torch.int32, device=DEV))
+    off = list(torch.zeros(layers, len(lens) * hkv + 1, dtype=torch.int64, device=DEV))
+    size = 2 * binding.refree_workspace_size(p, total) if small_workspace else binding.refree_layers_workspace_size(p, total)
+    ws = torch.zeros(size // 4, dtype=torch.int32, device=DEV)
+    binding.refree_compress_layers(p, binding.LayerPointers(q, k, k, ko, vo, lengths, off), ss, sl, total, hkv * total, ws)
+    scores = torch.zeros(hkv, total, dtype=torch.float32, device=DEV)
+    ws1 = torch.empty(binding.refree_workspace_size(p, total), dtype=torch.uint8, device=DEV)
+    binding.refree_score(p, q[-1], k[-1], ss, sl, total, scores, ws1)
+    torch.cuda.synchronize()
+    want = parity.bits(scores).reshape(-1)
+    key = want[want.numel() // 3]                      # a value from the middle says where the array may lie
+    at = [int(i) - want.numel() // 3 for i in (ws == key).nonzero()]
+    assert any(0 <= i <= ws.numel() - want.numel() and torch.equal(ws[i:i + want.numel()], want) for i in at)
