@@ -57,7 +57,9 @@ constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kMaxRowsTc = 512;
 constexpr int kMaxCtas = 256;
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kZLimit = 1.2676506e30f;         // 2^100: a tile sum above this is redone with a fresh reference
+// 2^100: the sum of a tile's half above this is taken again with a fresh reference.  A row has fewer than 2^25 such sums, so
+// neither a run's nor the row's total can leave the range of fp32.
+constexpr float kZLimit = 1.2676506e30f;
 
 // ------------------------------------------------------------------ PTX ------
 __device__ inline uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }

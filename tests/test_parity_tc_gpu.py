@@ -108,9 +108,9 @@ def test_tc_large_logits_do_not_overflow():
 
 @pytest.mark.parametrize("hq,hkv,w,n", [(8, 2, 16, 40_000), (8, 2, 64, 30_001), (14, 2, 64, 21_000), (8, 1, 64, 60_100)])
 def test_tc_logits_that_outgrow_the_reference_of_a_run(hq, hkv, w, n):
-    """A row's sum over a CTA's tiles is taken against the largest logit of its first tiles; keys that are far louder in
-    later tiles of the run take it out of fp32's range, and the row is formed again.  (Enough tiles that a CTA has several
-    pairs of them, an odd last one among them; 1, 2 and 4 row blocks.)"""
+    """A row's sum over a CTA's tiles is taken against the largest logit of its first tile; keys that are far louder in
+    later tiles of the run take it out of fp32's range, and the reference is renewed.  (Enough tiles that a CTA has several
+    of them; 1, 2 and 4 row blocks.)"""
     cfg = cfg_with(num_q_heads=hq, num_kv_heads=hkv, window=w)
     lay = workloads.make_layer(cfg, 1, seq_lens=[n])
     for g in range(hkv):
@@ -166,3 +166,27 @@ def test_run_of_layers_scores_a_layer_as_alone(hq, hkv, w, lens, layers, small_w
     key = want[want.numel() // 3]                      # a value from the middle says where the array may lie
     at = [int(i) - want.numel() // 3 for i in (ws == key).nonzero()]
     assert any(0 <= i <= ws.numel() - want.numel() and torch.equal(ws[i:i + want.numel()], want) for i in at)
+
+
+@pytest.mark.parametrize("loud", [45.75, 46.0, 55.75, 90.0])
+def test_tc_row_sums_far_above_the_reference_stay_finite(loud):
+    """One long unit over every SM, each range of it quiet in its first two tiles, from which a row's reference comes, and
+    loud behind them: tile sums of 2^99.4 and 2^99.9 (just inside the limit), 2^119.8 and beyond fp32, added up over some
+    hundred ranges."""
+    n, w = 60_100, 64
+    p = binding.Params(num_seqs=1, num_q_heads=4, num_kv_heads=1, head_dim=128, window=w, kv_tokens=n,
+                       k_strides=(0, 128, n * 128), v_strides=(0, 128, n * 128))
+    q, k = torch.zeros(1, 4, w, 128, dtype=torch.bfloat16), torch.zeros(1, n, 128, dtype=torch.bfloat16)
+    q[..., 0] = 16.0
+    tiles, ctas = -(-n // 128), torch.cuda.get_device_properties(0).multi_processor_count
+    begins = [-(-c * tiles // ctas) for c in range(ctas + 1)]
+    for b, e in zip(begins, begins[1:]):
+        k[0, 128 * (b + 2):128 * e, 0] = loud
+    sl, ss = torch.tensor([n], dtype=torch.int32), torch.zeros(1, dtype=torch.int32)
+    ws = torch.empty(binding.refree_workspace_size(p, n), dtype=torch.uint8, device=DEV)
+    scores = torch.full((1, n), float("nan"), device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    binding.refree_score(p, q.to(DEV), k.to(DEV), ss.to(DEV), sl.to(DEV), n, scores, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    parity.check_scores(scores, orc.score(parity.oracle_params(p), q, k, ss, sl))
