@@ -1437,7 +1437,7 @@ cudaError_t encode_maps(const refree_params &p, const TcShape &sh, const void *q
 
 // One launch of a run of layers: pass 2 of `finish` (nullable), then pass 1 of `begin` (nullable), and the rows
 // of `copy` (nullable) beside them.  The partials that pass 2 reads were completed by an earlier launch on the
-// stream, so no CTA waits for another and the launch is an ordinary one.
+// stream, so no CTA waits for another: the launch is not a cooperative one.
 cudaError_t launch_score_tc_pipe(const refree_params &p, const TcGroup *begin, const TcGroup *finish,
                                  const int32_t *seq_start, const int32_t *seq_len, int64_t total_tokens,
                                  int32_t *dev_status, Stream st, const TcCopyJob *copy, bool first)
@@ -1490,11 +1490,13 @@ cudaError_t launch_score_tc_pipe(const refree_params &p, const TcGroup *begin, c
     a.cj.piece_rows = piece_rows;
     const size_t smem = smem_bytes(sh, p.num_seqs, a.cj.nslots, piece_rows, p.num_seqs * p.num_kv_heads * a.cj.layers);
     if (smem > kSmemLimit) return cudaErrorInvalidValue;
-    // Launches of a run after the first may start while the one before drains: their CTAs set themselves up and
-    // then wait (griddepcontrol.wait) until that launch has completed and its results are visible.
-    a.dependent = first ? 0 : 1;
+    // Launches of a run after the first may start while the one before drains (unless the stream is not to be chained):
+    // their CTAs set themselves up and then wait (griddepcontrol.wait) until that launch has completed and its results are
+    // visible.
+    const bool chain = st.chain && !first;
+    a.dependent = chain ? 1 : 0;
     auto *kern = begin && finish ? score_tc_kernel<3> : begin ? score_tc_kernel<1> : score_tc_kernel<2>;
-    e = launch_dependent(kern, dim3(ctas), dim3(kThreadsTc), smem, Stream(st.s, !first), maps[0], maps[1], a);
+    e = launch_dependent(kern, dim3(ctas), dim3(kThreadsTc), smem, Stream(st.s, chain), maps[0], maps[1], a);
     if (e != cudaSuccess) return e;
     count_launches(1);
     return cudaGetLastError();
