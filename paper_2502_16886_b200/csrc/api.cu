@@ -648,10 +648,16 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
     if (!workspace || workspace_bytes < 2 * lay.total || (reinterpret_cast<uintptr_t>(workspace) & 255))
         return REFREE_ERR_WORKSPACE;
     if (num_layers == 0) return REFREE_OK;
+    // One layer has nothing to overlap with (fp32, 111 positions, w = 1: 57 us on two streams, 45 this way).
+    if (num_layers == 1) {
+        const Stream cs = (cudaStream_t)stream;
+        return enqueue_layer(p, q_win[0], k[0], v[0], seq_start, seq_len, total_tokens, k_out[0], v_out[0], capacity_rows,
+                             lengths[0], offsets[0], nullptr, nullptr, (char *)workspace, lay, device_status, cs, cs, nullptr);
+    }
     // Tensor-core path: one stream, layers in groups, no internal streams or events.  With position ranking and the rows of
     // a unit contiguous the scoring kernel of a group moves the kept rows of an earlier group with a warp of its own, and
     // the last group is compacted by a launch of its own; else selection and copy of a group are launches between.
-    bool fused = num_layers >= 2 && total_tokens > 0 && !p->force_full;
+    bool fused = total_tokens > 0 && !p->force_full;
     for (int l = 0; l < num_layers && fused; ++l) fused = use_tc(*p, q_win[l]);
     const bool by_score = p->rank_mode == REFREE_RANK_SCORE;
     const bool copy = fused && !by_score && score_tc_can_copy(*p, total_tokens);
@@ -749,7 +755,7 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
     // Single query row: scoring is a chain of short kernels, so the layers of a group go through each of them together, and
     // then through one copy.  (In place of one layer after the other with the copies on a second stream; a run, us: eight
     // layers of 32K positions 548 -> 512, 16 of 8K 543 -> 272, eight of 333 198 -> 18, with score ranking at 32K 653 -> 459.)
-    const int w1_n = num_layers >= 2 && total_tokens > 0 && !p->force_full && score_w1_supported(*p)
+    const int w1_n = total_tokens > 0 && !p->force_full && score_w1_supported(*p)
                          ? w1_batch(*p, total_tokens, num_layers, workspace_bytes) : 0;
     if (w1_n > 0 && w1_batch_layout(*p, total_tokens, w1_n).total <= workspace_bytes) {
         cudaStream_t cs = (cudaStream_t)stream;
