@@ -356,7 +356,9 @@ refree_status refree_select_budget_static(const refree_params *p, const float *s
  *            an empty segment gives a zero row
  *   workspace  refree_decode_workspace_size(params, max_rows_per_unit) bytes, 256-byte
  *            aligned (device, scratch).
- * Only num_seqs, num_q_heads, num_kv_heads, head_dim and dtype of params are read.
+ * Only num_seqs, num_q_heads, num_kv_heads, head_dim and dtype of params matter to the
+ * result; kv_tokens and k_stride_seq, where they describe the cache that was compressed,
+ * tell how ragged the lengths can be and with that how the rows are cut into blocks.
  * Products are exact (bf16) or fp32, sums and the softmax are fp32. */
 refree_status refree_decode_workspace_size(const refree_params *params, int64_t max_rows_per_unit, size_t *bytes);
 refree_status refree_decode_attention(const refree_params *params, const void *q_new,

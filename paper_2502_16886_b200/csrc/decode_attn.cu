@@ -721,7 +721,8 @@ int decode_shape(const refree_params &p, int64_t max_rows, bool mma, int &blocks
     // plan costs 1 to 3 us a call (24 units of 5000 rows: 20.8 us, fixed 19.1) and pays where the longest sequence is far
     // above the mean (8 heads, sequences of 20000, 2500, 1000 and 300 rows: 25.9 us, fixed 53.9; of 5000, 700, 300 and
     // 100: 15.4 and 18.9), as long as a unit can have two pieces.
-    if (2 * U <= std::min<int64_t>(sms, 2 * kPlanUnits) && p.num_seqs > 1 && p.kv_tokens > 0 && max_rows * p.num_seqs >= 3 * p.kv_tokens) {
+    const int64_t few = max_rows * p.num_seqs / 3 / (p.k_stride_seq != 0 ? p.num_seqs : 1);   // kv_tokens is per sequence, or of all
+    if (2 * U <= std::min<int64_t>(sms, 2 * kPlanUnits) && p.num_seqs > 1 && p.kv_tokens > 0 && p.kv_tokens <= few) {
         blocks = (int)sms;
         return kPlanned;
     }

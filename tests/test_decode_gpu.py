@@ -154,3 +154,31 @@ def test_units_of_very_different_lengths(units, hkv, longest, dtype, d, told):
     for lengths in (mixed, [longest] * units):
         check_against_oracle(units // hkv, 3 * hkv, hkv, d, dtype, lengths, seed=units + longest,
                              kv_tokens=max(1, sum(lengths) // (2 * hkv)) if told else 0)
+
+
+@pytest.mark.parametrize("lens", [[5000, 4700, 4100], [5000, 300, 100, 64]])
+def test_batch_strided_cache_takes_no_plan(lens):
+    """kv_tokens of a cache with a sequence stride is the extent of one sequence: a batch of full sequences is not ragged."""
+    B, hkv, G, d, n = len(lens), 2, 3, 128, max(lens)
+    gen = torch.Generator().manual_seed(3)
+    q, k, v = [torch.randn(s, generator=gen).to(torch.bfloat16) for s in ((B, hkv * G, d), (B, hkv, n, d), (B, hkv, n, d))]
+    p = binding.Params(num_seqs=B, num_q_heads=hkv * G, num_kv_heads=hkv, head_dim=d, kv_tokens=n, dtype=binding.DTYPE_BF16,
+                       k_strides=(hkv * n * d, d, n * d), v_strides=(hkv * n * d, d, n * d))
+    dev = [t.to(DEV) for t in (q, k, v)]
+    starts, sl = torch.zeros(B, dtype=torch.int32, device=DEV), torch.tensor(lens, dtype=torch.int32, device=DEV)
+    lengths = sl.repeat_interleave(hkv)
+    out = torch.zeros(B, hkv * G, d, device=DEV)
+    ws = torch.empty(binding.refree_decode_workspace_size(p, n), dtype=torch.uint8, device=DEV)
+
+    got = []
+    for tokens in (n, 0):                           # without a hint there is no plan
+        p.kv_tokens = tokens
+        binding.refree_decode_attention_inplace(p, *dev, starts, sl, lengths, binding.ANCHOR_FRONT, n, out, ws)
+        torch.cuda.synchronize()
+        got.append(out.cpu().numpy())
+    np.testing.assert_array_equal(got[0], got[1])   # the same cut: the same bits
+    rows = torch.cat([k[b, h, :lens[b]] for b in range(B) for h in range(hkv)])
+    vals = torch.cat([v[b, h, :lens[b]] for b in range(B) for h in range(hkv)])
+    off = np.concatenate([[0], np.cumsum(np.repeat(lens, hkv))])
+    want = orc.decode_attention(orc.OracleParams(B, hkv * G, hkv, d, dtype=1), q, rows, vals, off)
+    np.testing.assert_allclose(got[0], want, rtol=RTOL, atol=ATOL)
