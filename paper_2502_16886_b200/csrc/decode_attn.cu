@@ -504,11 +504,13 @@ __device__ inline void decode_lanes(const DecArgs &a, const Piece &pc, float *de
         float kf[RB][E], vf[RB][E];
 #pragma unroll
         for (int i = 0; i < RB; ++i) {
-            const int row = min(row0 + i * NW, end - 1);
+            const bool in = row0 + i * NW < end;
+            const int row = in ? row0 + i * NW : end - 1;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 kf[i][e] = to_float(kc[(int64_t)row * D + lane * E + e]);
-                vf[i][e] = to_float(vc[(int64_t)row * D + lane * E + e]);
+                const float x = to_float(vc[(int64_t)row * D + lane * E + e]);
+                vf[i][e] = in ? x : 0.f;             // (zero times an infinity must not reach the sums)
             }
         }
 #pragma unroll

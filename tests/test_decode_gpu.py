@@ -182,3 +182,21 @@ def test_batch_strided_cache_takes_no_plan(lens):
     off = np.concatenate([[0], np.cumsum(np.repeat(lens, hkv))])
     want = orc.decode_attention(orc.OracleParams(B, hkv * G, hkv, d, dtype=1), q, rows, vals, off)
     np.testing.assert_allclose(got[0], want, rtol=RTOL, atol=ATOL)
+
+
+@pytest.mark.parametrize("dtype,d,G", [("fp32", 64, 2), ("fp32", 128, 12)])
+@pytest.mark.parametrize("n", [1, 13, 77])
+def test_infinity_in_the_last_row_of_a_unit(dtype, d, G, n):
+    """Rows past the end of a unit weigh nothing, whatever is read in their place."""
+    tdt = torch.float32 if dtype == "fp32" else torch.bfloat16
+    k_c, v_c, offsets = workloads.make_ragged_cache(5, [n, n], d, tdt)
+    v_c[n - 1, 3], v_c[2 * n - 1, d - 1] = float("inf"), float("-inf")
+    q_new = torch.randn((1, 2 * G, d), generator=torch.Generator().manual_seed(6)).to(tdt)
+    p = binding.Params(num_seqs=1, num_q_heads=2 * G, num_kv_heads=2, head_dim=d,
+                       dtype=binding.DTYPE_F32 if dtype == "fp32" else binding.DTYPE_BF16)
+    got, status = run_decode(p, q_new, k_c, v_c, offsets, n)
+    want = orc.decode_attention(orc.OracleParams(1, 2 * G, 2, d, dtype=0 if dtype == "fp32" else 1), q_new, k_c, v_c,
+                                offsets.numpy())
+    assert status == 0
+    assert np.isinf(want).sum() == 2 * G
+    np.testing.assert_allclose(got, want, rtol=RTOL, atol=ATOL)
