@@ -238,7 +238,9 @@ refree_status refree_compress_layer_inplace(const refree_params *p, const void *
  * refree_compress_layer, whatever shares a launch.
  *   q_win, k, v, k_out, v_out, lengths, offsets  HOST arrays of `num_layers`
  *            DEVICE pointers, one per layer, each as in refree_compress_layer;
- *            the arrays themselves are read before the call returns
+ *            the arrays themselves are read before the call returns.  k_out and v_out
+ *            of a layer may lie over K and V of an earlier layer (layers then no longer
+ *            share a launch), not of its own or a later one
  *   seq_start, seq_len, total_tokens, capacity_rows  common to all layers (device
  *            pointers as in refree_compress_layer)
  *   workspace  refree_layers_workspace_size() bytes (two per-layer workspaces at least;

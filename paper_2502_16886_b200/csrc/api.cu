@@ -611,6 +611,27 @@ int run_batch(const refree_params &p, int64_t total_tokens, int num_layers, size
     while (n > 1 && ((copy && !score_tc_can_copy(p, total_tokens, n)) || 2 * batch_layout(p, total_tokens, n).total > workspace_bytes)) --n;
     return n;
 }
+
+// Whether a layer's output lies over the cache of one of the layers that could share a launch with it: a caller may write
+// a layer into the memory of an earlier one, whose rows have been moved by then if the layers are moved one by one.
+bool outputs_over_caches(const refree_params &p, int num_layers, const void *const *k, const void *const *v, void *const *k_out,
+                         void *const *v_out, int64_t capacity_rows)
+{
+    const size_t esz = p.dtype == REFREE_DTYPE_F32 ? 4 : 2, out = (size_t)capacity_rows * p.head_dim * esz;
+    auto extent = [&](int64_t seq, int64_t tok, int64_t head) {
+        return p.kv_tokens < 1 ? 0 : (size_t)((p.num_seqs - 1) * seq + (p.kv_tokens - 1) * tok + (p.num_kv_heads - 1) * head + p.head_dim) * esz;
+    };
+    const size_t kb = extent(p.k_stride_seq, p.k_stride_tok, p.k_stride_head), vb = extent(p.v_stride_seq, p.v_stride_tok, p.v_stride_head);
+    auto meet = [](const void *x, size_t nx, const void *y, size_t ny) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(x), b = reinterpret_cast<uintptr_t>(y);
+        return a < b + ny && b < a + nx;
+    };
+    for (int l = 1; l < num_layers; ++l)
+        for (int m = std::max(0, l - kMaxBatch + 1); m < l; ++m)
+            if (meet(k_out[l], out, k[m], kb) || meet(k_out[l], out, v[m], vb) || meet(v_out[l], out, k[m], kb) || meet(v_out[l], out, v[m], vb))
+                return true;
+    return false;
+}
 }  // namespace
 
 refree_status refree_layers_workspace_size(const refree_params *p, int64_t total_tokens, size_t *bytes)
@@ -659,6 +680,7 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
     // the last group is compacted by a launch of its own; else selection and copy of a group are launches between.
     bool fused = total_tokens > 0 && !p->force_full;
     for (int l = 0; l < num_layers && fused; ++l) fused = use_tc(*p, q_win[l]);
+    const bool one_by_one = outputs_over_caches(*p, num_layers, k, v, k_out, v_out, capacity_rows);
     const bool by_score = p->rank_mode == REFREE_RANK_SCORE;
     const bool copy = fused && !by_score && score_tc_can_copy(*p, total_tokens);
     if (fused) {
@@ -666,7 +688,7 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
         // the rows of group j - 2; then the last group's rows.  (Beyond their own launch the scores of a group are read by
         // the selection that follows it, before launch j + 1 writes into the same half of the workspace.)
         cudaStream_t cs = (cudaStream_t)stream;
-        const int n = run_batch(*p, total_tokens, num_layers, workspace_bytes, copy);
+        const int n = one_by_one ? 1 : run_batch(*p, total_tokens, num_layers, workspace_bytes, copy);
         const int ngroups = (num_layers + n - 1) / n;
         auto first_of = [&](int j) { return j < ngroups ? (int)((int64_t)num_layers * j / ngroups) : num_layers; };
         const BatchLayout bl = batch_layout(*p, total_tokens, n);
@@ -756,7 +778,7 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
     // then through one copy.  (In place of one layer after the other with the copies on a second stream; a run, us: eight
     // layers of 32K positions 548 -> 512, 16 of 8K 543 -> 272, eight of 333 198 -> 18, with score ranking at 32K 653 -> 459.)
     const int w1_n = total_tokens > 0 && !p->force_full && score_w1_supported(*p)
-                         ? w1_batch(*p, total_tokens, num_layers, workspace_bytes) : 0;
+                         ? one_by_one ? 1 : w1_batch(*p, total_tokens, num_layers, workspace_bytes) : 0;
     if (w1_n > 0 && w1_batch_layout(*p, total_tokens, w1_n).total <= workspace_bytes) {
         cudaStream_t cs = (cudaStream_t)stream;
         char *ws = (char *)workspace;
