@@ -777,7 +777,11 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
     // Single query row: scoring is a chain of short kernels, so the layers of a group go through each of them together, and
     // then through one copy.  (In place of one layer after the other with the copies on a second stream; a run, us: eight
     // layers of 32K positions 548 -> 512, 16 of 8K 543 -> 272, eight of 333 198 -> 18, with score ranking at 32K 653 -> 459.)
-    const int w1_n = total_tokens > 0 && !p->force_full && score_w1_supported(*p)
+    // Queries that start on 16 bytes take another kernel than those that do not: a run with both goes layer by layer, so that
+    // each layer takes the one that it takes alone.
+    int on16 = 0;
+    for (int l = 0; l < num_layers; ++l) on16 += !(reinterpret_cast<uintptr_t>(q_win[l]) & 15);
+    const int w1_n = total_tokens > 0 && !p->force_full && score_w1_supported(*p) && (on16 == 0 || on16 == num_layers)
                          ? one_by_one ? 1 : w1_batch(*p, total_tokens, num_layers, workspace_bytes) : 0;
     if (w1_n > 0 && w1_batch_layout(*p, total_tokens, w1_n).total <= workspace_bytes) {
         cudaStream_t cs = (cudaStream_t)stream;
