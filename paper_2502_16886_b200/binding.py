@@ -149,7 +149,10 @@ def _dp(t: Optional[torch.Tensor]):
 
 def _stream(stream):
     if stream is None:                         # torch.cuda.current_stream() builds a Stream object: 3 us against 0.3
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # (not a public function)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
 

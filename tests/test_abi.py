@@ -124,3 +124,12 @@ def test_missing_library_is_an_error(monkeypatch, lib):
     monkeypatch.setattr(binding, "LIB_PATH", "/nonexistent/librefreekv.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.lib()
+
+
+def test_current_stream_without_the_private_function(monkeypatch):
+    import types
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=4711))
+    assert binding._stream(None) == 4711
+    assert binding._stream(types.SimpleNamespace(cuda_stream=12)) == 12
