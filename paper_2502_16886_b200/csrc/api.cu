@@ -450,7 +450,7 @@ static refree_status enqueue_layer(const refree_params *p, const void *q_win, co
             return REFREE_ERR_CUDA;
     }
     e = launch_compact(*p, compact_job(k, v, lengths, offsets, kept, lean ? offsets : nullptr, k_out, v_out), seq_start, seq_len,
-                       ranges, capacity_rows, device_status, cc, split);
+                       ranges, capacity_rows, device_status, cc);
     return from_cuda(e);
 }
 
@@ -842,7 +842,7 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
         if (l >= 2 && cudaStreamWaitEvent(lp->hi, lp->compacted[slot], 0) != cudaSuccess) { result = REFREE_ERR_CUDA; break; }
         result = enqueue_layer(p, q_win[l], k[l], v[l], seq_start, seq_len, total_tokens, k_out[l], v_out[l],
                                capacity_rows, lengths[l], offsets[l], nullptr, nullptr,
-                               (char *)workspace + (size_t)slot * lay.total, lay, device_status, Stream(lp->hi, false), Stream(lp->lo, false),
+                               (char *)workspace + (size_t)slot * lay.total, lay, device_status, lp->hi, lp->lo,
                                lp->scored[slot]);
         if (result != REFREE_OK) break;
         if (cudaEventRecord(lp->compacted[slot], lp->lo) != cudaSuccess) { result = REFREE_ERR_CUDA; break; }

@@ -14,7 +14,6 @@ namespace refree {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kThreadsSlim = 128;   // block of a launch beside another stream's scoring (see launch_compact)
 constexpr int kUnroll = 4;
 
 __device__ inline int4 ld_stream(const int4 *p)
@@ -30,7 +29,6 @@ __device__ inline void st_stream(int4 *p, const int4 &v)
                  :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-template <int kThreads>
 __global__ void __launch_bounds__(kThreads)
 compact_kernel(refree_params p, const __grid_constant__ CompactJob job, const int32_t *seq_start, const int32_t *seq_len,
                int position_ranges, int64_t capacity_rows, int32_t *dev_status)
@@ -333,29 +331,17 @@ static Stream copy_stream(const refree_params &p, Stream st, int layers = 1)
 }
 
 cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const int32_t *seq_start, const int32_t *seq_len,
-                           bool position_ranges, int64_t capacity_rows, int32_t *dev_status, Stream st, bool beside_scoring)
+                           bool position_ranges, int64_t capacity_rows, int32_t *dev_status, Stream st)
 {
     const int U = p.num_seqs * p.num_kv_heads;
     const int ranges = position_ranges ? 1 : 0;
-    if (beside_scoring) {
-        // The launch shares the SMs with the scoring of the next layer on another stream: many short-lived blocks of
-        // 128 threads, so that a scoring block that becomes runnable finds room as soon as a few of them retire (32K
-        // positions, run of layers with w = 1: 565 us, and 604 with the long-lived blocks below, which hold the SMs
-        // until the whole copy is done; fewer of those, two or three an SM, leave the copy short of loads in flight:
-        // 708 and 640).
-        const int gx = max(1, (sm_count() * 32) / (U * job.layers));
-        const cudaError_t e = launch_dependent(compact_kernel<kThreadsSlim>, dim3(gx, U, job.layers), dim3(kThreadsSlim), 0, st, p, job,
-                                               seq_start, seq_len, ranges, capacity_rows, dev_status);
-        count_launches(1);
-        return e;
-    }
     // Two waves of blocks; four times as many where a large copy takes several layers, so that a long unit among short ones
     // is not left to one or two blocks (seven layers of twelve sequences of 83 to 15815 positions, 8 heads: 928 us and 527;
     // small copies would pay for the blocks: 18 and 25 us).
     const Stream cs = copy_stream(p, st, job.layers);
     const int per_sm = job.layers > 1 && !cs.chain ? 32 : 8;
     const int gx = max(1, (sm_count() * per_sm) / (U * job.layers));
-    const cudaError_t e = launch_dependent(compact_kernel<kThreads>, dim3(gx, U, job.layers), dim3(kThreads), 0,
+    const cudaError_t e = launch_dependent(compact_kernel, dim3(gx, U, job.layers), dim3(kThreads), 0,
                                            cs, p, job, seq_start, seq_len, ranges, capacity_rows, dev_status);
     count_launches(1);
     return e;

@@ -153,9 +153,9 @@ template <typename Tv> __device__ inline Tv warp_incl_scan(Tv x)
 //     path, so that the end of a kernel means the end of all before it);
 //   - the first kernel of a call triggers its dependents after that wait, later ones may do so at once: what a kernel
 //     reads before its wait (sequence tables, queries, keys: inputs of the call) was complete before the first one.
-// A stream, and whether launches on it may be chained this way.  Not where a second stream works beside it: blocks
-// that wait for their turn would hold the room the other stream's kernels need (run of layers on two streams, 32K
-// positions: w = 1 608 us chained, 587 without; score ranking 1033 and 1002).
+// A stream, and whether the next launch on it may be chained this way.  Also where a second stream works beside it (a run
+// of layers on two streams, us, chained and not: fp32 d 64, eight layers of 3000 positions, 32 rows, 208 and 287; bf16 d 64,
+// four of 32K 325 and 370; windows in chunks, six layers of 2000 positions, 1200 rows, 766 and 841).
 struct Stream {
     cudaStream_t s;
     bool chain;
@@ -318,8 +318,7 @@ inline SelectOut select_out(int32_t *lengths, int64_t *offsets, int32_t *kept)
 }
 
 cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const int32_t *seq_start, const int32_t *seq_len,
-                           bool position_ranges, int64_t capacity_rows, int32_t *dev_status, Stream st,
-                           bool beside_scoring = false);
+                           bool position_ranges, int64_t capacity_rows, int32_t *dev_status, Stream st);
 inline CompactJob compact_job(const void *k, const void *v, const int32_t *lengths, const int64_t *offsets, const int32_t *kept,
                               int64_t *offsets_out, void *k_out, void *v_out)
 {
