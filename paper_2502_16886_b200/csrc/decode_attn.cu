@@ -559,8 +559,9 @@ __device__ inline void decode_lanes(const DecArgs &a, const Piece &pc, float *de
     merge_and_store<D, NW>(a, dec_sm, GMAX, G, pc);
 }
 
-// Every thread of the grid waits for what is ahead on the stream before it reads anything.
-template <int D, int GP, int NW, typename Body>
+// Every thread of the grid waits for what is ahead on the stream before it reads anything.  CLUSTER: a unit's blocks are a
+// cluster.
+template <int D, int GP, int NW, bool CLUSTER, typename Body>
 __device__ inline void decode_block(const DecArgs &a, float *dec_sm, Body body)
 {
     dependency_wait();
@@ -585,15 +586,15 @@ __device__ inline void decode_block(const DecArgs &a, float *dec_sm, Body body)
                 a.out[((int64_t)(pc.u / Hkv) * a.p.num_q_heads + (pc.u % Hkv) * G) * D + e] = 0.f;
     }
     if (pc.u >= 0 && pc.x < pc.nblocks) body(pc);
-    if (a.mode == kCluster) merge_cluster<D, NW>(a, dec_sm, GP, G, pc);
+    if (CLUSTER) merge_cluster<D, NW>(a, dec_sm, GP, G, pc);
 }
 
-template <int D, bool UPPER, int NW>
+template <int D, bool UPPER, int NW>                 // four warps: the blocks of a cluster, eight: those of a cut
 __global__ void __launch_bounds__(32 * NW, 8 / NW)
 decode_mma_kernel(DecArgs a)
 {
     extern __shared__ float dec_sm[];
-    decode_block<D, UPPER ? 16 : 8, NW>(a, dec_sm, [&](const Piece &pc) { decode_mma<D, UPPER, NW>(a, pc, dec_sm); });
+    decode_block<D, UPPER ? 16 : 8, NW, NW == 4>(a, dec_sm, [&](const Piece &pc) { decode_mma<D, UPPER, NW>(a, pc, dec_sm); });
 }
 
 template <typename T, int D, int GMAX, int NW>
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(32 * NW)
 decode_lanes_kernel(DecArgs a)
 {
     extern __shared__ float dec_sm[];
-    decode_block<D, GMAX, NW>(a, dec_sm, [&](const Piece &pc) { decode_lanes<T, D, GMAX, NW>(a, pc, dec_sm); });
+    decode_block<D, GMAX, NW, false>(a, dec_sm, [&](const Piece &pc) { decode_lanes<T, D, GMAX, NW>(a, pc, dec_sm); });
 }
 
 // One block per (unit, head) merges the unit's records and normalises.  kCombineThreads / D groups of threads, one
@@ -698,11 +699,12 @@ cudaError_t run_mma(const DecArgs &a, dim3 grid, int G, Stream st)
     return run_kernel(decode_mma_kernel<D, true, NW>, a, grid, NW, smem, st);
 }
 
-template <int D, int NW>
+template <int D>
 cudaError_t run_attention(const DecArgs &a, dim3 grid, int G, bool f32, Stream st)
 {
-    if (a.native) return run_mma<D, NW>(a, grid, G, st);
-    return f32 ? run_lanes<float, D, NW>(a, grid, G, st) : run_lanes<__nv_bfloat16, D, NW>(a, grid, G, st);
+    if (a.mode == kCluster) return run_mma<D, 4>(a, grid, G, st);      // (only the mma form goes by clusters)
+    if (a.native) return run_mma<D, 8>(a, grid, G, st);
+    return f32 ? run_lanes<float, D, 8>(a, grid, G, st) : run_lanes<__nv_bfloat16, D, 8>(a, grid, G, st);
 }
 
 // How a cache of at most max_rows rows per unit is cut: the mode, and the blocks per unit or of the grid.  Times are of one
@@ -765,9 +767,7 @@ cudaError_t launch_decode_attention(const refree_params &p, const void *q_new, c
     a.cap = (int)std::min<int64_t>(a.mode == kFixed ? (int64_t)a.span * a.blocks : (max_rows + 15) / 16 * 16, INT_MAX / 2);
     const int U = p.num_seqs * p.num_kv_heads, G = p.num_q_heads / p.num_kv_heads;
     const dim3 grid = a.mode == kPlanned ? dim3(a.blocks) : dim3(a.blocks, U);
-    cudaError_t e;
-    if (a.mode != kCluster) e = p.head_dim == 64 ? run_attention<64, 8>(a, grid, G, f32, st) : run_attention<128, 8>(a, grid, G, f32, st);
-    else e = p.head_dim == 64 ? run_attention<64, 4>(a, grid, G, f32, st) : run_attention<128, 4>(a, grid, G, f32, st);
+    cudaError_t e = p.head_dim == 64 ? run_attention<64>(a, grid, G, f32, st) : run_attention<128>(a, grid, G, f32, st);
     count_launches(1);
     if (e != cudaSuccess || a.mode == kCluster || a.blocks == 1) return e;
     e = p.head_dim == 64 ? launch_dependent(decode_combine_kernel<64>, dim3(U * G), dim3(kCombineThreads), 0, st, a)

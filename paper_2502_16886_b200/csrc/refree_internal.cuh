@@ -79,42 +79,6 @@ int sm_count();
 
 inline __host__ __device__ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// Per-CTA tables: running sums of sequence lengths and of tiles per sequence.
-struct SeqTables {
-    int32_t pack[kMaxSeqs + 1];   // positions before sequence s in the packed score array
-    int32_t tiles[kMaxSeqs + 1];  // scoring tiles before sequence s
-    int32_t len[kMaxSeqs];        // copy of seq_len (clamped at 0)
-};
-
-__device__ inline void build_seq_tables(SeqTables &t, const int32_t *seq_len, int B)
-{
-    if (threadIdx.x == 0) {
-        int32_t a = 0, b = 0;
-        for (int s = 0; s < B; ++s) {
-            t.pack[s] = a;
-            t.tiles[s] = b;
-            const int n = max(seq_len[s], 0);
-            t.len[s] = n;
-            a += n;
-            b += ceil_div(n, kTile);
-        }
-        t.pack[B] = a;
-        t.tiles[B] = b;
-    }
-    __syncthreads();
-}
-
-// Largest s with table[s] <= x (table ascending, table[0] == 0).
-__device__ inline int find_seq(const int32_t *table, int B, int x)
-{
-    int lo = 0, hi = B;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (table[mid] <= x) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 // |a| as an integer: non-negative floats order like their bit patterns
 __device__ inline uint32_t mag_bits(float a) { return __float_as_uint(a) & 0x7fffffffu; }
 
