@@ -234,7 +234,8 @@ refree_status refree_compress_layer_inplace(const refree_params *p, const void *
  * while the kept rows of an earlier one are copied.  On the tensor-core path
  * and with a single query row several layers share a launch (as many as the run's
  * length, their size and the workspace suggest), all on the caller's stream; other
- * shapes use two internal streams.  Results are bit-identical to num_layers calls of
+ * shapes, and runs whose queries do not all start on 16 bytes, use two internal
+ * streams (a run of one layer does not).  Results are bit-identical to num_layers calls of
  * refree_compress_layer, whatever shares a launch.
  *   q_win, k, v, k_out, v_out, lengths, offsets  HOST arrays of `num_layers`
  *            DEVICE pointers, one per layer, each as in refree_compress_layer;
@@ -249,8 +250,8 @@ refree_status refree_compress_layer_inplace(const refree_params *p, const void *
  * Index lists and scores are not returned (use the per-layer call for them).
  * Nothing is allocated in device memory and the host is not synchronised: the
  * work is ordered after what `stream` holds at the call, and `stream` continues
- * only when every layer is done.  The first call on a device creates the two
- * internal streams (highest priority for scoring, lowest for compaction) and
+ * only when every layer is done.  The first call on a device that takes two
+ * streams creates them (highest priority for scoring, lowest for compaction) and
  * their events, which live until the process exits; the device that owns
  * `stream` must be the current device of the calling thread.  Calls from
  * several host threads on one device share the internal streams and are

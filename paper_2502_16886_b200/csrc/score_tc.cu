@@ -377,8 +377,8 @@ struct TcArgs {
     float *scores;
     int64_t total_tokens;
     int32_t *dev_status;
-    // Stopping rule inside the launch (position ranking per head): the finishing warp that completes a unit's
-    // last tile (a ticket per unit) evaluates the rule from the unit's records.  All nullable.
+    // Stopping rule inside the launch (position ranking per head): the CTA whose finishing warp completes a unit's
+    // last tile (a ticket per unit) evaluates the rule from the unit's records when it has left its passes.  All nullable.
     int32_t *sel_lengths[kMaxBatch];   // budgets out, per layer of the group
     Cut *sel_cuts;             // [units]
     uint32_t *tickets;         // [2 units] tiles finished per unit, then the unit's largest score; zero when the launch begins
@@ -1304,7 +1304,9 @@ bool shape_for(const refree_params &p, TcShape &sh)
     if (p.dtype != REFREE_DTYPE_BF16 || p.head_dim != kD) return false;
     const int G = p.num_q_heads / p.num_kv_heads;
     const int64_t R = (int64_t)G * p.window;
-    // one window row has a path of its own (score_w1.cu); few rows are padded to 32
+    // One window row has a path of its own (score_w1.cu); few rows are padded to 32, at any length: a layer takes the same
+    // form alone and in a run.  (2 to 31 rows, us, here and with the generic kernels: a layer of 200 positions 33 and 37, 2000
+    // 37 and 30, 8192 x 8 heads 58 and 74, 32768 x 8 121 and 246; a run of four of 1000 x 8 54 and 141.)
     if (R > kMaxRowsTc || (R < 32 && p.window == 1)) return false;
     sh.R = (int)R;
     sh.rblocks = (sh.R + kTile - 1) / kTile;

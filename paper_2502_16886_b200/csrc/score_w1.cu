@@ -733,7 +733,8 @@ cudaError_t launch_score_w1(const refree_params &p, const W1Group &g, const int3
     // A cluster per unit while the whole call is short (no unit is longer than the call) and its logits fit the default
     // limit of shared memory.  A layer compacted in place, 8 KV heads, with the two kernels below and this way: sequences of
     // 1000, 333 and 517 positions 21.0 and 15.4 us, one of 200 19.4 and 13.7, of 4096 21.1 and 16.8, of 8192 22.1 and 21.5,
-    // eight of 1000 24.1 and 23.0.
+    // eight of 1000 24.1 and 23.0.  Beyond the line (four layers, us): of 9000 104.0 and 103.9, of 12000 110 and 121, of 16000
+    // 112 and 137.
     const int64_t cluster = std::min<int64_t>(kMaxClusterW1, (total_tokens + 127) / 128);
     if (mma && total_tokens <= kUnitTokens) {
         const int stride = (int)((total_tokens + 32 * cluster - 1) / (32 * cluster) * 32 + 8);   // (+ 8 spreads the heads over the banks)

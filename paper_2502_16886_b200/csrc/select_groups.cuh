@@ -1,6 +1,7 @@
 // Position ranking, one budget per (sequence, KV head), from the per-32-position records (GroupPartial) that a
-// scoring kernel leaves: the arithmetic of the stopping rule shared by the selection kernel (a block per unit)
-// and by the scoring kernel's finishing warp (a warp per unit, for the unit whose last tile it has just scored).
+// scoring kernel leaves: the arithmetic of the stopping rule, evaluated by a block per unit (a launch of its own, the
+// cluster kernel of a single query row, a scoring CTA that has left its passes) or by a warp (a scoring CTA that
+// completed more units than its list holds).
 // Integer sums throughout, so the two agree bit for bit whatever the order of their additions.
 #pragma once
 
