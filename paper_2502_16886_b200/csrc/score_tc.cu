@@ -882,14 +882,18 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
     const float g = (float)(a.p.num_q_heads / a.p.num_kv_heads);
     const int slot_shift = 31 - __clz(a.sh.slots);
     // This CTA's tiles of a unit are counted once, when its run of them ends: the warp that brings the unit's count
-    // to its number of tiles sees every other tile's scores and records (fenced before their counts were added)
-    // and puts the unit on the CTA's list.  The rule itself (some ten dependent loads, scans and shuffles) waits until
-    // the CTA has left its passes and takes all its warps: beside sixteen warps that keep the exponential unit busy
-    // it took one warp 28 us, which ended the launch.
+    // to its number of tiles sees every other tile's scores and records (fenced before their counts were added).
+    // The rule is some ten dependent loads, scans and shuffles, 28 us for one warp beside sixteen that keep the exponential
+    // unit busy.  So the unit goes on the CTA's list, for all its threads when they have left the passes; but the warp
+    // evaluates it itself where it has time for that, beyond 256 query rows (two products a tile, and a long row pass behind)
+    // and with a unit for every fourth CTA at most.  Measured, us a pass, by the list and by the warp: ragged batch of eight
+    // x 4 layers, 448 rows (32 units a launch) 722 and 710, 20K x 8, 512 rows (16) 762 and 758, two layers of 17.5K, 512 rows
+    // (32) 239 and 229; 32K x 8, 256 rows (16) 674 and 674, 32K x 8, 64 rows (8) 219 and 241, 2K x 16, 256 rows (64) 180 and 188.
     int run_u = -1, run_ntiles = 0, run_ib = 0, run_tiles = 0;
     uint32_t run_max = 0;                       // largest score of the run (bit pattern)
     const int Hkv = a.p.num_kv_heads, U1 = a.p.num_seqs * Hkv, U = U1 * a.layers_b;
     const bool two_products = a.sh.cblocks > 1;
+    const int listed = two_products && 4 * U <= (int)gridDim.x ? 0 : kRuleList;
     auto close_run = [&]() {
         if (run_u < 0 || run_tiles == 0) return;
         if (lane == 0) atomicMax(&a.tickets[U + run_u], run_max);      // the unit's largest score, beside its count
@@ -904,7 +908,7 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
             if (lane == 0) umax = atomicMax(&a.tickets[U + run_u], 0u);
             umax = __shfl_sync(0xffffffffu, umax, 0);
             const int k = tl.rule_n;                                       // only this warp appends
-            if (k < kRuleList) {
+            if (k < listed) {
                 __syncwarp();
                 if (lane == 0) { tl.rule_unit[k] = run_u; tl.rule_max[k] = umax; tl.rule_n = k + 1; }
                 __syncwarp();
