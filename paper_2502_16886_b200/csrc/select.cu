@@ -1014,7 +1014,11 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
             while (nblk < kMaxCluster && avg >= (int64_t)nblk * 4096) nblk *= 2;
             // a block takes an SM, and clusters leave some SMs of a group of them unused: stay well within one wave (16
             // units of 32K positions: 61 us in clusters of eight, which came in two waves, 38 in clusters of four)
-            while (nblk > 1 && (int64_t)sel_units * layers * nblk * 4 > (int64_t)sm_count() * 3) nblk /= 2;
+            // (but not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some
+            // 100 us for it: eleven sequences of 69 to 29809 positions, 8 heads, four layers 1428 -> 1015)
+            const bool resident = p.scope == REFREE_SCOPE_HEAD;
+            while (nblk > 1 && (int64_t)sel_units * layers * nblk * 4 > (int64_t)sm_count() * 3 &&
+                   (!resident || (int64_t)(nblk / 2) * kThreads * 16 >= total_tokens)) nblk /= 2;
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(sel_units * nblk, layers);
