@@ -308,8 +308,14 @@ cudaError_t run_rows(const refree_params &p, const void *q_win, const void *k, c
     if (e == cudaSuccess)
         e = launch_dependent(score_combine_generic, dim3((R + 31) / 32, p.num_seqs * p.num_kv_heads), dim3(kThreads), 0, st, p, seq_len,
                              (const float2 *)part, lse);
+    // The blocks of a chained launch land on the SMs that are free at that moment, several to one while others come free later.
+    // That costs more than the launch where they take long and are too few to fill the machine: 36 blocks of 800 rows 111 to
+    // 168 us against 78 (a run of eight layers of 1078 positions 1195 -> 903), 79 of 400 rows (four layers of 5000 positions)
+    // 319 -> 257; with 8 blocks there is room for each (500 positions 182, not chained 210).
+    const unsigned sms = (unsigned)sm_count();
+    const bool spread = R > 256 && items >= sms / 8 && items < 2 * sms;
     if (e == cudaSuccess)
-        e = launch_dependent(score_colsum_generic<T, D, RA>, dim3(items), dim3(kThreads), kSmem, st, p, (const T *)q_win, (const T *)k,
+        e = launch_dependent(score_colsum_generic<T, D, RA>, dim3(items), dim3(kThreads), kSmem, Stream(st.s, st.chain && !spread), p, (const T *)q_win, (const T *)k,
                              seq_start, seq_len, (const float *)lse, total_tokens, scores, dev_status, q_vec);
     if (e != cudaSuccess) return e;
     count_launches(3);
