@@ -335,11 +335,13 @@ cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const 
 {
     const int U = p.num_seqs * p.num_kv_heads;
     const int ranges = position_ranges ? 1 : 0;
-    // Two waves of blocks; four times as many where a large copy takes several layers, so that a long unit among short ones
-    // is not left to one or two blocks (seven layers of twelve sequences of 83 to 15815 positions, 8 heads: 928 us and 527;
-    // small copies would pay for the blocks: 18 and 25 us).
+    // Two waves of blocks; four times as many for a large copy of several layers, or of three sequences and more, so that a
+    // long unit among short ones is not left to one or two blocks (us: seven layers of twelve sequences of 83 to 15815
+    // positions, 8 heads, 928 and 527; one layer of thirteen of 77 to 26835, 16 heads, 565 and 444 with its scoring; four
+    // of eleven, ranked by score, 1089 and 1015; small copies would pay for the blocks, 18 and 25, and so would units of one
+    // length, two of 16000 positions ranked by score 244 and 255).
     const Stream cs = copy_stream(p, st, job.layers);
-    const int per_sm = job.layers > 1 && !cs.chain ? 32 : 8;
+    const int per_sm = !cs.chain && (job.layers > 1 || p.num_seqs > 2) ? 32 : 8;
     const int gx = max(1, (sm_count() * per_sm) / (U * job.layers));
     const cudaError_t e = launch_dependent(compact_kernel, dim3(gx, U, job.layers), dim3(kThreads), 0,
                                            cs, p, job, seq_start, seq_len, ranges, capacity_rows, dev_status);
