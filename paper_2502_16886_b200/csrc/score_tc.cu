@@ -933,76 +933,51 @@ __device__ inline void finisher_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
         float *dst = a.scores + (int64_t)inf->g * a.total_tokens + inf->pack;
         GroupPartial *grp = a.groups ? a.groups + ((int64_t)inf->ib + tile) * 4 : nullptr;
         uint32_t tile_max = 0;
-        if ((reinterpret_cast<uintptr_t>(dst + (int64_t)tile * kTile) & 15) == 0) {
-            // A lane takes four consecutive positions: the shares come as 16-byte loads, the scores leave as one
-            // 16-byte store, and the 32 positions of a record are eight neighbouring lanes.  (Few instructions that
-            // go through the memory pipe: the sixteen epilogue warps keep it busy, and this warp paces the pass.)
-            const int p0 = 4 * lane, i0 = tile * kTile + p0;
-            float tot[4];
-            {
-                const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[0][p0]);
-                const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[1][p0]);
-                tot[0] = x.x + y.x; tot[1] = x.y + y.y; tot[2] = x.z + y.z; tot[3] = x.w + y.w;
-            }
-            if (two_products) {
-                const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[2][p0]);
-                const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[3][p0]);
-                tot[0] += x.x; tot[1] += x.y; tot[2] += x.z; tot[3] += x.w;
-                tot[0] += y.x; tot[1] += y.y; tot[2] += y.z; tot[3] += y.w;
-            }
-            float sc[4];
-            uint32_t bits[4];
+        // A lane takes four consecutive positions: the shares come as 16-byte loads, the scores leave as one 16-byte store
+        // where their row starts on 16 bytes, and the 32 positions of a record are eight neighbouring lanes.  (Few
+        // instructions that go through the memory pipe: the sixteen epilogue warps keep it busy, and this warp paces the pass.)
+        const int p0 = 4 * lane, i0 = tile * kTile + p0;
+        float tot[4];
+        {
+            const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[0][p0]);
+            const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[1][p0]);
+            tot[0] = x.x + y.x; tot[1] = x.y + y.y; tot[2] = x.z + y.z; tot[3] = x.w + y.w;
+        }
+        if (two_products) {
+            const float4 x = *reinterpret_cast<const float4 *>(&stage[slot].sum[2][p0]);
+            const float4 y = *reinterpret_cast<const float4 *>(&stage[slot].sum[3][p0]);
+            tot[0] += x.x; tot[1] += x.y; tot[2] += x.z; tot[3] += x.w;
+            tot[0] += y.x; tot[1] += y.y; tot[2] += y.z; tot[3] += y.w;
+        }
+        float sc[4];
+        uint32_t bits[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = i0 + k;
-                const int cnt_i = max(1, min(min(w, n), n - i));
-                sc[k] = i < n ? tot[k] / ((float)cnt_i * g) : 0.f;
-                bits[k] = (i < n && isfinite(sc[k])) ? mag_bits(sc[k]) : 0u;
-                if (i < n && !isfinite(sc[k]) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
-            }
-            if (i0 + 3 < n) {
-                *reinterpret_cast<float4 *>(dst + i0) = make_float4(sc[0], sc[1], sc[2], sc[3]);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (i0 + k < n) dst[i0 + k] = sc[k];
-            }
-            if (grp) {
-                // 32 positions = lanes 8q .. 8q + 7: largest score, and the exact squares summed at a scale set by it
-                uint32_t mx = max(max(bits[0], bits[1]), max(bits[2], bits[3]));
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                const int shift = kGroupShift - 2 * max(1, (int)(mx >> 23));
-                unsigned long long sq = sq_fixed(bits[0], shift) + sq_fixed(bits[1], shift) + sq_fixed(bits[2], shift) +
-                                        sq_fixed(bits[3], shift);
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-                if ((lane & 7) == 0) { GroupPartial gp; gp.max_bits = mx; gp.pad = 0u; gp.sum = sq; grp[lane >> 3] = gp; }
-                tile_max = __reduce_max_sync(0xffffffffu, mx);
-            }
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k;
+            const int cnt_i = max(1, min(min(w, n), n - i));
+            sc[k] = i < n ? tot[k] / ((float)cnt_i * g) : 0.f;
+            bits[k] = (i < n && isfinite(sc[k])) ? mag_bits(sc[k]) : 0u;
+            if (i < n && !isfinite(sc[k]) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
+        }
+        if (i0 + 3 < n && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+            *reinterpret_cast<float4 *>(dst + i0) = make_float4(sc[0], sc[1], sc[2], sc[3]);
         } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int pos = q * 32 + lane, i = tile * kTile + pos;
-            float tot = stage[slot].sum[0][pos] + stage[slot].sum[1][pos];
-            if (two_products) { tot += stage[slot].sum[2][pos]; tot += stage[slot].sum[3][pos]; }
-            const int cnt_i = max(1, min(min(w, n), n - i));
-            float sc = 0.f;
-            if (i < n) {
-                sc = tot / ((float)cnt_i * g);
-                if (!isfinite(sc) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
-                dst[i] = sc;
-            }
-            if (grp) {
-                // these 32 positions: largest score, and the exact squares summed at a scale set by it
-                const uint32_t bits = (i < n && isfinite(sc)) ? mag_bits(sc) : 0u;
-                const uint32_t mx = __reduce_max_sync(0xffffffffu, bits);
-                tile_max = max(tile_max, mx);
-                unsigned long long sq = sq_fixed(bits, kGroupShift - 2 * max(1, (int)(mx >> 23)));
-                for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-                if (lane == 0) { GroupPartial gp; gp.max_bits = mx; gp.pad = 0u; gp.sum = sq; grp[q] = gp; }
-            }
+            for (int k = 0; k < 4; ++k)
+                if (i0 + k < n) dst[i0 + k] = sc[k];
         }
+        if (grp) {
+            // 32 positions = lanes 8q .. 8q + 7: largest score, and the exact squares summed at a scale set by it
+            uint32_t mx = max(max(bits[0], bits[1]), max(bits[2], bits[3]));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const int shift = kGroupShift - 2 * max(1, (int)(mx >> 23));
+            unsigned long long sq = sq_fixed(bits[0], shift) + sq_fixed(bits[1], shift) + sq_fixed(bits[2], shift) +
+                                    sq_fixed(bits[3], shift);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if ((lane & 7) == 0) { GroupPartial gp; gp.max_bits = mx; gp.pad = 0u; gp.sum = sq; grp[lane >> 3] = gp; }
+            tile_max = __reduce_max_sync(0xffffffffu, mx);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&tl.stage_free[slot]);
