@@ -177,12 +177,12 @@ def algorithmic_bytes(cfg, seq_lens, lengths):
     return a, b4
 
 
-# dram__bytes_read + dram__bytes_write of one launch of the dominant kernel, from the ncu capture summarised under
-# profiles/.  The figure belongs to one version of the kernel source: it is reported only while the source file
-# still has the hash it was captured on, and null afterwards.
+# dram__bytes_read + dram__bytes_write of a layer's share of a launch of the dominant kernel (a launch takes a group of
+# layers), from the ncu capture summarised under profiles/.  The figure belongs to one version of the kernel source: it is
+# reported only while the source file still has the hash it was captured on, and null afterwards.
 NCU_TRAFFIC = {
-    # workload: (kernel source, first 16 hex digits of its sha256, bytes per launch)
-    "mistral7b_32k": ("paper_2502_16886_b200/csrc/score_tc.cu", "848012eefce12c48", 262_343_936 + 92_841_216),
+    # workload: (kernel source, first 16 hex digits of its sha256, bytes per layer)
+    "mistral7b_32k": ("paper_2502_16886_b200/csrc/score_tc.cu", "d2384a5e37f73516", (528_448_000 + 238_242_816) // 2),
 }
 
 
