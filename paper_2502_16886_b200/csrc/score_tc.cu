@@ -98,6 +98,11 @@ __device__ inline bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *a
     *abort_flag = 1;
     return false;
 }
+// The same for a whole warp, which goes on or gives up as one.
+__device__ inline bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
 __device__ inline void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ inline void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ inline void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -128,6 +133,13 @@ __device__ inline void tmem_alloc(uint32_t *dst_smem, uint32_t cols)
 __device__ inline void tmem_dealloc(uint32_t taddr, uint32_t cols)
 {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+}
+// One lane of a converged warp, the same one every time.
+__device__ inline bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
 }
 // D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate; issued by one thread.
 // The two shared-memory descriptors are passed as their low words (start address
@@ -454,26 +466,33 @@ __device__ inline void producer_loop(const TcArgs &a, const TcMaps &maps,
             const bool last = j + 1 == run;
             // the ring entry was last used sixteen items ago, which every consumer has long left behind
             ItemInfo &inf = tl.info[rs.icount++ & (kInfoRing - 1)];
-            inf.u = u; inf.g = layer * Hkv + g; inf.n = it.n; inf.tile = tile; inf.ntiles = it.ntiles; inf.pack = it.pack;
-            inf.ib = ib;
-            inf.flags = (j == 0 && new_unit ? kNewUnit : 0) | (last ? kRunLast : 0) | (last && last_run ? kPassLast : 0);
+            const int flags = (j == 0 && new_unit ? kNewUnit : 0) | (last ? kRunLast : 0) | (last && last_run ? kPassLast : 0);
             // The K tile first: the MMA thread learns of a unit change from the record, which it reads once
             // the tile has landed, and only then gives the Q image back.
-            ok = mbar_wait(&tl.k_empty[rs.stage], rs.kphase ^ 1, &tl.abort_flag);
+            ok = mbar_wait_warp(&tl.k_empty[rs.stage], rs.kphase ^ 1, &tl.abort_flag);
             if (!ok) break;
-            mbar_expect_tx(&tl.k_full[rs.stage], (uint32_t)kTileBytes);      // (release) orders the record before the tile
-            unsigned char *dst = smem_k + (size_t)rs.stage * kTileBytes;
-            load(dst, 0, tile);
-            load(dst + kHalfBytes, 1, tile);
+            if (elect_one()) {
+                inf.u = u; inf.g = layer * Hkv + g; inf.n = it.n; inf.tile = tile; inf.ntiles = it.ntiles; inf.pack = it.pack;
+                inf.ib = ib;
+                inf.flags = flags;
+                mbar_expect_tx(&tl.k_full[rs.stage], (uint32_t)kTileBytes);      // (release) orders the record before the tile
+                unsigned char *dst = smem_k + (size_t)rs.stage * kTileBytes;
+                load(dst, 0, tile);
+                load(dst + kHalfBytes, 1, tile);
+            }
+            __syncwarp();
             if (new_unit && j == 0) {
-                ok = mbar_wait(&tl.q_empty, rs.qphase ^ 1, &tl.abort_flag);
+                ok = mbar_wait_warp(&tl.q_empty, rs.qphase ^ 1, &tl.abort_flag);
                 if (!ok) break;
-                mbar_expect_tx(&tl.q_full, (uint32_t)sh.Rpad * 256u);
-                const int row0 = (it.s * a.p.num_q_heads + g * G) * a.p.window;
-                for (int h = 0; h < 2; ++h)
-                    for (int b = 0; b < sh.rblocks; ++b)
-                        tma_load_2d(smem_q + (size_t)h * sh.Rpad * 128 + (size_t)b * kHalfBytes, mapq, &tl.q_full,
-                                    h * 64, row0 + b * kTile);
+                if (elect_one()) {
+                    mbar_expect_tx(&tl.q_full, (uint32_t)sh.Rpad * 256u);
+                    const int row0 = (it.s * a.p.num_q_heads + g * G) * a.p.window;
+                    for (int h = 0; h < 2; ++h)
+                        for (int b = 0; b < sh.rblocks; ++b)
+                            tma_load_2d(smem_q + (size_t)h * sh.Rpad * 128 + (size_t)b * kHalfBytes, mapq, &tl.q_full,
+                                        h * 64, row0 + b * kTile);
+                }
+                __syncwarp();
                 rs.qphase ^= 1;
             }
             if (++rs.stage == sh.stages) { rs.stage = 0; rs.kphase ^= 1; }
@@ -494,9 +513,9 @@ __device__ inline void producer_loop(const TcArgs &a, const TcMaps &maps,
 // A unit begins: its Q must have landed (and the one before is given back with the products issued so far).
 __device__ inline bool mma_new_unit(TcSmemTail &tl, MmaState &ms)
 {
-    if (!ms.first) umma_commit(&tl.q_empty);
+    if (!ms.first && elect_one()) umma_commit(&tl.q_empty);
     ms.first = false;
-    if (!mbar_wait(&tl.q_full, ms.qphase, &tl.abort_flag)) return false;
+    if (!mbar_wait_warp(&tl.q_full, ms.qphase, &tl.abort_flag)) return false;
     ms.qphase ^= 1;
     tc_fence_after();
     return true;
@@ -514,7 +533,7 @@ __device__ inline void mma_loop_pass1(const TcArgs &a, unsigned char *smem_q, un
     const uint32_t idesc = make_idesc(kTile);
     uint32_t cnt0 = 0, cnt1 = 0;                                 // products per pair
     for (;;) {
-        if (!mbar_wait(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
+        if (!mbar_wait_warp(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
         tc_fence_after();
         const int flags = tl.info[ms.icount++ & (kInfoRing - 1)].flags;
         if ((flags & kNewUnit) && !mma_new_unit(tl, ms)) return;
@@ -523,19 +542,22 @@ __device__ inline void mma_loop_pass1(const TcArgs &a, unsigned char *smem_q, un
             const uint32_t pair = (uint32_t)(rb & 1), cnt = pair ? cnt1 : cnt0, acc = 2u * pair + (cnt & 1u);
             // a pair covers the columns of an accumulator of pass 2: the last product left there must have been handed back
             const uint32_t before = (ms.p2 + 1u - pair) >> 1;
-            if (cnt == 0 && before > 0 && !mbar_wait(&tl.p2_empty[pair], (before - 1u) & 1u, &tl.abort_flag)) return;
-            if (!mbar_wait(&tl.p1_empty[acc], ((cnt >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
+            if (cnt == 0 && before > 0 && !mbar_wait_warp(&tl.p2_empty[pair], (before - 1u) & 1u, &tl.abort_flag)) return;
+            if (!mbar_wait_warp(&tl.p1_empty[acc], ((cnt >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
             tc_fence_after();
             const uint32_t qa = q_lo + (uint32_t)rb * (kHalfBytes >> 4);
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const uint32_t h = kk >> 2, ko = (kk & 3) * 2;          // 32 bytes per K step of 16
-                umma_bf16(tmem_base + acc * 128u, qa + h * q_half + ko, kt + h * (kHalfBytes >> 4) + ko, kDescHi, idesc, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {
+                    const uint32_t h = kk >> 2, ko = (kk & 3) * 2;      // 32 bytes per K step of 16
+                    umma_bf16(tmem_base + acc * 128u, qa + h * q_half + ko, kt + h * (kHalfBytes >> 4) + ko, kDescHi, idesc, kk > 0);
+                }
+                umma_commit(&tl.p1_full[acc]);
+                if (rb + 1 == sh.rblocks) umma_commit(&tl.k_empty[ms.stage]);
             }
-            umma_commit(&tl.p1_full[acc]);
+            __syncwarp();
             if (pair) ++cnt1; else ++cnt0;
         }
-        umma_commit(&tl.k_empty[ms.stage]);
         if (++ms.stage == sh.stages) { ms.stage = 0; ms.kphase ^= 1; }
         if (flags & kPassLast) break;
     }
@@ -551,29 +573,35 @@ __device__ inline void mma_loop_pass2(const TcArgs &a, unsigned char *smem_q, un
     const uint32_t q_half = (uint32_t)(sh.Rpad * 128) >> 4;
     const uint32_t idesc = make_idesc(sh.ncol);
     for (;;) {
-        if (!mbar_wait(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
+        if (!mbar_wait_warp(&tl.k_full[ms.stage], ms.kphase, &tl.abort_flag)) return;
         tc_fence_after();
         const int flags = tl.info[ms.icount++ & (kInfoRing - 1)].flags;
         if ((flags & kNewUnit) && !mma_new_unit(tl, ms)) return;
         const uint32_t ka = k_lo + (uint32_t)ms.stage * (kTileBytes >> 4);
         for (int cb = 0; cb < sh.cblocks; ++cb) {
             const uint32_t buf = ms.p2 & 1u;
-            if (!mbar_wait(&tl.p2_empty[buf], ((ms.p2 >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
+            if (!mbar_wait_warp(&tl.p2_empty[buf], ((ms.p2 >> 1) & 1u) ^ 1u, &tl.abort_flag)) return;
             tc_fence_after();
             const uint32_t qb = q_lo + (uint32_t)cb * (uint32_t)(sh.ncol * 128 >> 4);
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const uint32_t h = kk >> 2, ko = (kk & 3) * 2;
-                umma_bf16(tmem_base + buf * 256u, ka + h * (kHalfBytes >> 4) + ko, qb + h * q_half + ko, kDescHi, idesc, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {
+                    const uint32_t h = kk >> 2, ko = (kk & 3) * 2;
+                    umma_bf16(tmem_base + buf * 256u, ka + h * (kHalfBytes >> 4) + ko, qb + h * q_half + ko, kDescHi, idesc, kk > 0);
+                }
+                umma_commit(&tl.p2_full[buf]);
+                if (cb + 1 == sh.cblocks) umma_commit(&tl.k_empty[ms.stage]);
             }
-            umma_commit(&tl.p2_full[buf]);
+            __syncwarp();
             ++ms.p2;
         }
-        umma_commit(&tl.k_empty[ms.stage]);
         if (++ms.stage == sh.stages) { ms.stage = 0; ms.kphase ^= 1; }
         if (flags & kPassLast) break;
     }
-    if (more) { umma_commit(&tl.q_empty); ms.first = true; }
+    if (more) {
+        if (elect_one()) umma_commit(&tl.q_empty);
+        ms.first = true;
+    }
 }
 
 // ------------------------------------------------------------- epilogues -----
@@ -1232,17 +1260,18 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
         if (P2) epilogue_pass2(a, tl, stage, sv, tmem_base, b0, nb, sp, es);
         if (P1 && na > 0 && !tl.abort_flag) epilogue_pass1(a, tl, tmem_base, es);
     } else if (warp == kEpiWarps) {
-        if (lane == 0) {
-            RingState rs;
-            if (P2) producer_loop<false>(a, maps_b, smem_q, smem_k, tl, sv, sp, sh_b, rs);
-            if (P1) producer_loop<true>(a, maps_a, smem_q, smem_k, tl, sv, sp, sh_a, rs);
-        }
+        RingState rs;
+        if (P2) producer_loop<false>(a, maps_b, smem_q, smem_k, tl, sv, sp, sh_b, rs);
+        if (P1) producer_loop<true>(a, maps_a, smem_q, smem_k, tl, sv, sp, sh_a, rs);
     } else if (warp == kEpiWarps + 1) {
-        if (lane == 0) {
-            MmaState ms;
-            if (P2 && nb > 0) mma_loop_pass2(a, smem_q, smem_k, tl, tmem_base, ms, P1);
-            if (P1 && na > 0 && !tl.abort_flag) mma_loop_pass1(a, smem_q, smem_k, tl, tmem_base, ms);
-        }
+        // All lanes of this warp and of the TMA warp walk their loops and one elected lane issues.  With a single lane in them the
+        // operands of every instruction went through the registers of a diverged warp, and products came at half the tensor
+        // cores' rate (N = 128: 116 cycles, 72 this way; us a run: 16 layers of 8K positions 428 -> 387, 32K x 8 688 -> 663,
+        // the ragged batch of eight x 4 697 -> 657, 20K x 8, 512 rows, 756 -> 731).
+        MmaState ms;
+        if (P2 && nb > 0) mma_loop_pass2(a, smem_q, smem_k, tl, tmem_base, ms, P1);
+        __syncwarp();
+        if (P1 && na > 0 && !tl.abort_flag) mma_loop_pass1(a, smem_q, smem_k, tl, tmem_base, ms);
     } else if (warp == kEpiWarps + 2) {
         if (a.cj.nslots > 0) copy_loop(a, tl, sv, smem_c, coff);
     } else {
