@@ -130,6 +130,7 @@ template <> struct Row16<float> {
 // The layers of a group, one to a grid row; what a layer keeps follows that of the layer before.
 struct W1Args {
     refree_params p;
+    int layers;
     const void *q_win[kMaxBatch], *k[kMaxBatch];
     int64_t layer_logits, layer_stats, layer_groups;        // elements per layer (scores: Hkv total_tokens)
     const int32_t *seq_start, *seq_len;
@@ -268,18 +269,17 @@ __device__ inline uint4 ld_row16(const char *p)
 // is the query of head r (and r + 8 for the second column tile) cut the same way, so every product
 // pairs the same element of k_i and q_h whatever slot of the k-step it occupies.  The accumulator
 // of lane (r, c) holds heads 2c, 2c + 1 for rows r and r + 8.  NT column tiles cover G <= 8 NT heads.
+// Bound by the stream over K.  The warps of one wave of blocks walk the spans of all layers of the group, and a warp asks for
+// the next 16 rows (of its next span too) before it works on those it has: a block per layer and piece of the grid, with the
+// rows of a step loaded and used in turn, kept HBM at 4.8 TB/s (eight layers of 32K positions x 8 heads, 107 us).
 template <int D, int NT>
-__global__ void __launch_bounds__(kThreadsW1)
+__global__ void __launch_bounds__(kThreadsW1, 2)
 w1_logits_mma_kernel(const __grid_constant__ W1Args a)
 {
     constexpr int CH = D / 32;                       // 16-byte pieces per lane and row
     constexpr int kWarpsW1 = kThreadsW1 / 32;
     __shared__ W1Tables tb;
     const refree_params &p = a.p;
-    const int layer = blockIdx.y;
-    const __nv_bfloat16 *const q_win = static_cast<const __nv_bfloat16 *>(a.q_win[layer]), *const k = static_cast<const __nv_bfloat16 *>(a.k[layer]);
-    float *const logits = a.logits + layer * a.layer_logits;
-    float2 *const stats = a.stats + layer * a.layer_stats;
     const int B = p.num_seqs, Hkv = p.num_kv_heads, G = p.num_q_heads / Hkv;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = lane >> 2, c = lane & 3;
@@ -287,19 +287,48 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
     dependency_wait();
     trigger_dependents();
     build_w1_tables(tb, a.seq_len, B, a.span);
-    const int items = tb.spans[B] * Hkv;
+    const int per_layer = tb.spans[B] * Hkv;
+    const int64_t items = (int64_t)per_layer * a.layers, step = (int64_t)gridDim.x * kWarpsW1;
     const int64_t tok_bytes = p.k_stride_tok * (int64_t)sizeof(__nv_bfloat16);
+    // a span of a layer: what it reads
+    struct Span { W1Item it; int layer, end; const char *base; };
+    auto span_of = [&](int64_t item) {
+        Span sp;
+        sp.layer = (int)(item / per_layer);
+        sp.it = decode_w1(tb, tb.spans, a.span, B, Hkv, (int)(item - (int64_t)sp.layer * per_layer));
+        sp.end = min(sp.it.n, sp.it.pos0 + a.span);
+        sp.base = static_cast<const char *>(a.k[sp.layer]) +
+                  ((int64_t)sp.it.s * p.k_stride_seq + (int64_t)a.seq_start[sp.it.s] * p.k_stride_tok + (int64_t)sp.it.g * p.k_stride_head) * 2;
+        return sp;
+    };
+    uint4 ka[CH], kb[CH];
+    auto load = [&](const Span &sp, int row0) {      // rows row0 + r and row0 + 8 + r; missing ones are zero
+        const int i0 = row0 + r, i1 = i0 + 8;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+            const int off = j * 64 + c * 16;
+            ka[j] = i0 < sp.end ? ld_row16(sp.base + (int64_t)i0 * tok_bytes + off) : make_uint4(0u, 0u, 0u, 0u);
+            kb[j] = i1 < sp.end ? ld_row16(sp.base + (int64_t)i1 * tok_bytes + off) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    int64_t item = (int64_t)blockIdx.x * kWarpsW1 + warp;
+    if (item >= items) return;
+    Span sp = span_of(item);
+    load(sp, sp.it.pos0);
     int cur_u = -1;
     uint4 qf[NT][CH];
-    for (int item = blockIdx.x * kWarpsW1 + warp; item < items; item += gridDim.x * kWarpsW1) {
-        const W1Item it = decode_w1(tb, tb.spans, a.span, B, Hkv, item);
-        const int u = it.s * Hkv + it.g;
+    for (;;) {
+        const W1Item it = sp.it;
+        const int layer = sp.layer, end = sp.end;
+        float *const logits = a.logits + layer * a.layer_logits;
+        float2 *const stats = a.stats + layer * a.layer_stats;
+        const int u = (layer * B + it.s) * Hkv + it.g;
         if (u != cur_u) {
+            const char *const q_win = static_cast<const char *>(a.q_win[layer]);
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
                 const int head = t * 8 + r;
-                const char *qrow = reinterpret_cast<const char *>(
-                    q_win + ((int64_t)it.s * p.num_q_heads + it.g * G + min(head, G - 1)) * D);
+                const char *qrow = q_win + ((int64_t)it.s * p.num_q_heads + it.g * G + min(head, G - 1)) * D * 2;
 #pragma unroll
                 for (int j = 0; j < CH; ++j) {
                     qf[t][j] = *reinterpret_cast<const uint4 *>(qrow + j * 64 + c * 16);
@@ -308,32 +337,32 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
             }
             cur_u = u;
         }
-        const char *base = reinterpret_cast<const char *>(
-            k + (int64_t)it.s * p.k_stride_seq + (int64_t)a.seq_start[it.s] * p.k_stride_tok + (int64_t)it.g * p.k_stride_head);
         float *unit_logits = logits + (int64_t)(it.g * G) * a.total_tokens + tb.pack[it.s];
-        const int end = min(it.n, it.pos0 + a.span);
+        item += step;
+        const bool more = item < items;
+        if (more) sp = span_of(item);                // the next span: its first rows are asked for under this one's last
         float m[NT][2], z[NT][2];
 #pragma unroll
         for (int t = 0; t < NT; ++t) { m[t][0] = m[t][1] = -INFINITY; z[t][0] = z[t][1] = 0.f; }
-#pragma unroll 2
+        const char *const base = static_cast<const char *>(a.k[layer]) +
+                                 ((int64_t)it.s * p.k_stride_seq + (int64_t)a.seq_start[it.s] * p.k_stride_tok + (int64_t)it.g * p.k_stride_head) * 2;
+        const Span cur = {it, layer, end, base};
         for (int row0 = it.pos0; row0 < end; row0 += 16) {
             const int i0 = row0 + r, i1 = i0 + 8;
             const bool v0 = i0 < end, v1 = i1 < end;
-            uint4 ka[CH], kb[CH];
+            uint4 xa[CH], xb[CH];
 #pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const int off = j * 64 + c * 16;
-                ka[j] = v0 ? ld_row16(base + (int64_t)i0 * tok_bytes + off) : make_uint4(0u, 0u, 0u, 0u);
-                kb[j] = v1 ? ld_row16(base + (int64_t)i1 * tok_bytes + off) : make_uint4(0u, 0u, 0u, 0u);
-            }
+            for (int j = 0; j < CH; ++j) { xa[j] = ka[j]; xb[j] = kb[j]; }
+            if (row0 + 16 < end) load(cur, row0 + 16);
+            else if (more) load(sp, sp.it.pos0);
             float acc[NT][4];
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
                 acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
 #pragma unroll
                 for (int j = 0; j < CH; ++j) {
-                    mma_bf16_16x8x16(acc[t], ka[j].x, kb[j].x, ka[j].y, kb[j].y, qf[t][j].x, qf[t][j].y);
-                    mma_bf16_16x8x16(acc[t], ka[j].z, kb[j].z, ka[j].w, kb[j].w, qf[t][j].z, qf[t][j].w);
+                    mma_bf16_16x8x16(acc[t], xa[j].x, xb[j].x, xa[j].y, xb[j].y, qf[t][j].x, qf[t][j].y);
+                    mma_bf16_16x8x16(acc[t], xa[j].z, xb[j].z, xa[j].w, xb[j].w, qf[t][j].z, qf[t][j].w);
                 }
             }
 #pragma unroll
@@ -371,6 +400,7 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
                     stats[((int64_t)tb.spans[it.s] * Hkv + (int64_t)it.g * (tb.spans[it.s + 1] - tb.spans[it.s]) +
                              it.chunk) * G + head] = make_float2(m[t][e], z[t][e]);
             }
+        if (!more) break;
     }
 }
 
@@ -556,7 +586,7 @@ w1_unit_kernel(const __grid_constant__ W1Args a, int stride)
 }
 
 template <int GMAX>
-__global__ void __launch_bounds__(kThreadsW1, GMAX <= 4 ? 5 : GMAX <= 8 ? 4 : 2)     // (fewer blocks an SM: 1.5 us of 22 more)
+__global__ void __launch_bounds__(kThreadsW1, GMAX <= 8 ? 4 : 2)
 w1_scores_kernel(const __grid_constant__ W1Args a)
 {
     constexpr int kWarpsW1 = kThreadsW1 / 32;
@@ -579,7 +609,7 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
     const int per = ceil_div(items, (int)gridDim.x);
     const int first = blockIdx.x * per, last = min(items, first + per);
     int cur_u = -1;
-    for (int item = first; item < last; ++item) {
+    for (int item = first; item < last;) {
         const W1Item it = decode_w1(tb, tb.chunks, kChunk, B, Hkv, item);
         const int u = it.s * Hkv + it.g;
         if (u != cur_u) {
@@ -613,28 +643,50 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
             cur_u = u;
             __syncthreads();
         }
-        const int i = it.pos0 + threadIdx.x;
-        const bool valid = i < it.n;
-        float sc = 0.f;
-        if (valid) {
-            float tot = 0.f;
-            for (int h = 0; h < G; ++h)
-                tot += ex2(logits[(int64_t)(it.g * G + h) * a.total_tokens + tb.pack[it.s] + i] - lse[h]);
-            sc = tot / (float)G;
-            if (!isfinite(sc) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
-            scores[(int64_t)it.g * a.total_tokens + tb.pack[it.s] + i] = sc;
-        }
-        if (groups) {                         // exact sum of squares of this warp's 32 positions
-            const uint32_t bits = (valid && isfinite(sc)) ? mag_bits(sc) : 0u;
-            const uint32_t mx = __reduce_max_sync(0xffffffffu, bits);
-            unsigned long long sq = sq_fixed(bits, kGroupShift - 2 * max(1, (int)(mx >> 23)));
-            for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            const int grp = (it.pos0 >> 5) + warp;
-            if (lane == 0 && grp * 32 < ceil_div(it.n, kTile) * kTile) {
-                GroupPartial gp; gp.max_bits = mx; gp.pad = 0u; gp.sum = sq;
-                groups[((int64_t)tb.tiles[it.s] * Hkv + (int64_t)it.g * ceil_div(it.n, kTile)) * 4 + grp] = gp;
+        // the run of this block's chunks inside the unit, kAhead of them at a time: their logits are in flight together
+        constexpr int kAhead = GMAX <= 4 ? 4 : 2;
+        const int run = min(last - item, ceil_div(it.n, kChunk) - it.chunk);
+        const float *const y = logits + (int64_t)(it.g * G) * a.total_tokens + tb.pack[it.s];
+        float *const dst = scores + (int64_t)it.g * a.total_tokens + tb.pack[it.s];
+        GroupPartial *const grp = groups ? groups + ((int64_t)tb.tiles[it.s] * Hkv + (int64_t)it.g * ceil_div(it.n, kTile)) * 4 : nullptr;
+        for (int j0 = 0; j0 < run; j0 += kAhead) {
+            float yl[kAhead][GMAX];
+#pragma unroll
+            for (int j = 0; j < kAhead; ++j) {
+                const int i = it.pos0 + (j0 + j) * kChunk + threadIdx.x;
+#pragma unroll
+                for (int h = 0; h < GMAX; ++h)
+                    if (h < G) yl[j][h] = j0 + j < run && i < it.n ? y[(int64_t)h * a.total_tokens + i] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < kAhead; ++j) {
+                if (j0 + j >= run) continue;
+                const int pos0 = it.pos0 + (j0 + j) * kChunk, i = pos0 + threadIdx.x;
+                const bool valid = i < it.n;
+                float sc = 0.f;
+                if (valid) {
+                    float tot = 0.f;
+#pragma unroll
+                    for (int h = 0; h < GMAX; ++h)
+                        if (h < G) tot += ex2(yl[j][h] - lse[h]);
+                    sc = tot / (float)G;
+                    if (!isfinite(sc) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
+                    dst[i] = sc;
+                }
+                if (grp) {                            // exact sum of squares of this warp's 32 positions
+                    const uint32_t bits = (valid && isfinite(sc)) ? mag_bits(sc) : 0u;
+                    const uint32_t mx = __reduce_max_sync(0xffffffffu, bits);
+                    unsigned long long sq = sq_fixed(bits, kGroupShift - 2 * max(1, (int)(mx >> 23)));
+                    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                    const int q = (pos0 >> 5) + warp;
+                    if (lane == 0 && q * 32 < ceil_div(it.n, kTile) * kTile) {
+                        GroupPartial gp; gp.max_bits = mx; gp.pad = 0u; gp.sum = sq;
+                        grp[q] = gp;
+                    }
+                }
             }
         }
+        item += run;
     }
 }
 
@@ -642,7 +694,8 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
 template <int GMAX>
 cudaError_t run_w1_scores(W1Args &a, int layers, int64_t chunk_items, Stream st)
 {
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * 4));
+    // one wave of blocks over all layers: a block reads the unit's records (some 300 per head) before its first chunk
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * 4 / layers));
     const cudaError_t e = launch_dependent(w1_scores_kernel<GMAX>, dim3(grid, layers), dim3(kThreadsW1), 0, st, a);
     count_launches(1);
     return e;
@@ -665,10 +718,10 @@ cudaError_t run_w1_lanes(W1Args &a, int layers, int grid, Stream st, int G)
 }
 
 template <int D>
-cudaError_t run_w1_mma(W1Args &a, int layers, int grid, Stream st, int G)
+cudaError_t run_w1_mma(W1Args &a, int grid, Stream st, int G)
 {
     auto *kern = G <= 8 ? w1_logits_mma_kernel<D, 1> : w1_logits_mma_kernel<D, 2>;
-    const cudaError_t e = launch_dependent(kern, dim3(grid, layers), dim3(kThreadsW1), 0, st, a);
+    const cudaError_t e = launch_dependent(kern, dim3(grid), dim3(kThreadsW1), 0, st, a);
     count_launches(1);
     return e;
 }
@@ -703,6 +756,7 @@ cudaError_t launch_score_w1(const refree_params &p, const W1Group &g, const int3
     const int layers = g.layers;
     W1Args a = {};
     a.p = p;
+    a.layers = layers;
     bool aligned = true;
     for (int l = 0; l < layers; ++l) {
         a.q_win[l] = g.q_win[l];
@@ -752,9 +806,9 @@ cudaError_t launch_score_w1(const refree_params &p, const W1Group &g, const int3
         int64_t span = (rows + warps - 1) / warps;
         span = std::min<int64_t>(kMaxSpan, std::max<int64_t>(kMinSpan, (span + 15) / 16 * 16));
         a.span = (int)span;
-        const int64_t span_items = (total_tokens / span + p.num_seqs) * p.num_kv_heads;
+        const int64_t span_items = (total_tokens / span + p.num_seqs) * p.num_kv_heads * layers;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((span_items + 7) / 8, sm_count() * 2));
-        e = p.head_dim == 64 ? run_w1_mma<64>(a, layers, grid, st, G) : run_w1_mma<128>(a, layers, grid, st, G);
+        e = p.head_dim == 64 ? run_w1_mma<64>(a, grid, st, G) : run_w1_mma<128>(a, grid, st, G);
     } else {
         a.span = kChunk;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * 8));
