@@ -39,6 +39,11 @@ namespace cg = cooperative_groups;
 constexpr int kThreads = 1024;
 constexpr int kMaxCluster = 8;     // blocks of a thread-block cluster that share one unit in score ranking
 constexpr int kWarps = kThreads / 32;
+// Mean positions of a block of a cluster, at least (staged calls on four sequences of 260 to 5120 positions, 8 heads, four
+// layers, us: 1024 296, 2048 304, 4096, which leaves them one block each, 325).
+constexpr int kClusterPositions = 1024;
+constexpr int kTables = 8;         // register-resident score ranking: histograms of a block, one for every fourth warp
+constexpr int kBinades = 16, kCopies = 16;   // ... its first level: digits and counters of a digit (256 in all)
 typedef unsigned long long u64;
 
 struct UnitView {
@@ -95,8 +100,8 @@ template <typename Tv, typename Op> __device__ inline Tv block_reduce(Tv x, Tv *
     __syncthreads();
     if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = x;
     __syncthreads();
-    Tv r = buf[0];
-    for (int wv = 1; wv < kWarps; ++wv) r = op(r, buf[wv]);
+    Tv r = buf[threadIdx.x & 31];                 // (kWarps == 32; commutative, so every lane ends with the same bits)
+    for (int o = 16; o; o >>= 1) r = op(r, __shfl_xor_sync(0xffffffffu, r, o));
     return r;
 }
 // Values combined over the blocks of a cluster through distributed shared memory: every block
@@ -118,6 +123,10 @@ struct AddOpU64 { __device__ unsigned long long operator()(unsigned long long a,
 
 struct MinOp { __device__ int operator()(int a, int b) const { return min(a, b); } };
 struct MaxOpU { __device__ uint32_t operator()(uint32_t a, uint32_t b) const { return max(a, b); } };
+// largest 31-bit value, beside a flag in the top bit that any side may set
+struct MaxFlagOp {
+    __device__ uint32_t operator()(uint32_t a, uint32_t b) const { return ((a | b) & 0x80000000u) | max(a & 0x7fffffffu, b & 0x7fffffffu); }
+};
 struct AddOpF { __device__ float operator()(float a, float b) const { return a + b; } };
 
 // Ranks [lo, lo + len) in the order given by `pos_of` are split into one
@@ -224,7 +233,7 @@ struct SelectSmem {
     uint32_t y_mx;                    // fixed point, exchanged once: a block's largest key and its sum of squares
     float y_acc;                      // at that key's scale
     uint32_t z_key;                   // the crossing key, told by the block that holds it when one position has it
-    unsigned int wcnt[kWarps][257];   // per-warp private histograms (padded: one bank per warp for a digit)
+    unsigned int wcnt[kWarps][257];   // private histograms (padded: one bank per warp for a digit)
     u64 wsum[kWarps][257];
     int pack;
     u64 c_min;
@@ -470,6 +479,12 @@ select_budget_kernel(refree_params p, const float *scores, const int32_t *seq_le
 // position (e * blocks + rank) * kThreads + thread is element e of a thread, E elements each.  Same rule, fixed
 // point and radix descent as select_budget_kernel; the scores are read once, and a level of the descent costs a
 // handful of block barriers and one cluster barrier.
+//
+// Bound by barriers and by the shared-memory adds of the first level, whose digit (the upper exponent bits) has a handful of
+// values: nearly every lane of a warp met at one counter, and same-address adds go one after the other.  That level counts
+// binades instead, kBinades digits from the largest key's downwards with kCopies counters each, a lane's by its number;
+// keys below share the last one, and if the sum should cross there the level is taken again with plain digits.  (With the
+// counters of four warps in one table, 32K positions x 8 heads x 2 layers 34 us before.)
 template <int E>
 __global__ void __launch_bounds__(kThreads)
 select_score_resident_kernel(refree_params p, const float *scores, const int32_t *seq_len,
@@ -483,13 +498,13 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
     const int unit = blockIdx.x / nblk;
     const int Hkv = p.num_kv_heads;
     const int s = unit / Hkv, g = unit % Hkv;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, table = warp & (kTables - 1);
     scores += (int64_t)blockIdx.y * Hkv * total_tokens;
     cuts += blockIdx.y * p.num_seqs * Hkv;
     if (chunk_counts) chunk_counts += (int64_t)blockIdx.y * p.num_seqs * Hkv * chunk_stride;
     int32_t *const lengths = out.lengths[blockIdx.y];
     auto clear_hist = [&]() {
-        for (int t = threadIdx.x; t < kWarps * 257; t += kThreads) {
+        for (int t = threadIdx.x; t < kTables * 257; t += kThreads) {
             (&sm.wcnt[0][0])[t] = 0u;
             (&sm.wsum[0][0])[t] = 0ull;
         }
@@ -540,10 +555,11 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
     // Fixed point of the unit: C_n * 2^S in [2^60, 2^61), from the binary order of magnitude of the sum of squares.
     // A block sums its squares at the scale of its own largest key; the blocks exchange (largest key, sum) once and
     // bring the sums to the scale of the unit's largest key, a power of two apart, in rank order.
-    const uint32_t mx_b = block_reduce<uint32_t>(mx, reinterpret_cast<uint32_t *>(sm.ibuf), MaxOpU());
+    // (the top bit says that some score is not finite)
+    const uint32_t mx_b = block_reduce<uint32_t>(mx | (bad ? 0x80000000u : 0u), reinterpret_cast<uint32_t *>(sm.ibuf), MaxFlagOp());
     float acc_b = 0.f;
     {
-        const float fb = ldexpf(1.0f, 127 - max(1, (int)(mx_b >> 23)));
+        const float fb = ldexpf(1.0f, 127 - max(1, (int)((mx_b & 0x7fffffffu) >> 23)));
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             if (e >= e_lim) continue;
@@ -566,12 +582,14 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
         }
         mx = 0u;
 #pragma unroll
-        for (int b = 0; b < kMaxCluster; ++b) mx = max(mx, rm[b]);
+        for (int b = 0; b < kMaxCluster; ++b) { mx = MaxFlagOp()(mx, rm[b]); rm[b] &= 0x7fffffffu; }
         acc = 0.f;
 #pragma unroll
         for (int b = 0; b < kMaxCluster; ++b)
-            if (b < nblk) acc += ldexpf(ra[b], 2 * (max(1, (int)(rm[b] >> 23)) - max(1, (int)(mx >> 23))));
+            if (b < nblk) acc += ldexpf(ra[b], 2 * (max(1, (int)(rm[b] >> 23)) - max(1, (int)((mx & 0x7fffffffu) >> 23))));
     }
+    const bool finite = !(mx >> 31);
+    mx &= 0x7fffffffu;
     if (n > 0 && mx != 0u) {
         const int emax = max(1, (int)(mx >> 23));
         v.sbias = 60 - ilogbf(fmaxf(acc, 0.25f)) - 2 * (emax - 127) - 300;
@@ -622,25 +640,43 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
             int digit_cnt = 0;
             bool any = true;
             bool spelled = false;             // the crossing key is known in full before the last level
+            const uint32_t top = mx >> 24;    // digit of the largest key
+            bool plain = !finite;             // the first level by plain digits
+            int hb = 1;                       // the histogram copy of this exchange
             for (int level = 0; level < 4 && any && !spelled; ++level) {
                 const int shift = 24 - 8 * level;
-                const int hb = level & 1;
+                const bool binades = level == 0 && !plain;
+                hb ^= 1;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
                     const int i = (e * nblk + rank) * kThreads + threadIdx.x;
                     if (e < e_lim && i >= v.lead && i < n - v.w_eff && (level == 0 || (kb[e] >> (shift + 8)) == prefix)) {
-                        const int dgt = (int)((kb[e] >> shift) & 255u);
-                        atomicAdd(&sm.wcnt[warp][dgt], 1u);
-                        add_u64_shared(&sm.wsum[warp][dgt], sq_fixed(kb[e], v.sbias));
+                        int dgt = (int)((kb[e] >> shift) & 255u);
+                        if (binades) dgt = min((int)top - dgt, kBinades - 1) * kCopies + (lane & (kCopies - 1));
+                        atomicAdd(&sm.wcnt[table][dgt], 1u);
+                        add_u64_shared(&sm.wsum[table][dgt], sq_fixed(kb[e], v.sbias));
                     }
                 }
                 __syncthreads();
                 if (threadIdx.x < 256) {
                     unsigned int c = 0u;
                     u64 sumv = 0ull;
-                    for (int wv = 0; wv < kWarps; ++wv) { c += sm.wcnt[wv][threadIdx.x]; sumv += sm.wsum[wv][threadIdx.x]; }
-                    sm.hcnt2[hb][threadIdx.x] = c;
-                    sm.hsum2[hb][threadIdx.x] = sumv;
+#pragma unroll
+                    for (int tb = 0; tb < kTables; ++tb) { c += sm.wcnt[tb][threadIdx.x]; sumv += sm.wsum[tb][threadIdx.x]; }
+                    int dgt = threadIdx.x;
+                    bool mine = true;
+                    if (binades) {            // the copies of a digit are neighbouring lanes; digits without counters are empty
+#pragma unroll
+                        for (int o = 1; o < kCopies; o <<= 1) {
+                            c += __shfl_xor_sync(0xffffffffu, c, o);
+                            sumv += __shfl_xor_sync(0xffffffffu, sumv, o);
+                        }
+                        const int below = (int)top - dgt;
+                        if (below < 0 || below >= kBinades) { sm.hcnt2[hb][dgt] = 0u; sm.hsum2[hb][dgt] = 0ull; }
+                        dgt = (int)top - (int)threadIdx.x / kCopies;
+                        mine = dgt >= 0 && (threadIdx.x & (kCopies - 1)) == 0;
+                    }
+                    if (mine) { sm.hcnt2[hb][dgt] = c; sm.hsum2[hb][dgt] = sumv; }
                 }
                 // thread t < 256 owns digit 255 - t: the cluster's totals of it (integers: any order)
                 unsigned int mycnt = 0u;
@@ -662,7 +698,7 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
                     __syncthreads();
                     if (threadIdx.x < 256) { mycnt = sm.hcnt2[hb][255 - threadIdx.x]; mysum = sm.hsum2[hb][255 - threadIdx.x]; }
                 }
-                clear_hist();                 // for the next level: the per-warp histograms were read before the barrier above
+                clear_hist();                 // for the next level: the tables were read before the barrier above
                 // sums from the top digit down; the first digit at which they reach what is missing
                 const u64 inc_s = warp_incl_scan(mysum);
                 const unsigned int inc_c = warp_incl_scan(mycnt);
@@ -690,6 +726,9 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
                     if (sm.dcand[wv] != INT_MAX) { cand = sm.dcand[wv]; cw = wv; }
                 if (cand == INT_MAX) {
                     any = false;              // the rule is never met: keep all
+                } else if (binades && 255 - cand == (int)top - (kBinades - 1)) {
+                    plain = true;             // (the counters are clear: a barrier has passed since)
+                    level = -1;
                 } else {
                     prefix = (prefix << 8) | (uint32_t)(255 - cand);
                     above_sum += sm.dabv_s[cw];
@@ -809,17 +848,22 @@ unit_rules_kernel(refree_params p, const float *scores, const int32_t *seq_len, 
     block_unit_rule<kThreadsRule>(ur, rule, out.lengths[blockIdx.y] + u, cuts + blockIdx.y * p.num_seqs * Hkv + u);
 }
 
-// Offsets (running sum of lengths) and the kept positions of each unit, ascending.
-__global__ void __launch_bounds__(kThreads)
+// Offsets (running sum of lengths) and the kept positions of each unit, ascending.  Bound by latency: what a block adds up
+// (budgets before its unit, kept positions before its run, its own positions) meets in one barrier (32K positions x 8 heads x
+// 2 layers: 20 us with a block of kThreads and a scan for each).  With score ranking a block takes a run of kThreads
+// positions, four to a thread.
+constexpr int kEmitThreads = 256, kEmitWarps = kEmitThreads / 32, kPerThread = kThreads / kEmitThreads;
+static_assert(kPerThread * kEmitWarps == 32, "one count per lane");
+__global__ void __launch_bounds__(kEmitThreads)
 emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_t total_tokens,
             const __grid_constant__ SelectOut out, const Cut *cuts,
             int64_t capacity_rows, int32_t *dev_status, const int2 *chunk_counts, int chunk_stride, int counted_upto)
 {
-    __shared__ long long lbuf[kWarps + 1];
-    __shared__ int ibuf[kWarps + 1];
-    __shared__ int s_pack;
+    __shared__ long long s_len[kEmitWarps], s_before[kEmitWarps];      // per warp: budgets; (kept for sure << 32) + ties
+    __shared__ int s_cnt[32];                                          // per 32 positions: (kept for sure << 16) + ties
     const int Hkv = p.num_kv_heads, U = p.num_seqs * Hkv;
     const int u = blockIdx.y, s = u / Hkv, g = u % Hkv;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     scores += (int64_t)blockIdx.z * Hkv * total_tokens;
     cuts += blockIdx.z * U;
     if (chunk_counts) chunk_counts += (int64_t)blockIdx.z * U * chunk_stride;
@@ -828,21 +872,96 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
     int32_t *const kept_idx = out.kept[blockIdx.z];
     dependency_wait();
     trigger_dependents();
+    const int n = max(seq_len[s], 0), chunk = blockIdx.x * kThreads;
+    const bool ranges = p.rank_mode == REFREE_RANK_POSITION || p.force_full;
     // score ranking: a block beyond the end of its sequence has nothing to do (the grid is sized for the longest
     // sequence a call can hold)
-    if (blockIdx.x > 0 && p.rank_mode != REFREE_RANK_POSITION && !p.force_full &&
-        (int64_t)blockIdx.x * kThreads >= max(seq_len[s], 0))
-        return;
-    // offsets[u] = sum of lengths before u
-    long long part = 0, off;
-    for (int t = threadIdx.x; t < u; t += kThreads) part += lengths[t];
-    {
-        long long tot;
-        block_excl_scan<long long>(part, lbuf, tot);
-        off = tot;
-    }
+    if (blockIdx.x > 0 && !ranges && chunk >= n) return;
     const Cut cut = cuts[u];
     const int b = cut.b;
+    long long part = 0, before = 0;
+    for (int t = threadIdx.x; t < u; t += kEmitThreads) part += lengths[t];
+    // kept for sure (above the crossing key, or protected and inside the budget) / at the crossing key, of
+    // which the cut.ties lowest positions are kept
+    const bool listed = kept_idx != nullptr && !ranges && chunk < n;
+    unsigned int smask[kPerThread], tmask[kPerThread];                 // of this warp's positions chunk + q kEmitThreads + threadIdx.x
+    if (listed) {
+        int pack = 0;
+        for (int t = lane; t < s; t += 32) pack += max(seq_len[t], 0);
+        pack = __reduce_add_sync(0xffffffffu, pack);
+        int lead = min(p.sink, n), w_eff = min(p.window, n);
+        if (lead + w_eff >= n) { lead = n; w_eff = 0; }
+        UnitView v;
+        const bool layer = p.scope == REFREE_SCOPE_LAYER;
+        v.sc = scores + (int64_t)(layer ? 0 : g) * total_tokens + pack;
+        v.head_stride = total_tokens;
+        v.heads = layer ? Hkv : 1;
+        v.n = n; v.lead = lead; v.w_eff = w_eff;
+        v.sbias = cut.sbias;
+        // the key is loaded first, without a branch around it, so that a thread's loads are in flight together
+        const bool one_head = v.heads == 1;
+        auto key_of = [&](int i) {
+            if (one_head) {                       // a plain predicated load, so the loads of an unrolled loop overlap
+                const int ic = min(max(i, 0), n - 1);
+                const uint32_t bits = mag_bits(v.sc[ic]);
+                return (i >= lead && i < n - w_eff) ? (u64)bits << 32 : 0ull;
+            }
+            return (i >= lead && i < n - w_eff) ? key_at(v, i) : 0ull;
+        };
+        auto classify = [&](int i, u64 key, bool &sure, bool &tie) {
+            sure = false; tie = false;
+            if (i >= n) return;
+            if (i < lead) {
+                sure = i < cut.prot_kept;
+            } else if (i >= n - w_eff) {
+                sure = lead + (i - (n - w_eff)) < cut.prot_kept;
+            } else {
+                sure = key > cut.tau;
+                tie = key == cut.tau;
+            }
+        };
+        u64 key[kPerThread];
+#pragma unroll
+        for (int q = 0; q < kPerThread; ++q) key[q] = key_of(chunk + q * kEmitThreads + (int)threadIdx.x);
+        // What the positions before the chunk contribute: left per run of kThreads positions by the kernel that chose
+        // the budget when it held the unit in registers; otherwise every block counts them itself (the scores are in L2).
+        if (chunk_counts && n <= counted_upto) {
+            for (int c = threadIdx.x; c < (int)blockIdx.x; c += kEmitThreads) {
+                const int2 cc = chunk_counts[(int64_t)u * chunk_stride + c];
+                before += ((long long)cc.x << 32) + (long long)cc.y;
+            }
+        } else
+        for (int i0 = threadIdx.x; i0 < chunk; i0 += 8 * kEmitThreads) {
+            u64 k8[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) k8[q] = key_of(i0 + q * kEmitThreads < chunk ? i0 + q * kEmitThreads : n);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                bool sure, tie;
+                classify(i0 + q * kEmitThreads < chunk ? i0 + q * kEmitThreads : n, k8[q], sure, tie);
+                before += ((long long)sure << 32) + (long long)tie;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kPerThread; ++q) {
+            bool sure, tie;
+            classify(chunk + q * kEmitThreads + (int)threadIdx.x, key[q], sure, tie);
+            smask[q] = __ballot_sync(0xffffffffu, sure);
+            tmask[q] = __ballot_sync(0xffffffffu, tie);
+            if (lane == 0) s_cnt[q * kEmitWarps + warp] = (__popc(smask[q]) << 16) + __popc(tmask[q]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        part += __shfl_xor_sync(0xffffffffu, part, o);
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+    }
+    if (lane == 0) { s_len[warp] = part; s_before[warp] = before; }
+    __syncthreads();
+    long long off = 0;                            // offsets[u] = sum of lengths before u
+    before = 0;
+#pragma unroll
+    for (int w = 0; w < kEmitWarps; ++w) { off += s_len[w]; before += s_before[w]; }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         offsets[u] = off;
         if (u == U - 1) offsets[U] = off + b;
@@ -852,115 +971,48 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
         return;
     }
     if (kept_idx == nullptr) return;
-    const int n = max(seq_len[s], 0);
-    int lead = min(p.sink, n), w_eff = min(p.window, n);
     int32_t *dst = kept_idx + off;
-    if (p.rank_mode == REFREE_RANK_POSITION || p.force_full) {
-        const int head = min(b, lead);
-        for (int t = blockIdx.x * kThreads + threadIdx.x; t < b; t += gridDim.x * kThreads)
+    if (ranges) {
+        const int head = min(b, min(p.sink, n));
+        for (int t = blockIdx.x * kEmitThreads + threadIdx.x; t < b; t += gridDim.x * kEmitThreads)
             dst[t] = t < head ? t : n - b + t;
         return;
     }
-    // Score ranking: block c of the unit owns positions [c * kThreads, (c + 1) * kThreads), one per thread.
-    const int chunk = blockIdx.x * kThreads;
-    if (chunk >= n) return;
-    if (threadIdx.x == 0) {
-        int a = 0;
-        for (int t = 0; t < s; ++t) a += max(seq_len[t], 0);
-        s_pack = a;
-    }
-    __syncthreads();
-    if (lead + w_eff >= n) { lead = n; w_eff = 0; }
-    UnitView v;
-    const bool layer = p.scope == REFREE_SCOPE_LAYER;
-    v.sc = scores + (int64_t)(layer ? 0 : g) * total_tokens + s_pack;
-    v.head_stride = total_tokens;
-    v.heads = layer ? Hkv : 1;
-    v.n = n; v.lead = lead; v.w_eff = w_eff;
-    v.sbias = cut.sbias;
-    // kept for sure (above the crossing key, or protected and inside the budget) / at the crossing key, of
-    // which the cut.ties lowest positions are kept
-    // the key is loaded first, without a branch around it, so that a thread's loads are in flight together
-    const bool one_head = v.heads == 1;
-    auto key_of = [&](int i) {
-        if (one_head) {                           // a plain predicated load, so the loads of an unrolled loop overlap
-            const int ic = min(max(i, 0), n - 1);
-            const uint32_t bits = mag_bits(v.sc[ic]);
-            return (i >= lead && i < n - w_eff) ? (u64)bits << 32 : 0ull;
-        }
-        return (i >= lead && i < n - w_eff) ? key_at(v, i) : 0ull;
-    };
-    auto classify = [&](int i, u64 key, bool &sure, bool &tie) {
-        sure = false; tie = false;
-        if (i >= n) return;
-        if (i < lead) {
-            sure = i < cut.prot_kept;
-        } else if (i >= n - w_eff) {
-            sure = lead + (i - (n - w_eff)) < cut.prot_kept;
-        } else {
-            sure = key > cut.tau;
-            tie = key == cut.tau;
-        }
-    };
-    // What the positions before the chunk contribute: left per run of kThreads positions by the kernel that chose
-    // the budget when it held the unit in registers; otherwise every block counts them itself (the scores are in L2).
-    long long before = 0;                                   // (sure << 32) + ties
-    if (chunk_counts && n <= counted_upto) {
-        for (int c = threadIdx.x; c < (int)blockIdx.x; c += kThreads) {
-            const int2 cc = chunk_counts[(int64_t)u * chunk_stride + c];
-            before += ((long long)cc.x << 32) + (long long)cc.y;
-        }
-    } else
-    for (int i0 = threadIdx.x; i0 < chunk; i0 += 8 * kThreads) {
-        u64 key[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) key[q] = key_of(i0 + q * kThreads < chunk ? i0 + q * kThreads : n);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            bool sure, tie;
-            classify(i0 + q * kThreads < chunk ? i0 + q * kThreads : n, key[q], sure, tie);
-            before += ((long long)sure << 32) + (long long)tie;
-        }
-    }
-    {
-        long long tot;
-        block_excl_scan<long long>(before, lbuf, tot);
-        before = tot;
-    }
+    if (!listed) return;
+    const int mine = s_cnt[lane], excl = warp_incl_scan(mine) - mine;
     const int ties_before = (int)(before & 0xffffffffll), sure_before = (int)(before >> 32);
-    const int lane = threadIdx.x & 31;
-    bool sure, tie;
-    classify(chunk + threadIdx.x, key_of(chunk + threadIdx.x), sure, tie);
-    const unsigned int tm = __ballot_sync(0xffffffffu, tie);
-    int tie_tot;
-    const int tie_base = block_excl_scan<int>(lane == 0 ? __popc(tm) : 0, ibuf, tie_tot);   // lane 0 carries the warp's count
-    const int tie_rank = ties_before + __shfl_sync(0xffffffffu, tie_base, 0) + __popc(tm & ((1u << lane) - 1u));
-    if (tie && tie_rank < cut.ties) sure = true;
-    const unsigned int km = __ballot_sync(0xffffffffu, sure);
-    int keep_tot;
-    const int keep_base = block_excl_scan<int>(lane == 0 ? __popc(km) : 0, ibuf, keep_tot);
-    const int mine = sure_before + min(ties_before, cut.ties) + __shfl_sync(0xffffffffu, keep_base, 0) +
-                     __popc(km & ((1u << lane) - 1u));
-    if (sure && mine < b) dst[mine] = chunk + threadIdx.x;
+    const unsigned int lower = (1u << lane) - 1u;
+#pragma unroll
+    for (int q = 0; q < kPerThread; ++q) {
+        const int x = __shfl_sync(0xffffffffu, excl, q * kEmitWarps + warp);
+        // of the ties before a position the first cut.ties are kept
+        const int ties = ties_before + (x & 0xffff) + __popc(tmask[q] & lower);
+        const int at = sure_before + (x >> 16) + __popc(smask[q] & lower) + min(ties, cut.ties);
+        const bool keep = ((smask[q] >> lane) & 1u) || (((tmask[q] >> lane) & 1u) && ties < cut.ties);
+        if (keep && at < b) dst[at] = chunk + q * kEmitThreads + (int)threadIdx.x;
+    }
 }
 
-// Whether clusters of `nblk` blocks of the kernel can run on the current device.  The answer is a property of the kernel
-// and the device; asking the runtime takes microseconds of every call, so it is kept (slot: which kernel).
+// Clusters of `nblk` blocks of the kernel that the current device holds at once (0: none can run).  The answer is a property
+// of the kernel and the device; asking the runtime takes microseconds of every call, so it is kept (slot: which kernel).
 template <typename Kern>
-bool cluster_fits(int slot, int nblk, Kern kern, const cudaLaunchConfig_t &cfg)
+int cluster_room(int slot, int nblk, Kern kern, const cudaLaunchConfig_t &cfg)
 {
     static std::mutex m;
-    static signed char known[64][17][kMaxCluster + 1] = {};            // 0 unknown, 1 yes, -1 no
+    static int known[64][17][kMaxCluster + 1] = {};                    // 0 unknown, else one more than the answer
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     std::lock_guard<std::mutex> hold(m);
-    signed char &k = known[dev][slot][nblk];
+    int &k = known[dev][slot][nblk];
     if (k == 0) {
         int clusters = 0;
-        k = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1 ? 1 : -1;
-        if (k < 0) (void)cudaGetLastError();
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+            clusters = 0;
+            (void)cudaGetLastError();
+        }
+        k = std::max(clusters, 0) + 1;
     }
-    return k > 0;
+    return k - 1;
 }
 
 }  // namespace
@@ -1008,37 +1060,39 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
     if (!have_budgets) {                     // (else the scoring launch left budgets and cuts already)
         // score ranking walks every score several times: a cluster of blocks shares a unit (distributed
         // shared memory for the few totals they exchange); position ranking keeps one block per unit
-        int nblk = 1;
-        if (p.rank_mode == REFREE_RANK_SCORE && !p.force_full) {
-            const int64_t avg = total_tokens / std::max(1, p.num_seqs);
-            while (nblk < kMaxCluster && avg >= (int64_t)nblk * 4096) nblk *= 2;
-            // a block takes an SM, and clusters leave some SMs of a group of them unused: stay well within one wave (16
-            // units of 32K positions: 61 us in clusters of eight, which came in two waves, 38 in clusters of four)
-            // (but not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some
-            // 100 us for it: eleven sequences of 69 to 29809 positions, 8 heads, four layers 1428 -> 1015)
-            const bool resident = p.scope == REFREE_SCOPE_HEAD;
-            while (nblk > 1 && (int64_t)sel_units * layers * nblk * 4 > (int64_t)sm_count() * 3 &&
-                   (!resident || (int64_t)(nblk / 2) * kThreads * 16 >= total_tokens)) nblk /= 2;
-        }
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(sel_units * nblk, layers);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = sizeof(SelectSmem);
         cfg.stream = st;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = nblk;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = st.chain ? 2 : 1;
-        if (nblk > 1 && !cluster_fits(0, nblk, select_budget_kernel, cfg)) {
-            nblk = 1;
-            cfg.gridDim = dim3(sel_units, layers);
-            attr[0].val.clusterDim.x = 1;
+        auto shape = [&](int n) {
+            attr[0].val.clusterDim.x = n;
+            cfg.gridDim = dim3(sel_units * n, layers);
+        };
+        int nblk = 1;
+        if (p.rank_mode == REFREE_RANK_SCORE && !p.force_full) {
+            const int64_t avg = total_tokens / std::max(1, p.num_seqs);
+            while (nblk < kMaxCluster && avg >= (int64_t)nblk * kClusterPositions) nblk *= 2;
+            // One wave: a block takes an SM, and clusters leave some SMs of a group of them unused (16 units of 32K positions:
+            // 61 us in clusters of eight, which came in two waves, 38 in clusters of four).
+            // (But not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some
+            // 100 us for it: eleven sequences of 69 to 29809 positions, 8 heads, four layers 1428 -> 1015.)
+            const bool resident = p.scope == REFREE_SCOPE_HEAD;
+            for (; nblk > 1; nblk /= 2) {
+                shape(nblk);
+                const int room = cluster_room(0, nblk, select_budget_kernel, cfg);
+                if (room == 0) continue;
+                if ((int64_t)sel_units * layers <= room || (resident && (int64_t)(nblk / 2) * kThreads * 16 < total_tokens)) break;
+            }
         }
+        shape(nblk);
         // Score ranking per head: units short enough for a cluster to hold in registers go to the kernel that
         // reads the scores once; the general kernel takes the rest (all of them when none is short enough).
         if (p.rank_mode == REFREE_RANK_SCORE && !p.force_full && p.scope == REFREE_SCOPE_HEAD) {
@@ -1054,7 +1108,7 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
             rc.attrs = rattr;
             rc.gridDim = dim3(sel_units * rb, layers);
             cudaError_t re = cudaErrorInvalidValue;
-            auto fits = [&](auto kern) { return rb == 1 || cluster_fits(E, rb, kern, rc); };
+            auto fits = [&](auto kern) { return rb == 1 || cluster_room(E, rb, kern, rc) > 0; };
             // counts per run of kThreads positions for the index list, where the caller's workspace has room for them
             if (emit && kept_idx && lay.part_bytes >= (size_t)U * layers * (size_t)chunk_stride * sizeof(int2))
                 chunk_counts = reinterpret_cast<int2 *>(ws + lay.part_off);
@@ -1084,12 +1138,12 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
     int gx = 1;
     if (ranges && kept_idx) {
         const int64_t per_unit = std::max<int64_t>(1, total_tokens / std::max(1, p.num_seqs));
-        gx = (int)std::min<int64_t>(16, (per_unit + 4 * kThreads - 1) / (4 * kThreads));
+        gx = (int)std::min<int64_t>(64, (per_unit + 4 * kEmitThreads - 1) / (4 * kEmitThreads));
     } else if (kept_idx) {
         // score ranking: a block per kThreads positions of the longest sequence there can be
         gx = (int)std::max<int64_t>(1, (total_tokens + kThreads - 1) / kThreads);
     }
-    const cudaError_t ee = launch_dependent(emit_kernel, dim3(gx, U, layers), dim3(kThreads), 0, st, p, scores, seq_len, total_tokens,
+    const cudaError_t ee = launch_dependent(emit_kernel, dim3(gx, U, layers), dim3(kEmitThreads), 0, st, p, scores, seq_len, total_tokens,
                                             out, cuts, capacity_rows, dev_status, chunk_counts,
                                             chunk_stride, skip_upto);
     if (ee != cudaSuccess) return ee;
