@@ -597,17 +597,28 @@ int w1_batch(const refree_params &p, int64_t total_tokens, int num_layers, size_
     return n;
 }
 
-// Layers of a run that one launch scores together.  A launch costs about 22 us beyond its tiles (setup, the first loads,
-// normalisers, the stopping rule, the last CTA of the chain), paid once per group; a group's rows, 2.7 us per layer and
-// item (128 positions of a KV head) of an SM, are moved without scoring beside them at the end of the run.  The sum is
-// smallest at sqrt(8 layers / items per SM) layers.  Measured, 8 KV heads of 256 rows: 16 layers of 8K positions 707 us
-// one by one, 527 in twos, 444 in fours, 418 in eights; of 2K positions 390, 341, 247 and 180; 8 layers of 32K 728 one by
-// one, 679 in twos, 716 in fours.
+// Layers of a run that one launch scores together, at most kMaxBatch.  A launch costs some 20 us beyond its tiles (setup, the
+// first loads, normalisers, the stopping rule, the last CTA of the chain), paid once per group.
+//   `copy` (the scoring moves an earlier group's rows): the rows of the last group, 2.7 us per layer and item (128 positions
+// of a KV head) of an SM, move without scoring beside them, those of the others at about a third of that time; so the sum is
+// smallest at a number of groups near sqrt(1.75 layers items / launch), where a launch counts 13 us at 129 to 256 query rows
+// and 24 below, where there is less to hide rows behind.  Beyond 256 rows Q leaves little room for rows on their way and
+// the fewest groups win.  Measured, us, 8 KV heads unless said (groups of 1, 2, 3, 4, 8): 256 rows, 8 layers of 32K positions
+// 693, 666, 685, 706, 747; four 370, 370, 370, 383; 16 of 8K 616, 453, 430, 396, 385; four 177, 138, 137, 132; 64 rows,
+// eight of 4K, 16 heads 274, 213, 208, 194, 183; 128 rows, 16 of 30K, 2 heads 550, 385, 407, 359, 321; 448 rows, 4 of the
+// ragged batch of eight 645, 680, 682, 608; 512 rows, 8 of 20K 717, 710, 713, 749, 700; 4 of 16K 324, 331, 331, 310.
+//   Else (score ranking, rows that are not contiguous) selection and copy are launches of their own and every group pays for
+// them: 32K x 8 ranked by score 896, 714, 657, 588, 548; 20K x 8 908, 762, 701, 633, 589; the ragged batch x 4 1011, 864,
+// 864, 791.
 int run_batch(const refree_params &p, int64_t total_tokens, int num_layers, size_t workspace_bytes, bool copy)
 {
-    const double items = (double)(total_tokens / kTile + p.num_seqs) * p.num_kv_heads / sm_count();
-    int n = (int)std::lround(std::sqrt(8.0 * num_layers / std::max(items, 0.125)));
-    n = std::max(1, std::min({n, kMaxBatch, num_layers}));
+    int n = std::min(kMaxBatch, num_layers);
+    const int rows = p.num_q_heads / p.num_kv_heads * p.window;
+    if (copy && rows <= 256) {
+        const double items = (double)(total_tokens / kTile + p.num_seqs) * p.num_kv_heads / sm_count();
+        const int groups = std::max(1, (int)std::lround(std::sqrt(1.75 * num_layers * items / (rows > 128 ? 13.0 : 24.0))));
+        n = std::min(n, (num_layers + groups - 1) / groups);
+    }
     while (n > 1 && ((copy && !score_tc_can_copy(p, total_tokens, n)) || 2 * batch_layout(p, total_tokens, n).total > workspace_bytes)) --n;
     return n;
 }
