@@ -70,9 +70,12 @@ compact_kernel(refree_params p, const __grid_constant__ CompactJob job, const in
     }
     const int head = min(b, min(p.sink, n));
     const int64_t tok0 = seq_start[s];
+    if (int32_t *const list = job.kept_out[layer])
+        for (int t = blockIdx.x * kThreads + threadIdx.x; t < b; t += gridDim.x * kThreads) list[off + t] = t < head ? t : n - b + t;
     const char *kb = k + ((int64_t)s * p.k_stride_seq + tok0 * p.k_stride_tok + (int64_t)g * p.k_stride_head) * esz;
     const char *vb = v + ((int64_t)s * p.v_stride_seq + tok0 * p.v_stride_tok + (int64_t)g * p.v_stride_head) * esz;
     const int64_t k_tok = p.k_stride_tok * esz, v_tok = p.v_stride_tok * esz;
+    const bool move_k = job.k_out[layer] != nullptr, move_v = job.v_out[layer] != nullptr;
     char *ko = job.k_out[layer] + off * row_bytes, *vo = job.v_out[layer] + off * row_bytes;
     const int32_t *idx = kept_idx ? kept_idx + off : nullptr;
     const int64_t nvec = (int64_t)b << vshift;
@@ -90,8 +93,8 @@ compact_kernel(refree_params p, const __grid_constant__ CompactJob job, const in
                 // an index list is the caller's: a row outside the sequence is reported, never read
                 good[r] = src >= 0 && src < n;
                 if (good[r]) {
-                    kv[r] = *reinterpret_cast<const int4 *>(kb + (int64_t)src * k_tok + c * 16);
-                    vv[r] = ld_stream(reinterpret_cast<const int4 *>(vb + (int64_t)src * v_tok + c * 16));
+                    if (move_k) kv[r] = *reinterpret_cast<const int4 *>(kb + (int64_t)src * k_tok + c * 16);
+                    if (move_v) vv[r] = ld_stream(reinterpret_cast<const int4 *>(vb + (int64_t)src * v_tok + c * 16));
                 } else if (dev_status) {
                     atomicOr(dev_status, REFREE_DEV_CAPACITY);
                 }
@@ -101,8 +104,8 @@ compact_kernel(refree_params p, const __grid_constant__ CompactJob job, const in
         for (int r = 0; r < kUnroll; ++r) {
             const int64_t e = e0 + r * stride;
             if (e < nvec && good[r]) {
-                st_stream(reinterpret_cast<int4 *>(ko + e * 16), kv[r]);
-                st_stream(reinterpret_cast<int4 *>(vo + e * 16), vv[r]);
+                if (move_k) st_stream(reinterpret_cast<int4 *>(ko + e * 16), kv[r]);
+                if (move_v) st_stream(reinterpret_cast<int4 *>(vo + e * 16), vv[r]);
             }
         }
     }

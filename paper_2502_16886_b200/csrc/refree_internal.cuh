@@ -182,7 +182,9 @@ inline cudaError_t allow_smem(Kern kern, size_t smem)
 cudaError_t launch_score_generic(const refree_params &p, const void *q_win, const void *k,
                                  const int32_t *seq_start, const int32_t *seq_len,
                                  int64_t total_tokens, float *scores, char *ws, const Workspace &lay,
-                                 int32_t *dev_status, Stream st);
+                                 int32_t *dev_status, Stream st, GroupPartial *groups = nullptr, int32_t *sel_lengths = nullptr);
+// Whether launch_score_generic evaluates the stopping rule too, given `groups` and `sel_lengths` (short calls).
+bool score_generic_rule(const refree_params &p, int64_t total_tokens);
 
 // Layers of a run that one launch scores together, at most (see refree_compress_layers).
 constexpr int kMaxBatch = 8;
@@ -262,7 +264,8 @@ struct CompactJob {
     const int64_t *offsets[kMaxBatch];      // read unless offsets_out forms them
     const int32_t *kept[kMaxBatch];         // nullable with position ranges
     int64_t *offsets_out[kMaxBatch];        // nullable: the kernel forms the running sum of the budgets itself
-    char *k_out[kMaxBatch], *v_out[kMaxBatch];
+    int32_t *kept_out[kMaxBatch];           // nullable, position ranges: the kernel writes the index list
+    char *k_out[kMaxBatch], *v_out[kMaxBatch];      // either null: those rows are not moved
 };
 
 // The stopping rule of every unit from the records that the scoring left (position ranking per head).
@@ -284,15 +287,24 @@ inline SelectOut select_out(int32_t *lengths, int64_t *offsets, int32_t *kept)
 cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const int32_t *seq_start, const int32_t *seq_len,
                            bool position_ranges, int64_t capacity_rows, int32_t *dev_status, Stream st);
 inline CompactJob compact_job(const void *k, const void *v, const int32_t *lengths, const int64_t *offsets, const int32_t *kept,
-                              int64_t *offsets_out, void *k_out, void *v_out)
+                              int64_t *offsets_out, void *k_out, void *v_out, int32_t *kept_out = nullptr)
 {
     CompactJob j = {};
     j.layers = 1;
     j.k[0] = (const char *)k; j.v[0] = (const char *)v;
     j.lengths[0] = lengths; j.offsets[0] = offsets; j.kept[0] = kept; j.offsets_out[0] = offsets_out;
+    j.kept_out[0] = kept_out;
     j.k_out[0] = (char *)k_out; j.v_out[0] = (char *)v_out;
     return j;
 }
+
+// Strides and alignment of a layer's caches.
+refree_status check_kv_layout(const refree_params *p, const void *k, const void *v, bool need_v);
+// Scoring and selection of one layer; launch_compact with `job` is what is left of it.
+cudaError_t enqueue_selection(const refree_params &p, const void *q_win, const void *k, const void *v, const int32_t *seq_start,
+                              const int32_t *seq_len, int64_t total_tokens, void *k_out, void *v_out, int64_t capacity_rows,
+                              int32_t *lengths, int64_t *offsets, int32_t *kept_idx, float *scores, char *ws, const Workspace &lay,
+                              int32_t *device_status, Stream cs, CompactJob &job);
 
 // With `lengths` and `offsets_out` (end-anchored form only) the kernel takes the budgets from `lengths` and
 // writes their running sum itself, so the selection need not emit offsets first.

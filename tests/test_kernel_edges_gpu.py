@@ -1,0 +1,112 @@
+"""Sizes at which the short-call kernels, the score ranking and the single-row stream can go wrong: edges of tiles and row
+chunks, spreads of the scores, layers that share a warp."""
+import dataclasses
+import math
+from fractions import Fraction
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2502_16886_b200 import binding, build, workloads
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+    binding.lib()
+
+
+def cfg_like(**kw):
+    return dataclasses.replace(workloads.CONFIGS[0], **kw)
+
+
+@pytest.mark.parametrize("dtype,d,hq,hkv,w,lens", [
+    ("fp32", 64, 4, 2, 16, [1]), ("fp32", 64, 3, 3, 5, [64, 0, 63, 65, 1]), ("bf16", 64, 6, 2, 11, [513 - 130, 64, 65]),
+    ("fp32", 128, 4, 4, 33, [512]), ("fp32", 128, 16, 4, 16, [200, 64, 0, 65, 183]), ("fp32", 64, 8, 2, 16, [513]),
+    ("fp32", 64, 2, 2, 65, [300]), ("bf16", 64, 2, 2, 17, [449]), ("bf16", 64, 34, 2, 1, [70, 90])])
+def test_short_units_from_keys_to_budgets(dtype, d, hq, hkv, w, lens):
+    """Row counts around the chunks (16, 32, 64) and one more than the most, one position, empty sequences, fewer tiles than
+    blocks, the longest call and one more position."""
+    cfg = cfg_like(num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype=dtype, window=w)
+    lay = workloads.make_layer(cfg, 0, seq_lens=lens)
+    for rank_mode, scope in ((0, 0), (0, 1), (1, 0)):
+        parity.run_fused_and_check(cfg, lay, rank_mode=rank_mode, scope=scope, threshold=0.05)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(8, 2, 128), (16, 1, 128), (12, 1, 64)])
+@pytest.mark.parametrize("lens", [[8193], [20_000, 255, 0, 257], [300] * 40])
+def test_single_query_row_beyond_the_short_calls(hq, hkv, d, lens):
+    cfg = cfg_like(num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype="bf16", window=1)
+    lay = workloads.make_layer(cfg, 1, seq_lens=lens)
+    parity.run_fused_and_check(cfg, lay, rank_mode=0)
+
+
+def _exact_rule(a, lead, w_eff, threshold):
+    """Budget and kept positions of one unit ranked by score, by the documented integers (squares in fixed point, C_n in
+    [2^60, 2^61))."""
+    n = len(a)
+    sq = [Fraction(float(x)) ** 2 for x in a]
+    scale = Fraction(2) ** (60 - math.floor(math.log2(float(sum(sq)))))
+    sq = [math.floor(x * scale) for x in sq]
+    prot = list(range(lead)) + list(range(n - w_eff, n))
+    order = prot + sorted(range(lead, n - w_eff), key=lambda i: (-float(a[i]), i))
+    total = sum(sq)
+    t = float(np.float32(threshold))
+    c_min = total - (math.ceil(float(total) * (t * (2.0 - t))) - 1)
+    c, j = 0, n
+    for r, i in enumerate(order):
+        c += sq[i]
+        if c >= c_min:
+            j = r + 1
+            break
+    b = max(j, len(prot))
+    return b, sorted(order[:b])
+
+
+@pytest.mark.parametrize("n", [700, 5000, 20_000])
+@pytest.mark.parametrize("binades,threshold", [(0, 0.01), (8, 0.1), (40, 0.01), (29, 1e-18), (30, 1e-18), (30, 1e-17)])
+def test_score_ranking_whatever_the_spread_of_the_scores(n, binades, threshold):
+    """Scores spread evenly over 2^-binades .. 1; with a tiny threshold one large score is protected and the sum crosses
+    among scores far below it, beyond the binades that the first level of the descent tells apart."""
+    gen = torch.Generator().manual_seed(n + binades)
+    if threshold > 1e-6:
+        scores = torch.exp2(-binades * torch.rand(1, n, generator=gen)) * (1 + torch.rand(1, n, generator=gen)) / 2
+    else:
+        scores = 2.0 ** -binades * (1 + torch.rand(1, n, generator=gen))
+        scores[0, 0] = 1.25
+    p = binding.Params(num_seqs=1, num_q_heads=2, num_kv_heads=1, head_dim=64, window=4, sink=2, threshold=threshold,
+                       rank_mode=binding.RANK_SCORE, dtype=binding.DTYPE_F32, kv_tokens=n, k_strides=(0, 64, n * 64),
+                       v_strides=(0, 64, n * 64))
+    lengths = torch.zeros(1, dtype=torch.int32, device=DEV)
+    offsets = torch.zeros(2, dtype=torch.int64, device=DEV)
+    kept = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(binding.refree_workspace_size(p, n), dtype=torch.uint8, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    binding.refree_select_budget(p, scores.to(DEV), torch.tensor([n], dtype=torch.int32, device=DEV), n, lengths, offsets, kept, n, ws, st)
+    torch.cuda.synchronize()
+    want_b, want = _exact_rule(scores[0].tolist(), 2, 4, threshold)
+    assert int(st.item()) == 0 and int(lengths.item()) == want_b
+    assert kept[:want_b].cpu().tolist() == want
+
+
+def test_score_ranking_counts_scores_that_are_not_finite():
+    n = 3000
+    scores = torch.rand(1, n, generator=torch.Generator().manual_seed(3)) * 1e-3
+    scores[0, 1500] = float("inf")
+    p = binding.Params(num_seqs=1, num_q_heads=2, num_kv_heads=1, head_dim=64, window=4, sink=2, threshold=0.01,
+                       rank_mode=binding.RANK_SCORE, dtype=binding.DTYPE_F32, kv_tokens=n, k_strides=(0, 64, n * 64),
+                       v_strides=(0, 64, n * 64))
+    lengths, offsets = torch.zeros(1, dtype=torch.int32, device=DEV), torch.zeros(2, dtype=torch.int64, device=DEV)
+    kept = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(binding.refree_workspace_size(p, n), dtype=torch.uint8, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    binding.refree_select_budget(p, scores.to(DEV), torch.tensor([n], dtype=torch.int32, device=DEV), n, lengths, offsets, kept, n, ws, st)
+    torch.cuda.synchronize()
+    b = int(lengths.item())
+    assert int(st.item()) == binding.DEV_NONFINITE and 1500 in kept[:b].cpu().tolist()        # its key is the largest
+    assert torch.equal(kept[:b].cpu(), kept[:b].cpu().unique()) and b < n
