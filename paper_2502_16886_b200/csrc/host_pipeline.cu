@@ -1,10 +1,12 @@
-// The pass of Algorithm 1 for a run of layers whose caches live in HOST memory, pipelined
-// over three streams: while layer l is compressed, the inputs of layer l + 1 are on their way
-// to the device and the kept rows of layer l - 1 on their way back.  With the cache on the
-// host the copies dominate (two 64 MB arrays in, ~two out, per 32K layer, against 0.13 ms of
-// kernels), and PCIe carries both directions at once, so the pipeline costs about one
-// direction's copy time per layer instead of both in sequence.
+// The pass of Algorithm 1 for a run of layers whose caches live in HOST memory, pipelined over three streams.  With the cache
+// on the host the copies dominate (two 16 MB arrays in and nearly two out per layer of 8K positions, 1.2 ms of PCIe against
+// 0.1 ms of kernels), and PCIe carries both directions at once (55 GB/s alone, 50 each way together), so the pipeline aims at
+// one direction's time: a layer's K travels first and is scored, and its kept rows leave, while its V arrives.  Nothing
+// waits on the host but the row count: a kernel writes it into pinned memory behind the copy of K.  (The status word read into
+// pageable memory held the next layer's copies back: four layers of 8K positions 4.7 ms.  Rows written to host memory by the
+// copy kernel itself: 43 GB/s beside a copy in the other direction.)
 #include <algorithm>
+#include <mutex>
 
 #include "refree_internal.cuh"
 
@@ -15,9 +17,79 @@ struct Slot {
     char *q, *k, *v, *ko, *vo;
     int32_t *lengths, *status;
     int64_t *offsets;
-    cudaEvent_t in_done, comp_done, meta_done, out_done;
-    int32_t h_status;
 };
+
+// What a layer in flight tells the host.
+struct HostMeta { long long rows; int32_t status; };
+
+__global__ void host_meta_kernel(const int64_t *rows, const int32_t *status, volatile HostMeta *out)
+{
+    out->rows = *rows;
+    out->status = *status;
+}
+
+// Streams, events and the pinned words of one call.  Making them takes half a millisecond, so they are kept for the next call:
+// a call takes a set for itself and gives it back idle; a handful are kept, whatever the number of threads.
+struct HostPipe {
+    int dev = -1;
+    cudaStream_t in = nullptr, comp = nullptr, out = nullptr;
+    struct { cudaEvent_t k_in, v_in, k_done, v_done, out_done; } ev[2] = {};
+    HostMeta *meta = nullptr;                        // two, pinned
+
+    bool make()
+    {
+        if (cudaGetDevice(&dev) != cudaSuccess) return false;
+        for (cudaStream_t *st : {&in, &comp, &out})
+            if (cudaStreamCreateWithFlags(st, cudaStreamNonBlocking) != cudaSuccess) return false;
+        for (auto &e : ev)
+            for (cudaEvent_t *x : {&e.k_in, &e.v_in, &e.k_done, &e.v_done, &e.out_done})
+                if (cudaEventCreateWithFlags(x, cudaEventDisableTiming) != cudaSuccess) return false;
+        return cudaHostAlloc(reinterpret_cast<void **>(&meta), 2 * sizeof(HostMeta), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
+    }
+    void destroy()
+    {
+        for (auto &e : ev)
+            for (cudaEvent_t x : {e.k_in, e.v_in, e.k_done, e.v_done, e.out_done})
+                if (x) cudaEventDestroy(x);
+        for (cudaStream_t st : {in, comp, out})
+            if (st) cudaStreamDestroy(st);
+        if (meta) cudaFreeHost(meta);
+    }
+};
+constexpr int kKeptPipes = 4;
+std::mutex g_pipes_mutex;
+HostPipe g_pipes[kKeptPipes];                        // idle sets, of any device
+int g_num_pipes = 0;
+
+bool take_pipe(HostPipe &hp)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    {
+        std::lock_guard<std::mutex> hold(g_pipes_mutex);
+        for (int i = 0; i < g_num_pipes; ++i)
+            if (g_pipes[i].dev == dev) {
+                hp = g_pipes[i];
+                g_pipes[i] = g_pipes[--g_num_pipes];
+                return true;
+            }
+    }
+    if (hp.make()) return true;
+    hp.destroy();
+    return false;
+}
+
+void give_pipe(HostPipe &hp, bool sound)
+{
+    if (sound) {
+        std::lock_guard<std::mutex> hold(g_pipes_mutex);
+        if (g_num_pipes < kKeptPipes) {
+            g_pipes[g_num_pipes++] = hp;
+            return;
+        }
+    }
+    hp.destroy();
+}
 
 inline size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -99,80 +171,83 @@ refree_status refree_compress_layers_host(const refree_params *p, int32_t num_la
         slot[i].lengths = reinterpret_cast<int32_t *>(take(z.lengths));
         slot[i].offsets = reinterpret_cast<int64_t *>(take(z.offsets));
         slot[i].status = reinterpret_cast<int32_t *>(take(z.status));
-        slot[i].in_done = slot[i].comp_done = slot[i].meta_done = slot[i].out_done = nullptr;
-        slot[i].h_status = 0;
     }
+    st = check_kv_layout(p, slot[0].k, slot[0].v, true);
+    if (st != REFREE_OK) return st;
+    const Workspace lay = workspace_layout(*p, total_tokens);
+    const bool ranges = p->rank_mode == REFREE_RANK_POSITION || p->force_full;
+    HostPipe hp;
+    if (!take_pipe(hp)) return REFREE_ERR_CUDA;
 
-    cudaStream_t s_in = nullptr, s_comp = nullptr, s_out = nullptr;
-    bool ok = cudaStreamCreateWithFlags(&s_in, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&s_comp, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&s_out, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; i < 2 && ok; ++i)
-        ok = cudaEventCreateWithFlags(&slot[i].in_done, cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&slot[i].comp_done, cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&slot[i].meta_done, cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&slot[i].out_done, cudaEventDisableTiming) == cudaSuccess;
-
-    refree_status result = ok ? REFREE_OK : REFREE_ERR_CUDA;
-    auto cu = [&](cudaError_t e) { if (e != cudaSuccess && result == REFREE_OK) result = REFREE_ERR_CUDA; return e == cudaSuccess; };
-
-    // kept rows of layer j come back once its budgets are known on the host
-    auto finish = [&](int j) {
-        Slot &sl = slot[j & 1];
-        if (!cu(cudaEventSynchronize(sl.meta_done))) return;
-        if (sl.h_status & REFREE_DEV_TIMEOUT) { result = REFREE_ERR_TIMEOUT; return; }
-        if (sl.h_status & REFREE_DEV_CAPACITY) { result = REFREE_ERR_CAPACITY; return; }
-        if (sl.h_status & REFREE_DEV_NONFINITE) { result = REFREE_ERR_NONFINITE; return; }
-        const int64_t rows = offsets[j][U];
-        cu(cudaMemcpyAsync(k_out[j], sl.ko, (size_t)rows * row_bytes, cudaMemcpyDeviceToHost, s_out));
-        cu(cudaMemcpyAsync(v_out[j], sl.vo, (size_t)rows * row_bytes, cudaMemcpyDeviceToHost, s_out));
-        cu(cudaEventRecord(sl.out_done, s_out));
+    refree_status result = REFREE_OK;
+    bool sound = true;                               // no CUDA call has failed
+    auto cu = [&](cudaError_t e) {
+        if (e == cudaSuccess) return true;
+        sound = false;
+        if (result == REFREE_OK) result = REFREE_ERR_CUDA;
+        return false;
     };
 
-    if (result == REFREE_OK) {
-        cu(cudaMemcpyAsync(d_start, seq_start, p->num_seqs * sizeof(int32_t), cudaMemcpyHostToDevice, s_in));
-        cu(cudaMemcpyAsync(d_len, seq_len, p->num_seqs * sizeof(int32_t), cudaMemcpyHostToDevice, s_in));
-    }
-    int finished = 0;
-    for (int l = 0; l < num_layers && result == REFREE_OK; ++l) {
-        Slot &sl = slot[l & 1];
+    // layer l: its copies in, its kernels
+    auto begin = [&](int l) {
+        const Slot &sl = slot[l & 1];
+        auto &ev = hp.ev[l & 1];
         // inputs of the slot are free once layer l - 2 has been compressed
-        if (l >= 2) cu(cudaStreamWaitEvent(s_in, sl.comp_done, 0));
-        cu(cudaMemcpyAsync(sl.q, q_win[l], q_bytes, cudaMemcpyHostToDevice, s_in));
-        cu(cudaMemcpyAsync(sl.k, k[l], kv_bytes, cudaMemcpyHostToDevice, s_in));
-        cu(cudaMemcpyAsync(sl.v, v[l], kv_bytes, cudaMemcpyHostToDevice, s_in));
-        cu(cudaEventRecord(sl.in_done, s_in));
+        if (l >= 2) cu(cudaStreamWaitEvent(hp.in, ev.v_done, 0));
+        cu(cudaMemcpyAsync(sl.q, q_win[l], q_bytes, cudaMemcpyHostToDevice, hp.in));
+        cu(cudaMemcpyAsync(sl.k, k[l], kv_bytes, cudaMemcpyHostToDevice, hp.in));
+        cu(cudaEventRecord(ev.k_in, hp.in));
+        cu(cudaMemcpyAsync(sl.v, v[l], kv_bytes, cudaMemcpyHostToDevice, hp.in));
+        cu(cudaEventRecord(ev.v_in, hp.in));
         // outputs of the slot are free once the rows of layer l - 2 have left
-        cu(cudaStreamWaitEvent(s_comp, sl.in_done, 0));
-        if (l >= 2) cu(cudaStreamWaitEvent(s_comp, sl.out_done, 0));
-        cu(cudaMemsetAsync(sl.status, 0, sizeof(int32_t), s_comp));
-        if (result != REFREE_OK) break;
-        st = refree_compress_layer(p, sl.q, sl.k, sl.v, d_start, d_len, total_tokens, sl.ko, sl.vo, capacity_rows,
-                                   sl.lengths, sl.offsets, nullptr, nullptr, d_ws, z.ws, sl.status, s_comp);
-        if (st != REFREE_OK) { result = st; break; }
-        cu(cudaEventRecord(sl.comp_done, s_comp));
-        cu(cudaStreamWaitEvent(s_out, sl.comp_done, 0));
-        cu(cudaMemcpyAsync(lengths[l], sl.lengths, U * sizeof(int32_t), cudaMemcpyDeviceToHost, s_out));
-        cu(cudaMemcpyAsync(offsets[l], sl.offsets, (U + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s_out));
-        cu(cudaMemcpyAsync(&sl.h_status, sl.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s_out));
-        cu(cudaEventRecord(sl.meta_done, s_out));
-        if (l >= 1 && result == REFREE_OK) { finish(l - 1); finished = l; }
+        cu(cudaStreamWaitEvent(hp.comp, ev.k_in, 0));
+        if (l >= 2) cu(cudaStreamWaitEvent(hp.comp, ev.out_done, 0));
+        cu(cudaMemsetAsync(sl.status, 0, sizeof(int32_t), hp.comp));
+        if (result != REFREE_OK) return;
+        CompactJob job = {};
+        if (!cu(enqueue_selection(*p, sl.q, sl.k, sl.v, d_start, d_len, total_tokens, sl.ko, nullptr, capacity_rows, sl.lengths,
+                                  sl.offsets, nullptr, nullptr, d_ws, lay, sl.status, hp.comp, job))) return;
+        if (!cu(launch_compact(*p, job, d_start, d_len, ranges, capacity_rows, sl.status, hp.comp))) return;
+        host_meta_kernel<<<1, 1, 0, hp.comp>>>(sl.offsets + U, sl.status, hp.meta + (l & 1));
+        count_launches(1);
+        if (!cu(cudaGetLastError())) return;
+        cu(cudaEventRecord(ev.k_done, hp.comp));
+        cu(cudaStreamWaitEvent(hp.comp, ev.v_in, 0));
+        job.k_out[0] = nullptr;
+        job.v_out[0] = sl.vo;
+        if (!cu(launch_compact(*p, job, d_start, d_len, ranges, capacity_rows, sl.status, hp.comp))) return;
+        cu(cudaEventRecord(ev.v_done, hp.comp));
+    };
+    // kept rows of layer j come back once their number is known on the host
+    auto finish = [&](int j) {
+        const Slot &sl = slot[j & 1];
+        auto &ev = hp.ev[j & 1];
+        if (!cu(cudaEventSynchronize(ev.k_done))) return;
+        const HostMeta m = hp.meta[j & 1];
+        cu(cudaStreamWaitEvent(hp.out, ev.k_done, 0));
+        cu(cudaMemcpyAsync(lengths[j], sl.lengths, U * sizeof(int32_t), cudaMemcpyDeviceToHost, hp.out));
+        cu(cudaMemcpyAsync(offsets[j], sl.offsets, (U + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, hp.out));
+        if (m.status & REFREE_DEV_TIMEOUT) { result = REFREE_ERR_TIMEOUT; return; }
+        if (m.status & REFREE_DEV_CAPACITY) { result = REFREE_ERR_CAPACITY; return; }
+        if (m.status & REFREE_DEV_NONFINITE) { result = REFREE_ERR_NONFINITE; return; }
+        cu(cudaMemcpyAsync(k_out[j], sl.ko, (size_t)m.rows * row_bytes, cudaMemcpyDeviceToHost, hp.out));
+        cu(cudaStreamWaitEvent(hp.out, ev.v_done, 0));
+        cu(cudaMemcpyAsync(v_out[j], sl.vo, (size_t)m.rows * row_bytes, cudaMemcpyDeviceToHost, hp.out));
+        cu(cudaEventRecord(ev.out_done, hp.out));
+    };
+
+    cu(cudaMemcpyAsync(d_start, seq_start, p->num_seqs * sizeof(int32_t), cudaMemcpyHostToDevice, hp.in));
+    cu(cudaMemcpyAsync(d_len, seq_len, p->num_seqs * sizeof(int32_t), cudaMemcpyHostToDevice, hp.in));
+    for (int l = 0; l <= num_layers && result == REFREE_OK; ++l) {
+        if (l < num_layers) begin(l);
+        if (l >= 1 && result == REFREE_OK) finish(l - 1);
     }
-    if (result == REFREE_OK && finished < num_layers) finish(num_layers - 1);
 
     // leave nothing in flight, whatever happened
-    if (s_in) cudaStreamSynchronize(s_in);
-    if (s_comp) cudaStreamSynchronize(s_comp);
-    if (s_out) { if (cudaStreamSynchronize(s_out) != cudaSuccess && result == REFREE_OK) result = REFREE_ERR_CUDA; }
-    for (int i = 0; i < 2; ++i) {
-        if (slot[i].in_done) cudaEventDestroy(slot[i].in_done);
-        if (slot[i].comp_done) cudaEventDestroy(slot[i].comp_done);
-        if (slot[i].meta_done) cudaEventDestroy(slot[i].meta_done);
-        if (slot[i].out_done) cudaEventDestroy(slot[i].out_done);
-    }
-    if (s_in) cudaStreamDestroy(s_in);
-    if (s_comp) cudaStreamDestroy(s_comp);
-    if (s_out) cudaStreamDestroy(s_out);
+    cu(cudaStreamSynchronize(hp.in));
+    cu(cudaStreamSynchronize(hp.comp));
+    cu(cudaStreamSynchronize(hp.out));
+    give_pipe(hp, sound);
     return result;
 }
 

@@ -1,7 +1,8 @@
-"""Sizes at which the short-call kernels, the score ranking and the single-row stream can go wrong: edges of tiles and row
-chunks, spreads of the scores, layers that share a warp."""
+"""Sizes at which the short-call kernels, the score ranking, the single-row stream and the host pipeline can go wrong: edges
+of tiles and row chunks, spreads of the scores, layers that share a warp, threads that share the pipelines."""
 import dataclasses
 import math
+import threading
 from fractions import Fraction
 
 import numpy as np
@@ -110,3 +111,47 @@ def test_score_ranking_counts_scores_that_are_not_finite():
     b = int(lengths.item())
     assert int(st.item()) == binding.DEV_NONFINITE and 1500 in kept[:b].cpu().tolist()        # its key is the largest
     assert torch.equal(kept[:b].cpu(), kept[:b].cpu().unique()) and b < n
+
+
+def _host_run(cfg, lays, p, cap, rounds, out):
+    try:
+        total, units = lays[0].total_tokens, p.num_seqs * p.num_kv_heads
+        arena = torch.empty(binding.refree_host_pipeline_arena_size(p, total, lays[0].k.numel(), cap), dtype=torch.uint8, device=DEV)
+        for _ in range(rounds):
+            ko = [torch.zeros(cap, p.head_dim, dtype=lays[0].k.dtype).pin_memory() for _ in lays]
+            vo = [torch.zeros_like(t).pin_memory() for t in ko]
+            ln = [torch.zeros(units, dtype=torch.int32) for _ in lays]
+            of = [torch.zeros(units + 1, dtype=torch.int64) for _ in lays]
+            rc = binding.refree_compress_layers_host(p, [l.q_win for l in lays], [l.k for l in lays], [l.v for l in lays], lays[0].seq_start,
+                                                     lays[0].seq_len, total, ko, vo, cap, ln, of, arena, check=False)
+            out.append((rc, ko, vo, ln, of))
+    except Exception as e:                                               # (shown by the test)
+        out.append(e)
+
+
+def test_host_pipelines_of_several_threads_and_after_an_error():
+    """Threads take pipelines of their own; one that ended with an error serves the next call."""
+    cfg = cfg_like(window=16, dtype="bf16", head_dim=128, num_q_heads=8, num_kv_heads=2)
+    lays = [workloads.make_layer(cfg, l, seq_lens=[900, 1, 333]) for l in range(3)]
+    p = binding.params_for(cfg, lays[0], threshold=0.05)
+    cap = p.num_kv_heads * lays[0].total_tokens
+    refs = [binding.compress_layer(p, *[t.to(DEV) for t in (l.q_win, l.k, l.v, l.seq_start, l.seq_len)], l.total_tokens) for l in lays]
+    torch.cuda.synchronize()
+    short = []
+    _host_run(cfg, lays, p, 40, 1, short)
+    assert short[0][0] == binding.ERR_CAPACITY
+    outs = [[] for _ in range(6)]
+    threads = [threading.Thread(target=_host_run, args=(cfg, lays, p, cap, 3, o)) for o in outs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for o in outs:
+        assert len(o) == 3
+        for rc, ko, vo, ln, of in o:
+            assert rc == 0
+            for ref, k, v, n, f in zip(refs, ko, vo, ln, of):
+                rows = int(f[-1])
+                assert torch.equal(n, ref.lengths.cpu().reshape(-1)) and torch.equal(f, ref.offsets.cpu())
+                assert torch.equal(parity.bits(k[:rows]), parity.bits(ref.k_out[:rows].cpu()))
+                assert torch.equal(parity.bits(v[:rows]), parity.bits(ref.v_out[:rows].cpu()))
