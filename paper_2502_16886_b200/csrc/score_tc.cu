@@ -663,12 +663,12 @@ __device__ inline void epilogue_pass1(const TcArgs &a, TcSmemTail &tl, uint32_t 
     // running reference and sum of this lane's rows (row blocks group and group + 2) over its half of the columns
     float cref[2] = {-INFINITY, -INFINITY}, zsum[2] = {0.f, 0.f};
     int rmod[2];
-    bool rvalid[2];
+    bool rows_here[2];                           // a warp without rows of the unit hands its products back unread
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        const int row = (group + 2 * j) * kTile + lane_base + lane;
-        rmod[j] = row % w;                       // offset of the row's query inside the window
-        rvalid[j] = row < sh.R;
+        const int row0 = (group + 2 * j) * kTile + lane_base;
+        rmod[j] = (row0 + lane) % w;             // offset of the row's query inside the window
+        rows_here[j] = row0 < sh.R;
     }
     for (;;) {
         const ItemInfo *inf = &tl.info[es.icount++ & (kInfoRing - 1)];
@@ -681,6 +681,11 @@ __device__ inline void epilogue_pass1(const TcArgs &a, TcSmemTail &tl, uint32_t 
             if (!mbar_wait(&tl.p1_full[acc], (cnt >> 1) & 1u, &tl.abort_flag)) return;
             ++cnt;
             tc_fence_after();
+            if (j == 0) { flags = inf->flags; tile_start = inf->tile * kTile; n = inf->n; rec = inf->ib; }   // valid once a product of the item is
+            if (!rows_here[j]) {
+                release_acc(&tl.p1_empty[acc], lane);
+                continue;
+            }
             const uint32_t taddr = tmem_base + acc * 128u + (uint32_t)(half * 64) + ((uint32_t)lane_base << 16);
             uint32_t ra[32], rb2[32];
             tmem_ld_issue(taddr, ra);
@@ -689,16 +694,11 @@ __device__ inline void epilogue_pass1(const TcArgs &a, TcSmemTail &tl, uint32_t 
             tmem_ld_wait(rb2);
             // the logits are in registers: the accumulator goes back to the MMA warp before any arithmetic
             release_acc(&tl.p1_empty[acc], lane);
-            if (j == 0) { flags = inf->flags; tile_start = inf->tile * kTile; n = inf->n; rec = inf->ib; }   // valid once a product of the item is
             const bool full = tile_start + kTile <= n - w + 1;      // tile wholly before the window
-            int limit = kTile;                                  // visible positions of the tile: [0, limit)
-            if (!full) {
-                limit = n - w + rmod[j] - tile_start + 1;           // up to this row's own position
-                limit = rvalid[j] ? max(0, min(kTile, limit)) : 0;
-            } else if (!rvalid[j]) {
-                limit = 0;
-            }
-            limit = max(0, min(64, limit - half * 64));         // inside this warp's columns
+            // visible positions of the tile, [0, limit), up to this row's own position, inside this warp's columns.  (Lanes past the
+            // unit's rows go along with the others: what they add up is never stored.)
+            int limit = full ? kTile : n - w + rmod[j] - tile_start + 1;
+            limit = max(0, min(64, limit - half * 64));
             const bool uniform = __all_sync(0xffffffffu, limit == 64);
             bool need_max = (cref[j] == -INFINITY) && limit > 0;
             float zt = 0.f;
