@@ -246,23 +246,6 @@ struct StageSlot {
     float sum[4][kTile];                      // partial column sums (share = product * 2 + half of its columns)
 };
 
-struct TcSmemTail {
-    uint64_t k_full[4], k_empty[4], q_full, q_empty, epi_bar;
-    uint64_t p1_full[4], p1_empty[4];         // pass 1: accumulator (group * 2 + slot), 128 tensor-memory columns each
-    uint64_t p2_full[2], p2_empty[2];         // pass 2: accumulators of 256 columns, one per group of eight warps
-    uint64_t chunk_ready[kStageSlots];        // pass 2: every share of a tile has been staged
-    uint64_t stage_free[kStageSlots];         // pass 2: the finishing warp has read the slot
-    uint64_t c_full[kMaxCopySlots];           // row copy: a piece has landed in its slot
-    uint32_t tmem_base;
-    int abort_flag;
-    int rule_n;                               // units waiting in rule_unit / rule_max
-    int rule_unit[kRuleList];
-    uint32_t rule_max[kRuleList];             // bit pattern of the unit's largest score
-    BlockRuleShared<kThreadsTc> rule;
-    alignas(16) ItemInfo info[kInfoRing];
-    alignas(16) float lse[kMaxRowsTc];        // pass 2: log2-sum-exp of the unit's rows
-};
-
 // Per-sequence tables of the CTA behind the tail, sized by the number of sequences:
 // pack[B + 1], tiles[B + 1] (running sums of lengths and of tiles), len[B], start[B], ne[B + 1] (non-empty
 // sequences before each).
@@ -360,19 +343,76 @@ __device__ inline int group_range_begin(const Split &sp, const SeqView &sv, int 
     const int l = q / sp.ctas;
     return l * sp.items + range_begin(sp, sv, B, q - l * sp.ctas);
 }
-// The ranges and items of this CTA in a pass over a group: items [first, first + count), ranges from `q` on.
-struct Share { int q, first, count; };
-__device__ inline Share cta_share(const Split &sp, const SeqView &sv, int B, int layers)
+// The ranges and items of this CTA in a pass over a group: items [first, first + count), ranges from `q` on; the first of those
+// ends before item `first_end`.
+struct Share { int q, first, count, first_end; };
+// What a CTA does, found by one warp behind the sequence tables and shared: the lanes look up the range boundaries side by
+// side, and the unit that pass 2 begins with (its last item's) and the ranges that hold its records.  Every warp by itself, one
+// boundary after the other, took 2.2 us at the head of every launch.  (With the first launch of a call chained to what is
+// ahead of it, us: four layers one by one of 4K positions, 128 rows 162 -> 144, of 2K, 256 rows 159 -> 144; 16 layers of 8K as
+// a run 388 -> 378.)
+struct Plan {
+    Split sp;
+    Share a, b;                               // pass 1, pass 2
+    int b_layer, b_unit, b_ib, b_ntiles, b_tile, b_clo, b_chi;
+};
+__device__ inline void make_plan(Plan &plan, const SeqView &sv, int B, int Hkv, int split_ctas, int layers_a, int layers_b)
 {
-    Share sh = {0, 0, 0};
-    const int Q = layers * sp.ctas, ctas = min((int)gridDim.x, Q);
-    if ((int)blockIdx.x < ctas && sp.items > 0) {
-        sh.q = (int)((int64_t)blockIdx.x * Q / ctas);
-        sh.first = group_range_begin(sp, sv, B, sh.q);
-        sh.count = group_range_begin(sp, sv, B, (int)((int64_t)(blockIdx.x + 1) * Q / ctas)) - sh.first;
+    const int lane = threadIdx.x & 31;
+    const Split sp = make_split(sv, B, Hkv, split_ctas);
+    // lanes 0 to 2: first, next and last boundary of pass 1; 3 to 5: of pass 2
+    const int layers = lane < 3 ? layers_a : layers_b, Q = layers * sp.ctas, ctas = min((int)gridDim.x, Q);
+    const bool on = lane < 6 && (int)blockIdx.x < ctas && sp.items > 0;
+    int q = 0, x = 0;
+    if (on) {
+        const int which = lane < 3 ? lane : lane - 3;
+        q = (int)div_nonneg((int64_t)(blockIdx.x + (which == 2 ? 1 : 0)) * Q, ctas) + (which == 1 ? 1 : 0);
+        x = group_range_begin(sp, sv, B, q);
     }
-    return sh;
+    Share sh[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        sh[i].q = __shfl_sync(0xffffffffu, q, 3 * i);
+        sh[i].first = __shfl_sync(0xffffffffu, x, 3 * i);
+        sh[i].first_end = __shfl_sync(0xffffffffu, x, 3 * i + 1);
+        sh[i].count = __shfl_sync(0xffffffffu, x, 3 * i + 2) - sh[i].first;
+    }
+    int layer = 0, u = 0, ib = 0, nt = 1, tile = 0, c = 0;
+    if (sh[1].count > 0) {
+        const int last = sh[1].first + sh[1].count - 1;
+        layer = last / sp.items;
+        const ItemTc it = decode_item_tc(sv, B, Hkv, last - layer * sp.items);
+        u = it.s * Hkv + it.g;
+        ib = sv.tiles[it.s] * Hkv + it.g * it.ntiles;
+        nt = it.ntiles;
+        tile = it.tile;
+        c = range_of_item(sp, sv, lane == 0 ? ib : ib + nt - 1, u);
+    }
+    const int chi = __shfl_sync(0xffffffffu, c, 1);
+    if (lane == 0) {
+        plan.sp = sp;
+        plan.a = sh[0]; plan.b = sh[1];
+        plan.b_layer = layer; plan.b_unit = u; plan.b_ib = ib; plan.b_ntiles = nt; plan.b_tile = tile; plan.b_clo = c; plan.b_chi = chi;
+    }
 }
+struct TcSmemTail {
+    uint64_t k_full[4], k_empty[4], q_full, q_empty, epi_bar;
+    uint64_t p1_full[4], p1_empty[4];         // pass 1: accumulator (group * 2 + slot), 128 tensor-memory columns each
+    uint64_t p2_full[2], p2_empty[2];         // pass 2: accumulators of 256 columns, one per group of eight warps
+    uint64_t chunk_ready[kStageSlots];        // pass 2: every share of a tile has been staged
+    uint64_t stage_free[kStageSlots];         // pass 2: the finishing warp has read the slot
+    uint64_t c_full[kMaxCopySlots];           // row copy: a piece has landed in its slot
+    uint32_t tmem_base;
+    int abort_flag;
+    Plan plan;
+    int rule_n;                               // units waiting in rule_unit / rule_max
+    int rule_unit[kRuleList];
+    uint32_t rule_max[kRuleList];             // bit pattern of the unit's largest score
+    BlockRuleShared<kThreadsTc> rule;
+    alignas(16) ItemInfo info[kInfoRing];
+    alignas(16) float lse[kMaxRowsTc];        // pass 2: log2-sum-exp of the unit's rows
+};
+
 // Pass 1 leaves one record per (range, unit, half of a tile's columns); record of range c and unit u of layer l.
 __device__ inline int record_index(int l, int c, int u, int U) { return l * (kMaxCtas + U) + c + u; }
 
@@ -395,7 +435,7 @@ struct TcArgs {
     Cut *sel_cuts;             // [units]
     uint32_t *tickets;         // [2 units] tiles finished per unit, then the unit's largest score; zero when the launch begins
     uint32_t *tickets_next;    // [2 units] those of the launch that follows, cleared by this one
-    int dependent;             // launched with programmatic stream serialization: wait for the launch before
+    int dependent;             // launched with programmatic stream serialization: 1, behind another launch of the call; 2, its first
     TcCopyJob cj;          // rows of earlier layers to move while these are scored (nslots == 0: none)
 };
 struct TcMaps {
@@ -442,7 +482,7 @@ __device__ inline void producer_loop(const TcArgs &a, const TcMaps &maps,
     if (PASS1) asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
     else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     bool ok = true;
-    int q = share.q - 1, range_end = item0, last_u = -1;     // pass 1: the range of item x, and the item it ends at
+    int q = share.q, range_end = share.first_end, last_u = -1;      // pass 1: the range of item x, and the item it ends at
     for (int x = PASS1 ? item0 : item1 - 1; ok && x >= item0 && x < item1;) {
         const int layer = x / sp.items;
         const ItemTc it = decode_item_tc(sv, B, Hkv, x - layer * sp.items);
@@ -784,13 +824,11 @@ __device__ inline float col_product(int nch, uint32_t taddr, uint64_t *empty_bar
 
 // L[row] = log2 sum over the row of 2^y for the rows of unit u of a layer, merged from the (reference, sum) pairs that
 // pass 1 left per (range, unit, column half), in ascending record order (the same in every CTA that needs the unit).
-// Called by all epilogue threads; `ib` = index of the unit's first item in its layer, `ts` = its tiles.
-__device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, const SeqView &sv, const Split &sp, int layer, int u, int ib,
-                                      int ts, uint32_t &ephase)
+// Called by all epilogue threads; [c_lo, c_hi] = the ranges that hold the unit's items.
+__device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, int layer, int u, int c_lo, int c_hi, uint32_t &ephase)
 {
     const TcShape &sh = a.sh;
     const int tid = threadIdx.x;
-    const int c_lo = range_of_item(sp, sv, ib, u), c_hi = range_of_item(sp, sv, ib + ts - 1, u);
     // two threads per row when there are enough threads: even and odd records, then one exchange
     const int per_row = 2 * sh.R <= kEpiWarps * 32 ? 2 : 1;
     const int r = tid / per_row, sub = tid % per_row;
@@ -866,12 +904,21 @@ __device__ inline void epilogue_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
             // products.  The unit is looked up in the sequence tables, not in the item's record, which a warp
             // that takes none of the item's products has no barrier to wait for.  The normalisers do not wait
             // for the tile either: the partials come from the row pass, not from anything this pass loads.
-            const int x = item0 + (nitems - 1 - item), layer = x / sp.items;
-            const ItemTc it = decode_item_tc(sv, a.p.num_seqs, Hkv, x - layer * sp.items);
-            if (item > 0 && !epi_sync(tl, es.ephase)) return;      // nobody still reads the previous unit's L
-            if (!merge_unit_lse(a, tl, sv, sp, layer, it.s * Hkv + it.g, sv.tiles[it.s] * Hkv + it.g * it.ntiles, it.ntiles, es.ephase))
-                return;
-            next_change = item + it.tile + 1;                      // the unit's earlier tiles follow
+            const Plan &pl = tl.plan;
+            int layer = pl.b_layer, u = pl.b_unit, tile = pl.b_tile, c_lo = pl.b_clo, c_hi = pl.b_chi;
+            if (item > 0) {
+                const int x = item0 + (nitems - 1 - item);
+                layer = x / sp.items;
+                const ItemTc it = decode_item_tc(sv, a.p.num_seqs, Hkv, x - layer * sp.items);
+                const int ib = sv.tiles[it.s] * Hkv + it.g * it.ntiles;
+                u = it.s * Hkv + it.g;
+                tile = it.tile;
+                c_lo = range_of_item(sp, sv, ib, u);
+                c_hi = range_of_item(sp, sv, ib + it.ntiles - 1, u);
+                if (!epi_sync(tl, es.ephase)) return;              // nobody still reads the previous unit's L
+            }
+            if (!merge_unit_lse(a, tl, layer, u, c_lo, c_hi, es.ephase)) return;
+            next_change = item + tile + 1;                         // the unit's earlier tiles follow
         }
         for (int cb = 0; cb < sh.cblocks; ++cb) {
             const uint32_t j = (uint32_t)item * (uint32_t)sh.cblocks + (uint32_t)cb;      // product index in this pass
@@ -1200,6 +1247,10 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
         tl.rule_n = 0;
         fence_barrier_init();
     }
+    SeqView sv;
+    sv.pack = t_pack; sv.tiles = t_tiles; sv.len = t_len; sv.start = t_start; sv.ne = t_ne;
+    // the first launch of a call reads nothing before what is ahead of it on the stream has completed
+    if (a.dependent == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int t = threadIdx.x; t < B; t += kThreadsTc) t_start[t] = a.seq_start[t];
     if (warp == 1) {                             // running sums over the sequences, 32 at a time
         int32_t pa = 0, ti = 0, ne = 0;
@@ -1219,20 +1270,17 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
             ne += __popc(nonempty);
         }
         if (lane == 0) { t_pack[B] = pa; t_tiles[B] = ti; t_ne[B] = ne; }
+        __syncwarp();
+        // a layer's items in min(SMs, items) ranges, so that no range is empty
+        make_plan(tl.plan, sv, B, a.p.num_kv_heads, a.split_ctas, P1 ? a.layers_a : 0, P2 ? a.layers_b : 0);
     }
     if (warp == kEpiWarps + 1) tmem_alloc(&tl.tmem_base, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tl.tmem_base;
-    SeqView sv;
-    sv.pack = t_pack; sv.tiles = t_tiles; sv.len = t_len; sv.start = t_start; sv.ne = t_ne;
-
-    // the layer's items in min(SMs, items) ranges, so that no range is empty
-    const Split sp = make_split(sv, B, a.p.num_kv_heads, a.split_ctas);
-    Share sh_a = {0, 0, 0}, sh_b = {0, 0, 0};    // pass 1, pass 2
-    if (P2) sh_b = cta_share(sp, sv, B, a.layers_b);
-    if (P1) sh_a = P2 && a.layers_a == a.layers_b ? sh_b : cta_share(sp, sv, B, a.layers_a);
+    const Split sp = tl.plan.sp;
+    const Share sh_a = tl.plan.a, sh_b = tl.plan.b;       // pass 1, pass 2
     const int na = sh_a.count, b0 = sh_b.first, nb = sh_b.count;
 
     // A run of layers: the launch that follows may put a CTA on an SM as soon as this one's has left it (programmatic
@@ -1240,7 +1288,7 @@ score_tc_kernel(const __grid_constant__ TcMaps maps_a, const __grid_constant__ T
     // its setup, and the loads of Q and K and the products on them, which are the caller's inputs.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool inputs_only = warp == kEpiWarps || warp == kEpiWarps + 1;
-    if (a.dependent && !inputs_only) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (a.dependent == 1 && !inputs_only) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0 && !inputs_only) {
         const int t0 = threadIdx.x < kEpiWarps * 32 ? threadIdx.x : threadIdx.x - 64;
         if (P1 && a.tickets_next)
@@ -1500,13 +1548,12 @@ cudaError_t launch_score_tc_pipe(const refree_params &p, const TcGroup *begin, c
     a.cj.piece_rows = piece_rows;
     const size_t smem = smem_bytes(sh, p.num_seqs, a.cj.nslots, piece_rows, p.num_seqs * p.num_kv_heads * a.cj.layers);
     if (smem > kSmemLimit) return cudaErrorInvalidValue;
-    // Launches of a run after the first may start while the one before drains (unless the stream is not to be chained):
-    // their CTAs set themselves up and then wait (griddepcontrol.wait) until that launch has completed and its results are
-    // visible.
-    const bool chain = st.chain && !first;
-    a.dependent = chain ? 1 : 0;
+    // A launch may start while the one before drains (unless the stream is not to be chained): its CTAs set themselves up and
+    // then wait (griddepcontrol.wait) until that launch has completed and its results are visible.  The first one of a call
+    // waits before it reads anything, since what is ahead of it may still be writing Q and K.
+    a.dependent = !st.chain ? 0 : first ? 2 : 1;
     auto *kern = begin && finish ? score_tc_kernel<3> : begin ? score_tc_kernel<1> : score_tc_kernel<2>;
-    e = launch_dependent(kern, dim3(ctas), dim3(kThreadsTc), smem, Stream(st.s, chain), maps[0], maps[1], a);
+    e = launch_dependent(kern, dim3(ctas), dim3(kThreadsTc), smem, st, maps[0], maps[1], a);
     if (e != cudaSuccess) return e;
     count_launches(1);
     return cudaGetLastError();
