@@ -807,6 +807,10 @@ __device__ inline float col_product(int nch, uint32_t taddr, uint64_t *empty_bar
 {
     uint32_t b0[16], b1[16];
     float s0 = 0.f, s1 = 0.f;
+    if (nch == 0) {                                                 // none of the unit's rows
+        release_acc(empty_bar, lane);
+        return 0.f;
+    }
     tmem_ld_issue(taddr, b0);
     tmem_ld_wait(b0);
     for (int c = 0; c < nch; c += 2) {
@@ -892,7 +896,6 @@ __device__ inline void epilogue_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
     const int w = a.p.window, Hkv = a.p.num_kv_heads;
     const int pos_in_tile = lane_base + lane;
     const int c_width = sh.ncol >> 1, c_begin = half * c_width;     // this warp's columns of a product
-    const bool exact = sh.cblocks * sh.ncol == sh.R;               // no padding columns in the products
     const uint32_t taddr = tmem_base + (uint32_t)group * 256u + (uint32_t)c_begin + ((uint32_t)lane_base << 16);
     const int slot_shift = 31 - __clz(sh.slots);
     uint32_t gcnt = 0;                                             // products this group has taken
@@ -929,12 +932,13 @@ __device__ inline void epilogue_pass2(const TcArgs &a, TcSmemTail &tl, StageSlot
             // the item's record is valid once one of its products is
             const int tile_start = inf->tile * kTile, n = inf->n;
             const int pos_gap = tile_start + pos_in_tile - (n - w);
+            // chunks with rows of the unit among this warp's columns (the last product is padded: 400 rows, whose products of 224
+            // went through the masked sums tile after tile, four layers of 8000 positions x 8 heads 196 us, 166 this way)
+            const int r0 = cb * sh.ncol + c_begin, nch = (max(0, min(c_width, sh.R - r0)) + 15) >> 4;
             // tile wholly before the window and wholly inside the sequence: every row sees every position
-            const bool full = tile_start + kTile <= n - w + 1 && exact;
-            const float part = full ? col_product<false>(c_width >> 4, taddr, &tl.p2_empty[group], lane, scale, tl.lse,
-                                                         cb * sh.ncol + c_begin, sh.R, w, pos_gap)
-                                    : col_product<true>(c_width >> 4, taddr, &tl.p2_empty[group], lane, scale, tl.lse,
-                                                        cb * sh.ncol + c_begin, sh.R, w, pos_gap);
+            const bool full = tile_start + kTile <= n - w + 1 && r0 + 16 * nch <= max(sh.R, r0);
+            const float part = full ? col_product<false>(nch, taddr, &tl.p2_empty[group], lane, scale, tl.lse, r0, sh.R, w, pos_gap)
+                                    : col_product<true>(nch, taddr, &tl.p2_empty[group], lane, scale, tl.lse, r0, sh.R, w, pos_gap);
             // the slot's previous tile has been read by the finishing warp
             const uint32_t slot = (uint32_t)item & (uint32_t)(sh.slots - 1);
             if (!mbar_wait(&tl.stage_free[slot], (((uint32_t)item >> slot_shift) & 1u) ^ 1u, &tl.abort_flag)) return;
