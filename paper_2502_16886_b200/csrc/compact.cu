@@ -205,23 +205,38 @@ compact_inplace_back_kernel(refree_params p, char *k, char *v, const int32_t *se
     __shared__ long long s_part[kThreads / 32];
     const int Hkv = p.num_kv_heads;
     const int u = blockIdx.x, s = u / Hkv, g = u % Hkv;
-    dependency_wait();
-    trigger_dependents();
     const int esz = p.dtype == REFREE_DTYPE_F32 ? 4 : 2;
     const int vec_per_row = (p.head_dim * esz) >> 4;
     const int vshift = 31 - __clz(vec_per_row);
-    const int n = max(seq_len[s], 0);
+    // Behind the selection of the same call everything but the budgets was complete before that began: tables and leading rows
+    // are read while it drains (a thread has one piece of K and of V where they are few).
+    if (!lengths) dependency_wait();
+    trigger_dependents();
+    const int n = max(seq_len[s], 0), lead = min(p.sink, n);
+    const int64_t tok0 = seq_start[s];
+    char *kb = k + ((int64_t)s * p.k_stride_seq + tok0 * p.k_stride_tok + (int64_t)g * p.k_stride_head) * esz;
+    char *vb = v + ((int64_t)s * p.v_stride_seq + tok0 * p.v_stride_tok + (int64_t)g * p.v_stride_head) * esz;
+    const int64_t k_tok = p.k_stride_tok * esz, v_tok = p.v_stride_tok * esz;
+    const bool few = lead << vshift <= kThreads, mine = few && (int)threadIdx.x < lead << vshift;
+    int4 kv = {}, vv = {};
+    auto load = [&](int e) {
+        const int row = e >> vshift, c = e & (vec_per_row - 1);
+        kv = __ldcg(reinterpret_cast<const int4 *>(kb + (int64_t)row * k_tok + c * 16));
+        vv = __ldcg(reinterpret_cast<const int4 *>(vb + (int64_t)row * v_tok + c * 16));
+    };
+    if (mine) load(threadIdx.x);
+    if (lengths) dependency_wait();
     int64_t off, b64;
     if (lengths) {
         // fused pass: budgets come straight from the selection, and the running sum is formed here
+        b64 = lengths[u];
         long long part = 0;
         for (int t = threadIdx.x; t < u; t += kThreads) part += lengths[t];
         for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
-        __syncthreads();
+        __syncthreads();                             // (and the leading rows have been read)
         off = 0;
         for (int wv = 0; wv < kThreads / 32; ++wv) off += s_part[wv];
-        b64 = lengths[u];
         if (threadIdx.x == 0) {
             offsets_out[u] = off;
             if (u == (int)gridDim.x - 1) offsets_out[u + 1] = off + b64;
@@ -229,32 +244,29 @@ compact_inplace_back_kernel(refree_params p, char *k, char *v, const int32_t *se
     } else {
         off = offsets[u];
         b64 = offsets[u + 1] - off;
+        __syncthreads();
     }
     if (off < 0 || b64 < 0 || b64 > n) {
         if (threadIdx.x == 0 && dev_status) atomicOr(dev_status, REFREE_DEV_CAPACITY);
         return;
     }
-    const int b = (int)b64, head = min(b, min(p.sink, n)), shift = n - b;
+    const int b = (int)b64, head = min(b, lead), shift = n - b;
     if (shift == 0 || head == 0) return;
-    const int64_t tok0 = seq_start[s];
-    char *kb = k + ((int64_t)s * p.k_stride_seq + tok0 * p.k_stride_tok + (int64_t)g * p.k_stride_head) * esz;
-    char *vb = v + ((int64_t)s * p.v_stride_seq + tok0 * p.v_stride_tok + (int64_t)g * p.v_stride_head) * esz;
-    const int64_t k_tok = p.k_stride_tok * esz, v_tok = p.v_stride_tok * esz;
     const int total_vec = head << vshift;
+    auto store = [&](int e) {
+        const int row = e >> vshift, c = e & (vec_per_row - 1);
+        *reinterpret_cast<int4 *>(kb + (int64_t)(row + shift) * k_tok + c * 16) = kv;
+        *reinterpret_cast<int4 *>(vb + (int64_t)(row + shift) * v_tok + c * 16) = vv;
+    };
+    if (few) {
+        if ((int)threadIdx.x < total_vec) store(threadIdx.x);
+        return;
+    }
     for (int c0 = (total_vec - 1) / kThreads * kThreads; c0 >= 0; c0 -= kThreads) {
         const int e = c0 + threadIdx.x;
-        const bool on = e < total_vec;
-        const int row = e >> vshift, c = e & (vec_per_row - 1);
-        int4 kv = {}, vv = {};
-        if (on) {
-            kv = __ldcg(reinterpret_cast<const int4 *>(kb + (int64_t)row * k_tok + c * 16));
-            vv = __ldcg(reinterpret_cast<const int4 *>(vb + (int64_t)row * v_tok + c * 16));
-        }
+        if (e < total_vec) load(e);
         __syncthreads();
-        if (on) {
-            *reinterpret_cast<int4 *>(kb + (int64_t)(row + shift) * k_tok + c * 16) = kv;
-            *reinterpret_cast<int4 *>(vb + (int64_t)(row + shift) * v_tok + c * 16) = vv;
-        }
+        if (e < total_vec) store(e);
     }
 }
 
