@@ -39,9 +39,6 @@ namespace cg = cooperative_groups;
 constexpr int kThreads = 1024;
 constexpr int kMaxCluster = 8;     // blocks of a thread-block cluster that share one unit in score ranking
 constexpr int kWarps = kThreads / 32;
-// Mean positions of a block of a cluster, at least (staged calls on four sequences of 260 to 5120 positions, 8 heads, four
-// layers, us: 1024 296, 2048 304, 4096, which leaves them one block each, 325).
-constexpr int kClusterPositions = 1024;
 constexpr int kTables = 8;         // register-resident score ranking: histograms of a block, one for every fourth warp
 constexpr int kBinades = 16, kCopies = 16;   // ... its first level: digits and counters of a digit (256 in all)
 typedef unsigned long long u64;
@@ -870,33 +867,42 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
     const int32_t *const lengths = out.lengths[blockIdx.z];
     int64_t *const offsets = out.offsets[blockIdx.z];
     int32_t *const kept_idx = out.kept[blockIdx.z];
-    dependency_wait();
     trigger_dependents();
+    // The selection before this launch triggered it after its own wait: lengths and scores were complete by then, and are read
+    // before the wait for the selection.
     const int n = max(seq_len[s], 0), chunk = blockIdx.x * kThreads;
     const bool ranges = p.rank_mode == REFREE_RANK_POSITION || p.force_full;
     // score ranking: a block beyond the end of its sequence has nothing to do (the grid is sized for the longest
     // sequence a call can hold)
-    if (blockIdx.x > 0 && !ranges && chunk >= n) return;
+    if (blockIdx.x > 0 && !ranges && chunk >= n) { dependency_wait(); return; }
+    const bool listed = kept_idx != nullptr && !ranges && chunk < n, layer = p.scope == REFREE_SCOPE_LAYER;
+    UnitView v;
+    uint32_t near[kPerThread] = {};                                    // one head: this thread's scores
+    if (listed) {
+        int pack = 0;
+        for (int t = lane; t < s; t += 32) pack += max(seq_len[t], 0);
+        pack = __reduce_add_sync(0xffffffffu, pack);
+        v.lead = min(p.sink, n);
+        v.w_eff = min(p.window, n);
+        if (v.lead + v.w_eff >= n) { v.lead = n; v.w_eff = 0; }
+        v.sc = scores + (int64_t)(layer ? 0 : g) * total_tokens + pack;
+        v.head_stride = total_tokens;
+        v.heads = layer ? Hkv : 1;
+        v.n = n;
+        if (v.heads == 1)
+#pragma unroll
+            for (int q = 0; q < kPerThread; ++q) near[q] = mag_bits(__ldcg(v.sc + min(chunk + q * kEmitThreads + (int)threadIdx.x, n - 1)));
+    }
+    dependency_wait();
     const Cut cut = cuts[u];
     const int b = cut.b;
     long long part = 0, before = 0;
     for (int t = threadIdx.x; t < u; t += kEmitThreads) part += lengths[t];
     // kept for sure (above the crossing key, or protected and inside the budget) / at the crossing key, of
     // which the cut.ties lowest positions are kept
-    const bool listed = kept_idx != nullptr && !ranges && chunk < n;
     unsigned int smask[kPerThread], tmask[kPerThread];                 // of this warp's positions chunk + q kEmitThreads + threadIdx.x
     if (listed) {
-        int pack = 0;
-        for (int t = lane; t < s; t += 32) pack += max(seq_len[t], 0);
-        pack = __reduce_add_sync(0xffffffffu, pack);
-        int lead = min(p.sink, n), w_eff = min(p.window, n);
-        if (lead + w_eff >= n) { lead = n; w_eff = 0; }
-        UnitView v;
-        const bool layer = p.scope == REFREE_SCOPE_LAYER;
-        v.sc = scores + (int64_t)(layer ? 0 : g) * total_tokens + pack;
-        v.head_stride = total_tokens;
-        v.heads = layer ? Hkv : 1;
-        v.n = n; v.lead = lead; v.w_eff = w_eff;
+        const int lead = v.lead, w_eff = v.w_eff;
         v.sbias = cut.sbias;
         // the key is loaded first, without a branch around it, so that a thread's loads are in flight together
         const bool one_head = v.heads == 1;
@@ -922,7 +928,10 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
         };
         u64 key[kPerThread];
 #pragma unroll
-        for (int q = 0; q < kPerThread; ++q) key[q] = key_of(chunk + q * kEmitThreads + (int)threadIdx.x);
+        for (int q = 0; q < kPerThread; ++q) {
+            const int i = chunk + q * kEmitThreads + (int)threadIdx.x;
+            key[q] = !one_head ? key_of(i) : i >= lead && i < n - w_eff ? (u64)near[q] << 32 : 0ull;
+        }
         // What the positions before the chunk contribute: left per run of kThreads positions by the kernel that chose
         // the budget when it held the unit in registers; otherwise every block counts them itself (the scores are in L2).
         if (chunk_counts && n <= counted_upto) {
@@ -1079,7 +1088,10 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
         int nblk = 1;
         if (p.rank_mode == REFREE_RANK_SCORE && !p.force_full) {
             const int64_t avg = total_tokens / std::max(1, p.num_seqs);
-            while (nblk < kMaxCluster && avg >= (int64_t)nblk * kClusterPositions) nblk *= 2;
+            // Blocks by the mean length (four layers one by one of 8 heads, us, with clusters of 1, 2, 4 and 8): 1100 positions 163,
+            // 186; 2100 -, 207, 209; 4100 -, -, 223, 235; 6000 -, -, 249, 259; staged calls on four sequences of 260 to 5120
+            // positions 325, 304, 296.
+            nblk = avg < 2048 ? 1 : avg < 8192 ? 4 : kMaxCluster;
             // One wave: a block takes an SM, and clusters leave some SMs of a group of them unused (16 units of 32K positions:
             // 61 us in clusters of eight, which came in two waves, 38 in clusters of four).
             // (But not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some
