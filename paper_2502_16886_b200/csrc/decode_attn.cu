@@ -78,17 +78,24 @@ __device__ inline int64_t unit_len(const DecArgs &a, int u)
     const int n = max(a.seq_len[u / a.p.num_kv_heads], 0);
     return max(0, min(a.lengths[u], n));
 }
+// The loads go out together, and the strides are divided by the constant head dimension: this is the head of every call's
+// chain of waits (a 64-bit division is a routine of some hundred instructions; both, 1.9 us before the first row was asked for).
+template <int D>
 __device__ inline void unit_rows(const DecArgs &a, int u, int64_t &lo_k, int64_t &lo_v, int64_t &len64)
 {
-    len64 = unit_len(a, u);
     if (!a.lengths) {
-        lo_k = lo_v = a.offsets[u];
+        const int64_t lo = a.offsets[u], hi = a.offsets[u + 1];
+        lo_k = lo_v = lo;
+        len64 = hi - lo;
         return;
     }
-    const int Hkv = a.p.num_kv_heads, s = u / Hkv, g = u % Hkv;
-    const int64_t first = (int64_t)a.seq_start[s] + (a.anchor_back ? max(a.seq_len[s], 0) - len64 : 0);
-    lo_k = ((int64_t)s * a.p.k_stride_seq + (int64_t)g * a.p.k_stride_head) / a.p.head_dim + first;
-    lo_v = ((int64_t)s * a.p.v_stride_seq + (int64_t)g * a.p.v_stride_head) / a.p.head_dim + first;
+    const int Hkv = a.p.num_kv_heads, s = u / Hkv, g = u - s * Hkv;
+    const int n0 = a.seq_len[s], b = a.lengths[u], start = a.seq_start[s];
+    const int n = max(n0, 0);
+    len64 = max(0, min(b, n));
+    const int64_t first = (int64_t)start + (a.anchor_back ? n - len64 : 0);
+    lo_k = (int64_t)((uint64_t)((int64_t)s * a.p.k_stride_seq + (int64_t)g * a.p.k_stride_head) / D) + first;
+    lo_v = (int64_t)((uint64_t)((int64_t)s * a.p.v_stride_seq + (int64_t)g * a.p.v_stride_head) / D) + first;
 }
 __device__ inline int clamp_len(const DecArgs &a, int64_t len64) { return (int)max((int64_t)0, min(len64, (int64_t)a.cap)); }
 
@@ -231,32 +238,51 @@ __device__ __host__ inline int native_col(int idx, int native)
 }
 
 // Merge the warps' (max, sum, O) through shared memory in warp order and store the block's
-// result: the final output when the unit has one block, a record otherwise.
-// sm: [NW][GP][D + 2] floats, then the block's own record [GP][D + 2] (cluster).
+// result: the final output when the unit has one block, a record otherwise.  What a warp counts is worked out once per head.
+// sm: [NW][GP][D + 2] floats, then the block's own record [GP][D + 2] (cluster), then the factors [GP][NW + 1].
 template <int D, int NW>
 __device__ inline void merge_and_store(const DecArgs &a, float *sm, int GP, int G, const Piece &pc)
 {
+    float *const fac = sm + (NW + 1) * GP * (D + 2);
     __syncthreads();
-    const int Hkv = a.p.num_kv_heads, s = pc.u / Hkv, g = pc.u % Hkv;
+    const int Hkv = a.p.num_kv_heads, s = pc.u / Hkv, g = pc.u - s * Hkv;
     float *recs = a.mode == kCluster ? sm + NW * GP * (D + 2) : a.part + (int64_t)pc.rec * G * (D + 2);
-    for (int e = threadIdx.x; e < G * (D + 2); e += 32 * NW) {
-        const int h = e / (D + 2), idx = e % (D + 2);
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) M = fmaxf(M, sm[(w * GP + h) * (D + 2) + D]);
-        float val = 0.f, L = 0.f;
+    if (threadIdx.x < G) {
+        const int h = threadIdx.x;
+        float m[NW], l[NW], M = -INFINITY, L = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
-            const float *rec = sm + (w * GP + h) * (D + 2);
-            const float f = rec[D] == -INFINITY ? 0.f : dec_ex2(rec[D] - M);
-            val += rec[idx < D ? idx : 0] * f;
-            L += rec[D + 1] * f;
+            m[w] = sm[(w * GP + h) * (D + 2) + D];
+            l[w] = sm[(w * GP + h) * (D + 2) + D + 1];
+            M = fmaxf(M, m[w]);
+        }
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const float f = m[w] == -INFINITY ? 0.f : dec_ex2(m[w] - M);
+            fac[h * (NW + 1) + w] = f;
+            L += l[w] * f;
+        }
+        fac[h * (NW + 1) + NW] = L;
+        if (pc.nblocks > 1) { recs[h * (D + 2) + D] = M; recs[h * (D + 2) + D + 1] = L; }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < G * (D / 2); e += 32 * NW) {
+        const int h = e / (D / 2), idx = 2 * (e % (D / 2));
+        float2 val = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const float2 x = *reinterpret_cast<const float2 *>(sm + (w * GP + h) * (D + 2) + idx);
+            const float f = fac[h * (NW + 1) + w];
+            val.x += x.x * f;
+            val.y += x.y * f;
         }
         if (pc.nblocks == 1) {
-            if (idx < D)
-                a.out[((int64_t)s * a.p.num_q_heads + g * G + h) * D + native_col(idx, a.native)] = L > 0.f ? val / L : 0.f;
+            const float L = fac[h * (NW + 1) + NW];
+            float *out = a.out + ((int64_t)s * a.p.num_q_heads + g * G + h) * D;
+            out[native_col(idx, a.native)] = L > 0.f ? val.x / L : 0.f;
+            out[native_col(idx + 1, a.native)] = L > 0.f ? val.y / L : 0.f;
         } else {
-            recs[e] = idx < D ? val : (idx == D ? M : L);
+            *reinterpret_cast<float2 *>(recs + h * (D + 2) + idx) = val;
         }
     }
 }
@@ -570,9 +596,9 @@ __device__ inline void decode_block(const DecArgs &a, float *dec_sm, Body body)
     int64_t lo_k = 0, lo_v = 0, len64 = 0;
     if (a.mode == kPlanned) {
         pc = make_plan(a, -(int)blockIdx.x - 1);
-        if (pc.u >= 0) unit_rows(a, pc.u, lo_k, lo_v, len64);
+        if (pc.u >= 0) unit_rows<D>(a, pc.u, lo_k, lo_v, len64);
     } else {
-        unit_rows(a, blockIdx.y, lo_k, lo_v, len64);
+        unit_rows<D>(a, blockIdx.y, lo_k, lo_v, len64);
         pc = unit_piece(a, blockIdx.y, blockIdx.x, clamp_len(a, len64));
     }
     pc.len = clamp_len(a, len64);
@@ -679,12 +705,15 @@ cudaError_t run_kernel(Kern kern, const DecArgs &a, dim3 grid, int warps, size_t
     return launch_dependent_cluster(kern, a.mode == kCluster ? a.blocks : 1, grid, dim3(32 * warps), smem, st, a);
 }
 
-// Shared memory: the warps' records, then the block's own (the staging ring of the mma form uses the space before).
+// Shared memory: the warps' records, then the block's own, then the merge's factors (the staging ring of the mma form uses the
+// space before).
+constexpr size_t record_smem(int D, int NW, int gp) { return (size_t)(NW + 1) * gp * (D + 2 + 1) * sizeof(float); }
+
 template <typename T, int D, int NW>
 cudaError_t run_lanes(const DecArgs &a, dim3 grid, int G, Stream st)
 {
     const int gp = G <= 4 ? 4 : (G <= 8 ? 8 : 16);
-    const size_t smem = (size_t)(NW + 1) * gp * (D + 2) * sizeof(float);
+    const size_t smem = record_smem(D, NW, gp);
     if (gp == 4) return run_kernel(decode_lanes_kernel<T, D, 4, NW>, a, grid, NW, smem, st);
     if (gp == 8) return run_kernel(decode_lanes_kernel<T, D, 8, NW>, a, grid, NW, smem, st);
     return run_kernel(decode_lanes_kernel<T, D, 16, NW>, a, grid, NW, smem, st);
@@ -694,7 +723,7 @@ template <int D, int NW>
 cudaError_t run_mma(const DecArgs &a, dim3 grid, int G, Stream st)
 {
     const size_t ring = (size_t)NW * kDecStages * 2 * 16 * D * 2 + (size_t)NW * kDecStages * sizeof(uint64_t);
-    const size_t smem = std::max(ring, (size_t)(NW + 1) * (G <= 8 ? 8 : 16) * (D + 2) * sizeof(float));
+    const size_t smem = std::max(ring, record_smem(D, NW, G <= 8 ? 8 : 16));
     if (G <= 8) return run_kernel(decode_mma_kernel<D, false, NW>, a, grid, NW, smem, st);
     return run_kernel(decode_mma_kernel<D, true, NW>, a, grid, NW, smem, st);
 }
@@ -721,17 +750,22 @@ int decode_shape(const refree_params &p, int64_t max_rows, bool mma, int &blocks
         blocks = (int)n;
         return kCluster;
     }
-    // Lengths are on the device; what the host has is the mean, if the caller says how many tokens the cache holds.  The
-    // plan costs 1 to 3 us a call (24 units of 5000 rows: 20.8 us, fixed 19.1) and pays where the longest sequence is far
-    // above the mean (8 heads, sequences of 20000, 2500, 1000 and 300 rows: 25.9 us, fixed 53.9; of 5000, 700, 300 and
-    // 100: 15.4 and 18.9), as long as a unit can have two pieces.
-    const int64_t few = max_rows * p.num_seqs / 3 / (p.k_stride_seq != 0 ? p.num_seqs : 1);   // kv_tokens is per sequence, or of all
-    if (2 * U <= std::min<int64_t>(sms, 2 * kPlanUnits) && p.num_seqs > 1 && p.kv_tokens > 0 && p.kv_tokens <= few) {
+    // about one block per SM (one wave: prologue and merge are paid once), at least a 16-row block per warp
+    const int64_t fixed = std::max<int64_t>(1, std::min<int64_t>(sms / U, (max_rows + 127) / 128));
+    // Lengths are on the device; what the host has is their sum, if the caller says how many tokens the cache holds.  By the
+    // fixed cut the longest unit's blocks set the time; by the plan the rows spread over the SMs, less what its rounding
+    // wastes, and a call takes 2 us longer, as long as some 200 rows of a block (bf16; fp32 rows take five times as long), or 5 us
+    // with fewer than eight units, whose records are many.  Us a call, fixed and planned: 8 heads, sequences of 20000, 10000 and
+    // 5000 rows 42.2 and 30.4; of 9000 and 5000 19.5 and 19.3; 13 of 100 to 9000 86.6 and 53.2; 4 heads, eight of 2531 to 16214
+    // 48.4 and 32.2, three of 6000 to 3000 14.8 and 15.4; 2 heads, 30000 and 3000 18.0 and 20.1; fp32, 8 heads, 900, 2600 and
+    // 300 36.4 and 23.6.
+    const int64_t rows = p.kv_tokens * p.num_kv_heads * (p.k_stride_seq != 0 ? p.num_seqs : 1);     // kv_tokens is per sequence, or of all
+    if (p.num_seqs > 1 && p.kv_tokens > 0 && U <= kPlanUnits && U < sms &&
+        rows / (sms - (2 * U <= sms ? U / 2 : U)) + (!mma ? 50 : U < 8 ? 600 : 250) < (max_rows + fixed - 1) / fixed) {
         blocks = (int)sms;
         return kPlanned;
     }
-    // about one block per SM (one wave: prologue and merge are paid once), at least a 16-row block per warp
-    blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms / U, (max_rows + 127) / 128));
+    blocks = (int)fixed;
     return kFixed;
 }
 

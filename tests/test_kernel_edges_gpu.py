@@ -39,6 +39,44 @@ def test_short_units_from_keys_to_budgets(dtype, d, hq, hkv, w, lens):
         parity.run_fused_and_check(cfg, lay, rank_mode=rank_mode, scope=scope, threshold=0.05)
 
 
+@pytest.mark.parametrize("dtype,d,hq,hkv,w", [("fp32", 64, 8, 2, 16), ("fp32", 128, 3, 1, 11), ("bf16", 64, 4, 4, 1), ("bf16", 64, 2, 1, 32)])
+@pytest.mark.parametrize("layout", ["head_major", "token_major"])
+@pytest.mark.parametrize("q_offset", [0, 1])
+def test_short_units_score_as_in_a_longer_call(dtype, d, hq, hkv, w, layout, q_offset):
+    """A short call takes the cluster per unit, one with a long sequence more the three kernels: same bits for the sequences
+    that they share, whatever the order of the cache and wherever the queries start."""
+    cfg = cfg_like(num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype=dtype, window=w)
+    lens = [65, 1, 0, 127, 300, 600]
+    lay = workloads.make_layer(cfg, 0, seq_lens=lens, layout=layout)
+    if w == 1 and hq // hkv <= 16:
+        cfg = dataclasses.replace(cfg, window=2)                         # (a single row has a path of its own)
+        lay = workloads.make_layer(cfg, 0, seq_lens=lens, layout=layout)
+    p = binding.params_for(cfg, lay)
+    buf = torch.empty(lay.q_win.numel() + 8, dtype=lay.q_win.dtype, device=DEV)
+    q = buf[q_offset:q_offset + lay.q_win.numel()].view(lay.q_win.shape)
+    q.copy_(lay.q_win)
+    k, start, length = [t.to(DEV) for t in (lay.k, lay.seq_start, lay.seq_len)]
+    got = []
+    for seqs in (6, 5):
+        p.num_seqs, total = seqs, sum(lens[:seqs])
+        scores = torch.full((hkv, total), float("nan"), device=DEV)
+        ws = torch.empty(binding.refree_workspace_size(p, total), dtype=torch.uint8, device=DEV)
+        binding.refree_score(p, q[:seqs], k, start[:seqs], length[:seqs], total, scores, ws)
+        got.append(scores)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0][:, :sum(lens[:5])], got[1])
+
+
+@pytest.mark.parametrize("hq,hkv,dtype,d", [(8, 8, "bf16", 128), (4, 2, "bf16", 64), (28, 4, "bf16", 128), (8, 8, "fp32", 64)])
+@pytest.mark.parametrize("rows", [[9000, 100, 3000, 1, 700, 2500, 0, 1200, 40, 500, 4000, 900, 300], [3000, 40], [6000, 1500, 700]])
+def test_decode_of_lengths_that_differ(hq, hkv, dtype, d, rows):
+    """Units that a plan cuts in proportion to their rows: more units than half the SMs, a few, empty ones; two heads of a
+    sequence that keep different numbers of rows."""
+    from tests.test_decode_gpu import check_against_oracle
+    lengths = [max(0, r - 37 * g) for r in rows for g in range(hkv)]
+    check_against_oracle(len(rows), hq, hkv, d, dtype, lengths, seed=41, max_rows=max(rows), kv_tokens=sum(rows))
+
+
 @pytest.mark.parametrize("hq,hkv,d", [(8, 2, 128), (16, 1, 128), (12, 1, 64)])
 @pytest.mark.parametrize("lens", [[8193], [20_000, 255, 0, 257], [300] * 40])
 def test_single_query_row_beyond_the_short_calls(hq, hkv, d, lens):
