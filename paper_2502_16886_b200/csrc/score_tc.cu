@@ -840,7 +840,7 @@ __device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, int layer
     if (r < sh.R) {
         const float2 *rec = a.part_b + (int64_t)record_index(layer, c_lo, u, a.p.num_seqs * a.p.num_kv_heads) * 2 * sh.Rpad + r;
         const int nrec = 2 * (c_hi - c_lo + 1);             // records: (range, column half)
-        constexpr int kBatch = 12;                          // independent loads in flight per thread
+        constexpr int kBatch = 20;                          // independent loads in flight per thread: mostly all there are
         for (int s0 = sub; s0 < nrec; s0 += kBatch * per_row) {
             float2 pr[kBatch];
 #pragma unroll
@@ -848,18 +848,12 @@ __device__ inline bool merge_unit_lse(const TcArgs &a, TcSmemTail &tl, int layer
                 pr[q] = s0 + q * per_row < nrec ? __ldcg(rec + (int64_t)(s0 + q * per_row) * sh.Rpad) : make_float2(0.f, 0.f);
             // Z 2^M + y 2^x, record after record, at the larger of the two references.  What a step scales by depends on
             // the references alone, so the exponentials do not wait for the sums.
-            float f[kBatch];
-            unsigned grows = 0;
 #pragma unroll
             for (int q = 0; q < kBatch; ++q) {
                 const bool up = pr[q].y > 0.f && pr[q].x > M;
-                f[q] = ex2(up ? M - pr[q].x : pr[q].x - M);
-                if (up) { M = pr[q].x; grows |= 1u << q; }
-            }
-#pragma unroll
-            for (int q = 0; q < kBatch; ++q) {
-                const bool up = (grows >> q) & 1u;
-                if (pr[q].y > 0.f) Z = fmaf(up ? Z : pr[q].y, f[q], up ? pr[q].y : Z);
+                const float f = ex2(up ? M - pr[q].x : pr[q].x - M);
+                if (pr[q].y > 0.f) Z = fmaf(up ? Z : pr[q].y, f, up ? pr[q].y : Z);
+                if (up) M = pr[q].x;
             }
         }
     }
