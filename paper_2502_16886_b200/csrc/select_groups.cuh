@@ -103,6 +103,17 @@ struct UnitRule {
         }
         return INT_MAX;
     }
+    // rank count of the crossing inside the group of rank r, `base` being the sum before it, by a warp
+    __device__ inline int cross_group(int r, unsigned long long base, unsigned long long c_min) const
+    {
+        const int lane = threadIdx.x & 31, k = ng - 1 - r;
+        const int hi = min(n, 32 * k + 32) - 1, lo = max(lead, 32 * k);
+        const int pos = hi - lane;
+        const unsigned long long x = warp_incl_scan(pos >= lo ? square(pos) : 0ull);
+        const unsigned mp = __ballot_sync(0xffffffffu, pos >= lo && base + x >= c_min);
+        // rank count of position pos: the leading ones, then n-1 down to pos
+        return lead + (n - (mp ? hi - (__ffs(mp) - 1) : lo));
+    }
     // rank count of the crossing inside ranks [q0, q1) of the groups, `run` being the sum before them, by a warp
     __device__ inline int cross_run(int q0, int q1, unsigned long long run, unsigned long long c_min) const
     {
@@ -113,14 +124,8 @@ struct UnitRule {
             const unsigned long long vi = warp_incl_scan(v);
             const unsigned m = __ballot_sync(0xffffffffu, r < q1 && run + vi >= c_min);
             if (m) {
-                const int src = __ffs(m) - 1, k = ng - 1 - (rb + src);
-                const unsigned long long base = run + __shfl_sync(0xffffffffu, vi - v, src);
-                const int hi = min(n, 32 * k + 32) - 1, lo = max(lead, 32 * k);
-                const int pos = hi - lane;
-                const unsigned long long x = warp_incl_scan(pos >= lo ? square(pos) : 0ull);
-                const unsigned mp = __ballot_sync(0xffffffffu, pos >= lo && base + x >= c_min);
-                // rank count of position pos: the leading ones, then n-1 down to pos
-                return lead + (n - (mp ? hi - (__ffs(mp) - 1) : lo));
+                const int src = __ffs(m) - 1;
+                return cross_group(rb + src, run + __shfl_sync(0xffffffffu, vi - v, src), c_min);
             }
             run += __shfl_sync(0xffffffffu, vi, 31);
         }
@@ -187,7 +192,8 @@ __device__ inline void block_unit_rule(const UnitRule &ur, BlockRuleShared<NT> &
     const int owner = sh.first;
     if (owner != INT_MAX && (owner >> 5) == warp) {
         const u64 base = __shfl_sync(0xffffffffu, run_end - local, owner & 31);
-        jstar = ur.cross_run(min(ur.ng, owner * per), min(ur.ng, owner * per + per), base, c_min);
+        // (a group to a thread: the thread's run is the group, and its record need not be read again)
+        jstar = per == 1 ? ur.cross_group(owner, base, c_min) : ur.cross_run(min(ur.ng, owner * per), min(ur.ng, owner * per + per), base, c_min);
     }
     if (warp == (owner == INT_MAX ? 0 : owner >> 5) && lane == 0) store(ur.cut_at(jstar));
     __syncthreads();                                       // the shared words may be used again
