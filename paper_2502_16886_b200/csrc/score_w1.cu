@@ -694,7 +694,8 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
 template <int GMAX>
 cudaError_t run_w1_scores(W1Args &a, int layers, int64_t chunk_items, Stream st)
 {
-    // one wave of blocks over all layers: a block reads the unit's records (some 300 per head) before its first chunk
+    // One wave of blocks over all layers: a block reads the unit's records (some 300 per head) before its first chunk.  (A grid
+    // of four blocks an SM for every layer: 55 us for eight layers of 32K positions, 12 this way.)
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * 4 / layers));
     const cudaError_t e = launch_dependent(w1_scores_kernel<GMAX>, dim3(grid, layers), dim3(kThreadsW1), 0, st, a);
     count_launches(1);
