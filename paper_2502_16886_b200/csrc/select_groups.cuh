@@ -156,16 +156,39 @@ __device__ inline void block_unit_rule(const UnitRule &ur, BlockRuleShared<NT> &
     // groups in ranked order: thread t owns a contiguous run of ranks
     const int per = ceil_div(ur.ng, NT);
     const int r0 = min(ur.ng, tid * per), r1 = min(ur.ng, r0 + per);
-    u64 local = 0, sink;
+    constexpr int kRun = 4;                                // a short run's records are loaded together and kept
+    u64 local = 0, sink, kept[kRun] = {};
+    uint4 rec[kRun];
+    const bool short_run = per <= kRun;
+    if (short_run)
+#pragma unroll
+        for (int q = 0; q < kRun; ++q) rec[q] = r0 + q < r1 ? ur.record(r0 + q) : make_uint4(0u, 0u, 0u, 0u);
     const u64 lead_inc = warp_incl_scan(ur.lead <= 32 && lane < ur.lead ? ur.square(lane) : 0ull);     // (usually four positions)
     if (ur.lead <= 32) {
         sink = __shfl_sync(0xffffffffu, lead_inc, 31);     // all of them in the last-ranked group
-        for (int r = r0; r < r1; ++r) {
-            const u64 v = ur.whole(ur.record(r));
-            local += r < ur.ng - 1 ? v : (v > sink ? v - sink : 0ull);
+        auto rest = [&](const uint4 &x, int r) {
+            const u64 v = ur.whole(x);
+            return r < ur.ng - 1 ? v : (v > sink ? v - sink : 0ull);
+        };
+        if (short_run) {
+#pragma unroll
+            for (int q = 0; q < kRun; ++q) {
+                if (r0 + q < r1) kept[q] = rest(rec[q], r0 + q);
+                local += kept[q];
+            }
+        } else {
+            for (int r = r0; r < r1; ++r) local += rest(ur.record(r), r);
         }
     } else {
-        for (int r = r0; r < r1; ++r) local += ur.rest_of(ur.record(r), r);
+        if (short_run) {
+#pragma unroll
+            for (int q = 0; q < kRun; ++q) {
+                if (r0 + q < r1) kept[q] = ur.rest_of(rec[q], r0 + q);
+                local += kept[q];
+            }
+        } else {
+            for (int r = r0; r < r1; ++r) local += ur.rest_of(ur.record(r), r);
+        }
         sink = ur.sink_mass();                             // every warp for itself
     }
     const u64 inc = warp_incl_scan(local);
@@ -191,9 +214,19 @@ __device__ inline void block_unit_rule(const UnitRule &ur, BlockRuleShared<NT> &
     __syncthreads();
     const int owner = sh.first;
     if (owner != INT_MAX && (owner >> 5) == warp) {
-        const u64 base = __shfl_sync(0xffffffffu, run_end - local, owner & 31);
-        // (a group to a thread: the thread's run is the group, and its record need not be read again)
-        jstar = per == 1 ? ur.cross_group(owner, base, c_min) : ur.cross_run(min(ur.ng, owner * per), min(ur.ng, owner * per + per), base, c_min);
+        u64 base = run_end - local;                        // the sum before the thread's run
+        if (short_run) {                                   // the owner knows in which of its groups the sum crosses
+            int r = r0;
+#pragma unroll
+            for (int q = 0; q + 1 < kRun; ++q)
+                if (r == r0 + q && r + 1 < r1 && base + kept[q] < c_min) { base += kept[q]; ++r; }
+            base = __shfl_sync(0xffffffffu, base, owner & 31);
+            r = __shfl_sync(0xffffffffu, r, owner & 31);
+            jstar = ur.cross_group(r, base, c_min);
+        } else {
+            base = __shfl_sync(0xffffffffu, base, owner & 31);
+            jstar = ur.cross_run(min(ur.ng, owner * per), min(ur.ng, owner * per + per), base, c_min);
+        }
     }
     if (warp == (owner == INT_MAX ? 0 : owner >> 5) && lane == 0) store(ur.cut_at(jstar));
     __syncthreads();                                       // the shared words may be used again
