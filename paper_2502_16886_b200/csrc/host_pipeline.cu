@@ -215,6 +215,7 @@ refree_status refree_compress_layers_host(const refree_params *p, int32_t num_la
         cu(cudaStreamWaitEvent(hp.comp, ev.v_in, 0));
         job.k_out[0] = nullptr;
         job.v_out[0] = sl.vo;
+        job.offsets_out[0] = nullptr;                // (on their way to the host since k_done: read, not formed again)
         if (!cu(launch_compact(*p, job, d_start, d_len, ranges, capacity_rows, sl.status, hp.comp))) return;
         cu(cudaEventRecord(ev.v_done, hp.comp));
     };
