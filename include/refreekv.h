@@ -298,9 +298,10 @@ refree_status refree_compress_layer_host(const refree_params *p, const void *q_w
  *   arena    DEVICE buffer of refree_host_pipeline_arena_size() bytes, 256-byte
  *            aligned: two sets of staging buffers and one workspace
  * Index lists and scores are not returned (use the per-layer call for them).
- * The call creates and destroys its streams and events, blocks until every layer
- * is back in host memory, and returns the first error met (device-side
- * conditions as REFREE_ERR_CAPACITY / _TIMEOUT / _NONFINITE). */
+ * The call takes streams and events of its own (a few idle sets are kept for later
+ * calls in the same context), blocks until every layer is back in host memory, and
+ * returns the first error met (device-side conditions as REFREE_ERR_CAPACITY /
+ * _TIMEOUT / _NONFINITE). */
 refree_status refree_host_pipeline_arena_size(const refree_params *p, int64_t total_tokens, int64_t kv_elems,
                                               int64_t capacity_rows, size_t *bytes);
 refree_status refree_compress_layers_host(const refree_params *p, int32_t num_layers,

@@ -5,6 +5,8 @@
 // waits on the host but the row count: a kernel writes it into pinned memory behind the copy of K.  (The status word read into
 // pageable memory held the next layer's copies back: four layers of 8K positions 4.7 ms.  Rows written to host memory by the
 // copy kernel itself: 43 GB/s beside a copy in the other direction.)
+#include <cuda.h>
+
 #include <algorithm>
 #include <mutex>
 
@@ -28,17 +30,47 @@ __global__ void host_meta_kernel(const int64_t *rows, const int32_t *status, vol
     out->status = *status;
 }
 
-// Streams, events and the pinned words of one call.  Making them takes half a millisecond, so they are kept for the next call:
-// a call takes a set for itself and gives it back idle; a handful are kept, whatever the number of threads.
+// The context that the calling thread's work goes to.  The handle alone does not tell: after cudaDeviceReset the same handle
+// stands for another context, in which the old streams and events are gone; the number is never used again.
+struct Context {
+    CUcontext handle = nullptr;
+    unsigned long long id = 0;                       // 0: not known
+};
+Context current_context()
+{
+    typedef CUresult (*GetCurrent)(CUcontext *);
+    typedef CUresult (*GetId)(CUcontext, unsigned long long *);
+    static GetCurrent get_current = nullptr;
+    static GetId get_id = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        auto look_up = [](const char *name) {
+            void *fn = nullptr;
+            cudaDriverEntryPointQueryResult res;
+            return cudaGetDriverEntryPoint(name, &fn, cudaEnableDefault, &res) == cudaSuccess && res == cudaDriverEntryPointSuccess ? fn : nullptr;
+        };
+        get_current = reinterpret_cast<GetCurrent>(look_up("cuCtxGetCurrent"));
+        get_id = reinterpret_cast<GetId>(look_up("cuCtxGetId"));
+    });
+    Context c;
+    if (!get_current || !get_id) return c;
+    auto known = [&] { return get_current(&c.handle) == CUDA_SUCCESS && c.handle && get_id(c.handle, &c.id) == CUDA_SUCCESS; };
+    // a thread that has not called the runtime yet (or not since a reset) has no context until the device is set
+    int dev = 0;
+    if (known() || (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && known())) return c;
+    return {};
+}
+
+// Streams, events and the pinned words of one call.  Making them takes half a millisecond, so they are kept for the next call
+// in the same context: a call takes a set for itself and gives it back idle; a handful are kept, whatever the number of threads.
 struct HostPipe {
-    int dev = -1;
+    Context ctx;
     cudaStream_t in = nullptr, comp = nullptr, out = nullptr;
     struct { cudaEvent_t k_in, v_in, k_done, v_done, out_done; } ev[2] = {};
     HostMeta *meta = nullptr;                        // two, pinned
 
     bool make()
     {
-        if (cudaGetDevice(&dev) != cudaSuccess) return false;
         for (cudaStream_t *st : {&in, &comp, &out})
             if (cudaStreamCreateWithFlags(st, cudaStreamNonBlocking) != cudaSuccess) return false;
         for (auto &e : ev)
@@ -58,22 +90,24 @@ struct HostPipe {
 };
 constexpr int kKeptPipes = 4;
 std::mutex g_pipes_mutex;
-HostPipe g_pipes[kKeptPipes];                        // idle sets, of any device
+HostPipe g_pipes[kKeptPipes];                        // idle sets, of any context
 int g_num_pipes = 0;
 
 bool take_pipe(HostPipe &hp)
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    {
+    const Context ctx = current_context();
+    if (ctx.id) {
         std::lock_guard<std::mutex> hold(g_pipes_mutex);
-        for (int i = 0; i < g_num_pipes; ++i)
-            if (g_pipes[i].dev == dev) {
-                hp = g_pipes[i];
-                g_pipes[i] = g_pipes[--g_num_pipes];
-                return true;
-            }
+        for (int i = 0; i < g_num_pipes;) {
+            const Context &c = g_pipes[i].ctx;
+            const bool same = c.id == ctx.id;
+            if (same) hp = g_pipes[i];
+            // a set of a context that is gone (its handle stands for another now) is forgotten: its streams went with it
+            if (same || c.handle == ctx.handle) g_pipes[i] = g_pipes[--g_num_pipes]; else ++i;
+            if (same) return true;
+        }
     }
+    hp.ctx = ctx;
     if (hp.make()) return true;
     hp.destroy();
     return false;
@@ -81,7 +115,7 @@ bool take_pipe(HostPipe &hp)
 
 void give_pipe(HostPipe &hp, bool sound)
 {
-    if (sound) {
+    if (sound && hp.ctx.id) {
         std::lock_guard<std::mutex> hold(g_pipes_mutex);
         if (g_num_pipes < kKeptPipes) {
             g_pipes[g_num_pipes++] = hp;

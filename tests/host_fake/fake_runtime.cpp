@@ -16,6 +16,7 @@ static std::string g_log;
 static long g_next = 1;
 static std::set<long> g_live;                          // streams and events of the context that is current
 static unsigned long long g_ctx = 1;
+static bool g_bound = false;                           // whether the calling thread has a context
 static long long g_rows = 0;
 static int g_status = 0;
 
@@ -47,10 +48,10 @@ template <typename H> static cudaError_t drop(H h)
 extern "C" {
 const char *fake_log() { return g_log.c_str(); }
 void fake_reset(long long rows, int status) { g_log.clear(); g_rows = rows; g_status = status; }
-void fake_new_context() { ++g_ctx; g_live.clear(); }    // what cudaDeviceReset leaves: the same handle, another context
+void fake_new_context() { ++g_ctx; g_bound = false; g_live.clear(); }    // what cudaDeviceReset leaves: the same handle, another context
 long fake_live() { return (long)g_live.size(); }
 
-static CUresult ctx_current(CUcontext *c) { *c = reinterpret_cast<CUcontext>((intptr_t)0x1000); return CUDA_SUCCESS; }
+static CUresult ctx_current(CUcontext *c) { *c = reinterpret_cast<CUcontext>((intptr_t)(g_bound ? 0x1000 : 0)); return CUDA_SUCCESS; }
 static CUresult ctx_id(CUcontext, unsigned long long *id) { *id = g_ctx; return CUDA_SUCCESS; }
 cudaError_t cudaGetDriverEntryPoint(const char *name, void **fn, unsigned long long, cudaDriverEntryPointQueryResult *r)
 {
@@ -59,7 +60,7 @@ cudaError_t cudaGetDriverEntryPoint(const char *name, void **fn, unsigned long l
     return cudaSuccess;
 }
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
-cudaError_t cudaFree(void *) { return cudaSuccess; }
+cudaError_t cudaSetDevice(int) { g_bound = true; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = malloc(n); say("pinned %ld", num(*p)); return cudaSuccess; }
 cudaError_t cudaFreeHost(void *p) { say("unpinned %ld", num(p)); free(p); return cudaSuccess; }

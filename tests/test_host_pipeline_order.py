@@ -103,3 +103,22 @@ def test_no_two_streams_touch_the_same_bytes_unordered(pipeline, rank, layers):
     rc, log = pipeline.run(layers=layers, rank=rank)
     assert rc == 0 and sum(line.split()[2] == "rows" for line in log if line.startswith("op")) == 2 * layers
     assert races(log) == []
+
+
+def test_kept_streams_serve_the_next_call(pipeline):
+    pipeline.run()
+    first = pipeline.lib.fake_live()
+    rc, log = pipeline.run()
+    assert rc == 0 and pipeline.lib.fake_live() == first and not any(line.startswith(("pinned", "destroy")) for line in log)
+
+
+@pytest.mark.parametrize("status,error", [(binding.DEV_CAPACITY, binding.ERR_CAPACITY), (0, 0)])
+def test_streams_of_a_context_that_is_gone_are_not_touched(pipeline, status, error):
+    """After a reset of the device a call makes its own streams, once; what was kept before is neither used nor destroyed."""
+    assert pipeline.run(status=status)[0] == error
+    for _ in range(2):
+        pipeline.lib.fake_new_context()
+        for made in (True, False):
+            rc, log = pipeline.run()
+            assert rc == 0 and not any("dead" in line for line in log)
+            assert any(line.startswith("pinned") for line in log) == made
