@@ -848,14 +848,20 @@ unit_rules_kernel(refree_params p, const float *scores, const int32_t *seq_len, 
 // Offsets (running sum of lengths) and the kept positions of each unit, ascending.  Bound by latency: what a block adds up
 // (budgets before its unit, kept positions before its run, its own positions) meets in one barrier (32K positions x 8 heads x
 // 2 layers: 20 us with a block of kThreads and a scan for each).  With score ranking a block takes a run of kThreads
-// positions, four to a thread.
-constexpr int kEmitThreads = 256, kEmitWarps = kEmitThreads / 32, kPerThread = kThreads / kEmitThreads;
-static_assert(kPerThread * kEmitWarps == 32, "one count per lane");
-__global__ void __launch_bounds__(kEmitThreads)
+// positions, kThreads / NT to a thread.
+// Where the selection leaves no counts of a unit a block adds up the kept positions before its run itself, a chain of loads that
+// falls with the threads: one layer ranked across its heads, 256 and 1024 threads, us: 9481 positions x 8 heads 180 and 159,
+// 60000 x 2 267 and 174; per head without counts, 32000 x 8 59 and 40.  Blocks of short units are mostly beyond the end of their
+// sequence and cost what they hold of an SM: twelve of 1800 x 8 heads 30 and 42; 500 x 8 12.9 and 13.8.
+constexpr int kCountFrom = 2048;   // mean length from which blocks that count for themselves have 1024 threads
+template <int NT>
+__global__ void __launch_bounds__(NT)
 emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_t total_tokens,
             const __grid_constant__ SelectOut out, const Cut *cuts,
             int64_t capacity_rows, int32_t *dev_status, const int2 *chunk_counts, int chunk_stride, int counted_upto)
 {
+    constexpr int kEmitWarps = NT / 32, kPerThread = kThreads / NT;
+    static_assert(kPerThread * kEmitWarps == 32, "one count per lane");
     __shared__ long long s_len[kEmitWarps], s_before[kEmitWarps];      // per warp: budgets; (kept for sure << 32) + ties
     __shared__ int s_cnt[32];                                          // per 32 positions: (kept for sure << 16) + ties
     const int Hkv = p.num_kv_heads, U = p.num_seqs * Hkv;
@@ -891,29 +897,21 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
         v.n = n;
         if (v.heads == 1)
 #pragma unroll
-            for (int q = 0; q < kPerThread; ++q) near[q] = mag_bits(__ldcg(v.sc + min(chunk + q * kEmitThreads + (int)threadIdx.x, n - 1)));
+            for (int q = 0; q < kPerThread; ++q) near[q] = mag_bits(__ldcg(v.sc + min(chunk + q * NT + (int)threadIdx.x, n - 1)));
     }
     dependency_wait();
     const Cut cut = cuts[u];
     const int b = cut.b;
     long long part = 0, before = 0;
-    for (int t = threadIdx.x; t < u; t += kEmitThreads) part += lengths[t];
+    for (int t = threadIdx.x; t < u; t += NT) part += lengths[t];
     // kept for sure (above the crossing key, or protected and inside the budget) / at the crossing key, of
     // which the cut.ties lowest positions are kept
-    unsigned int smask[kPerThread], tmask[kPerThread];                 // of this warp's positions chunk + q kEmitThreads + threadIdx.x
+    unsigned int smask[kPerThread], tmask[kPerThread];                 // of this warp's positions chunk + q NT + threadIdx.x
     if (listed) {
         const int lead = v.lead, w_eff = v.w_eff;
         v.sbias = cut.sbias;
-        // the key is loaded first, without a branch around it, so that a thread's loads are in flight together
         const bool one_head = v.heads == 1;
-        auto key_of = [&](int i) {
-            if (one_head) {                       // a plain predicated load, so the loads of an unrolled loop overlap
-                const int ic = min(max(i, 0), n - 1);
-                const uint32_t bits = mag_bits(v.sc[ic]);
-                return (i >= lead && i < n - w_eff) ? (u64)bits << 32 : 0ull;
-            }
-            return (i >= lead && i < n - w_eff) ? key_at(v, i) : 0ull;
-        };
+        auto key_of = [&](int i) { return i >= lead && i < n - w_eff ? key_at(v, i) : 0ull; };      // of several heads
         auto classify = [&](int i, u64 key, bool &sure, bool &tie) {
             sure = false; tie = false;
             if (i >= n) return;
@@ -929,32 +927,42 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
         u64 key[kPerThread];
 #pragma unroll
         for (int q = 0; q < kPerThread; ++q) {
-            const int i = chunk + q * kEmitThreads + (int)threadIdx.x;
-            key[q] = !one_head ? key_of(i) : i >= lead && i < n - w_eff ? (u64)near[q] << 32 : 0ull;
+            const int i = chunk + q * NT + (int)threadIdx.x;
+            key[q] = one_head ? (u64)near[q] << 32 : key_of(i);
         }
         // What the positions before the chunk contribute: left per run of kThreads positions by the kernel that chose
         // the budget when it held the unit in registers; otherwise every block counts them itself (the scores are in L2).
         if (chunk_counts && n <= counted_upto) {
-            for (int c = threadIdx.x; c < (int)blockIdx.x; c += kEmitThreads) {
+            for (int c = threadIdx.x; c < (int)blockIdx.x; c += NT) {
                 const int2 cc = chunk_counts[(int64_t)u * chunk_stride + c];
                 before += ((long long)cc.x << 32) + (long long)cc.y;
             }
-        } else
-        for (int i0 = threadIdx.x; i0 < chunk; i0 += 8 * kEmitThreads) {
-            u64 k8[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) k8[q] = key_of(i0 + q * kEmitThreads < chunk ? i0 + q * kEmitThreads : n);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
+        } else {
+            auto count = [&](int i, u64 key) {
                 bool sure, tie;
-                classify(i0 + q * kEmitThreads < chunk ? i0 + q * kEmitThreads : n, k8[q], sure, tie);
+                classify(i < chunk ? i : n, key, sure, tie);
                 before += ((long long)sure << 32) + (long long)tie;
+            };
+            for (int i0 = threadIdx.x; i0 < chunk; i0 += 8 * NT) {
+                if (one_head) {                   // loads without a branch around them are in flight together
+                    uint32_t x[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) x[q] = mag_bits(__ldcg(v.sc + min(i0 + q * NT, n - 1)));
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) count(i0 + q * NT, (u64)x[q] << 32);
+                } else {
+                    u64 x[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) x[q] = key_of(i0 + q * NT < chunk ? i0 + q * NT : n);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) count(i0 + q * NT, x[q]);
+                }
             }
         }
 #pragma unroll
         for (int q = 0; q < kPerThread; ++q) {
             bool sure, tie;
-            classify(chunk + q * kEmitThreads + (int)threadIdx.x, key[q], sure, tie);
+            classify(chunk + q * NT + (int)threadIdx.x, key[q], sure, tie);
             smask[q] = __ballot_sync(0xffffffffu, sure);
             tmask[q] = __ballot_sync(0xffffffffu, tie);
             if (lane == 0) s_cnt[q * kEmitWarps + warp] = (__popc(smask[q]) << 16) + __popc(tmask[q]);
@@ -983,7 +991,7 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
     int32_t *dst = kept_idx + off;
     if (ranges) {
         const int head = min(b, min(p.sink, n));
-        for (int t = blockIdx.x * kEmitThreads + threadIdx.x; t < b; t += gridDim.x * kEmitThreads)
+        for (int t = blockIdx.x * NT + threadIdx.x; t < b; t += gridDim.x * NT)
             dst[t] = t < head ? t : n - b + t;
         return;
     }
@@ -998,7 +1006,7 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
         const int ties = ties_before + (x & 0xffff) + __popc(tmask[q] & lower);
         const int at = sure_before + (x >> 16) + __popc(smask[q] & lower) + min(ties, cut.ties);
         const bool keep = ((smask[q] >> lane) & 1u) || (((tmask[q] >> lane) & 1u) && ties < cut.ties);
-        if (keep && at < b) dst[at] = chunk + q * kEmitThreads + (int)threadIdx.x;
+        if (keep && at < b) dst[at] = chunk + q * NT + (int)threadIdx.x;
     }
 }
 
@@ -1150,14 +1158,15 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
     int gx = 1;
     if (ranges && kept_idx) {
         const int64_t per_unit = std::max<int64_t>(1, total_tokens / std::max(1, p.num_seqs));
-        gx = (int)std::min<int64_t>(64, (per_unit + 4 * kEmitThreads - 1) / (4 * kEmitThreads));
+        gx = (int)std::min<int64_t>(64, (per_unit + kThreads - 1) / kThreads);
     } else if (kept_idx) {
         // score ranking: a block per kThreads positions of the longest sequence there can be
         gx = (int)std::max<int64_t>(1, (total_tokens + kThreads - 1) / kThreads);
     }
-    const cudaError_t ee = launch_dependent(emit_kernel, dim3(gx, U, layers), dim3(kEmitThreads), 0, st, p, scores, seq_len, total_tokens,
-                                            out, cuts, capacity_rows, dev_status, chunk_counts,
-                                            chunk_stride, skip_upto);
+    const bool count = !ranges && kept_idx && (!chunk_counts || skip_upto < total_tokens) && total_tokens / std::max(1, p.num_seqs) >= kCountFrom;
+    auto *const kern = count ? emit_kernel<1024> : emit_kernel<256>;
+    const cudaError_t ee = launch_dependent(kern, dim3(gx, U, layers), dim3(count ? 1024 : 256), 0, st, p, scores, seq_len, total_tokens,
+                                            out, cuts, capacity_rows, dev_status, chunk_counts, chunk_stride, skip_upto);
     if (ee != cudaSuccess) return ee;
     count_launches(1);
     return cudaGetLastError();

@@ -133,6 +133,38 @@ def test_score_ranking_whatever_the_spread_of_the_scores(n, binades, threshold):
     assert kept[:want_b].cpu().tolist() == want
 
 
+@pytest.mark.parametrize("lens", [[2047], [2048], [1024, 3073], [5120, 1, 2049], [9000, 0, 1023]])
+@pytest.mark.parametrize("levels", [3, 1 << 20])
+def test_index_list_of_units_without_counts(lens, levels):
+    """Ranked per head the selection leaves counts where the workspace has room for them, in the built-in scratch there is none:
+    the same list, with ties at every step of the scores and without."""
+    n, units = sum(lens), 2 * len(lens)
+    scores = (torch.randint(1, levels + 1, (2, n), generator=torch.Generator().manual_seed(n + levels)).float() / levels).to(DEV)
+    p = binding.Params(num_seqs=len(lens), num_q_heads=2, num_kv_heads=2, head_dim=64, window=4, sink=2, threshold=0.1,
+                       rank_mode=binding.RANK_SCORE, dtype=binding.DTYPE_F32, kv_tokens=n, k_strides=(0, 64, n * 64),
+                       v_strides=(0, 64, n * 64))
+    length = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    ws = torch.empty(binding.refree_workspace_size(p, n), dtype=torch.uint8, device=DEV)
+    got = []
+    for static in (False, True):
+        out = [torch.zeros(units, dtype=torch.int32, device=DEV), torch.zeros(units + 1, dtype=torch.int64, device=DEV),
+               torch.full((2 * n,), -1, dtype=torch.int32, device=DEV)]
+        if static:
+            binding.refree_select_budget_static(p, scores, length, n, *out, 2 * n)
+        else:
+            binding.refree_select_budget(p, scores, length, n, *out, 2 * n, ws)
+        got.append([t.cpu() for t in out])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("lens", [[2048], [2049, 3000], [4097]])
+def test_index_list_of_a_layer_ranked_across_its_heads(lens):
+    cfg = cfg_like(num_q_heads=4, num_kv_heads=2, head_dim=64, dtype="fp32", window=8)
+    lay = workloads.make_layer(cfg, 0, seq_lens=lens)
+    parity.run_fused_and_check(cfg, lay, rank_mode=1, scope=1, threshold=0.1)
+
+
 def test_score_ranking_counts_scores_that_are_not_finite():
     n = 3000
     scores = torch.rand(1, n, generator=torch.Generator().manual_seed(3)) * 1e-3
