@@ -1096,10 +1096,14 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
         int nblk = 1;
         if (p.rank_mode == REFREE_RANK_SCORE && !p.force_full) {
             const int64_t avg = total_tokens / std::max(1, p.num_seqs);
-            // Blocks by the mean length (four layers one by one of 8 heads, us, with clusters of 1, 2, 4 and 8): 1100 positions 163,
-            // 186; 2100 -, 207, 209; 4100 -, -, 223, 235; 6000 -, -, 249, 259; staged calls on four sequences of 260 to 5120
-            // positions 325, 304, 296.
-            nblk = avg < 2048 ? 1 : avg < 8192 ? 4 : kMaxCluster;
+            // Blocks by the length.  One sequence, us of a selection of 8 heads with 1, 4 and 8 blocks to a unit: 2100 positions 17.2,
+            // 21.5, 24.9, 4100 21.4, 21.8, 25.2, 9500 31.9, 23.5, 25.5, 20000 71.5, 27.7, 26.3; ranked across the heads 2100 84, 103,
+            // 109, 4100 118, 135, 141, 9500 230, 153, 158, 20000 430, 234, 184.  Of several the mean is known and the longest is not:
+            // three of 3000 27.1, 22.7, 46.7, of 9000, 500 and 300 30.5, 23.4, 42.1.
+            if (p.num_seqs == 1)
+                nblk = avg <= 4096 ? 1 : avg <= 16384 ? 4 : kMaxCluster;
+            else
+                nblk = avg < 2048 ? 1 : avg < 8192 ? 4 : kMaxCluster;
             // One wave: a block takes an SM, and clusters leave some SMs of a group of them unused (16 units of 32K positions:
             // 61 us in clusters of eight, which came in two waves, 38 in clusters of four).
             // (But not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some

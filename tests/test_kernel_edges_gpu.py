@@ -133,7 +133,7 @@ def test_score_ranking_whatever_the_spread_of_the_scores(n, binades, threshold):
     assert kept[:want_b].cpu().tolist() == want
 
 
-@pytest.mark.parametrize("lens", [[2047], [2048], [1024, 3073], [5120, 1, 2049], [9000, 0, 1023]])
+@pytest.mark.parametrize("lens", [[2047], [2048], [4096], [4097], [16385], [1024, 3073], [5120, 1, 2049], [9000, 0, 1023]])
 @pytest.mark.parametrize("levels", [3, 1 << 20])
 def test_index_list_of_units_without_counts(lens, levels):
     """Ranked per head the selection leaves counts where the workspace has room for them, in the built-in scratch there is none:
