@@ -447,6 +447,7 @@ cudaError_t enqueue_selection(const refree_params &p, const void *q_win, const v
     // with two-range kept sets the copy forms the offsets and the index list itself: no launch for them (fp32 d 64, a layer of
     // 8 heads x 3000 positions with its list 81.3 -> 77.6 us, d 128, 1500 positions 40.5 -> 37.0)
     job = compact_job(k, v, lengths, offsets, ranges ? nullptr : kept, ranges ? offsets : nullptr, k_out, v_out, ranges ? kept : nullptr);
+    job.after_rule = ranges && !groups;
     return launch_select(p, sc, seq_len, total_tokens, select_out(lengths, offsets, kept), capacity_rows, ws, lay, device_status, cs,
                          !ranges, groups != nullptr);
 }

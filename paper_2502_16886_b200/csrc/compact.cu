@@ -338,11 +338,14 @@ compact_paged_kernel(refree_params p, const char *k, const char *v, const int32_
 // that moment, and those of one long unit end up side by side: 2 us of launch latency saved, but 129 us against 105 for a
 // copy of 250 MB out of a ragged batch (eight sequences of 92 to 19791 positions, 16 heads).  So only where the cache is
 // small enough for the latency to count.
-static Stream copy_stream(const refree_params &p, Stream st, int layers = 1)
+static int64_t cache_bytes(const refree_params &p, int layers)      // K and V; 0: the caller does not say
 {
     const int64_t rows = layers * p.kv_tokens * p.num_kv_heads * (p.k_stride_seq != 0 ? p.num_seqs : 1);
-    const int64_t bytes = rows * p.head_dim * (p.dtype == REFREE_DTYPE_F32 ? 8 : 4);      // K and V
-    return Stream(st.s, st.chain && bytes <= (int64_t)64 << 20);
+    return rows * p.head_dim * (p.dtype == REFREE_DTYPE_F32 ? 8 : 4);
+}
+static Stream copy_stream(const refree_params &p, Stream st, int layers = 1)
+{
+    return Stream(st.s, st.chain && cache_bytes(p, layers) <= (int64_t)64 << 20);
 }
 
 cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const int32_t *seq_start, const int32_t *seq_len,
@@ -355,9 +358,22 @@ cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const 
     // positions, 8 heads, 928 and 527; one layer of thirteen of 77 to 26835, 16 heads, 565 and 444 with its scoring; four
     // of eleven, ranked by score, 1089 and 1015; small copies would pay for the blocks, 18 and 25, and so would units of one
     // length, two of 16000 positions ranked by score 244 and 255).
-    const Stream cs = copy_stream(p, st, job.layers);
+    Stream cs = copy_stream(p, st, job.layers);
     const int per_sm = !cs.chain && (job.layers > 1 || p.num_seqs > 2) ? 32 : 8;
-    const int gx = max(1, (sm_count() * per_sm) / (U * job.layers));
+    int gx = max(1, (sm_count() * per_sm) / (U * job.layers));
+    // Position ranges: no more blocks than the longest unit there can be has rows for, two pieces to a thread; a block without
+    // rows waits, reads tables and budgets and holds the next launch up like the others.  And a copy of up to 32 MB behind a launch
+    // of the stopping rule, which fills an SM's shared memory, asks for the same split of it: an SM changes its split only when it
+    // is empty, so blocks that wait there for the rule to end kept the next call's scoring away.  (A layer with its list, us,
+    // without either, with the first, with both: bf16 d 64, 600 positions x 2 heads 24.5, 17.2, 17.2, 2000 x 4 34.7, 33.8, 28.9;
+    // six sequences of 69 to 2141 x 2 25.6, 22.4, 22.0; fp32 d 128, 1500 x 2 31.0, 30.4, 22.3; of 46 MB, 2800 x 16, 59.9, 60.3,
+    // 61.7.  Behind launches with little shared memory the split costs: a single query row, 20000 x 8 51.4 and 57.5.  Ranked by
+    // score, where few rows are kept, fewer blocks gain nothing: bf16 d 64, 1500 x 2 42.1 and 45.2.)
+    if (position_ranges && p.kv_tokens > 0) {
+        const int64_t pieces = std::min<int64_t>(p.kv_tokens, INT32_MAX) * p.head_dim * (p.dtype == REFREE_DTYPE_F32 ? 4 : 2) / 16;
+        gx = (int)std::min<int64_t>(gx, (pieces + 2 * kThreads - 1) / (2 * kThreads));
+    }
+    if (job.after_rule && cs.chain && cache_bytes(p, job.layers) <= (int64_t)32 << 20) cs.carveout = 100;
     const cudaError_t e = launch_dependent(compact_kernel, dim3(gx, U, job.layers), dim3(kThreads), 0,
                                            cs, p, job, seq_start, seq_len, ranges, capacity_rows, dev_status);
     count_launches(1);

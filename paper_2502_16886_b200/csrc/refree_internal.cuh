@@ -123,6 +123,7 @@ template <typename Tv> __device__ inline Tv warp_incl_scan(Tv x)
 struct Stream {
     cudaStream_t s;
     bool chain;
+    int carveout = -1;       // share of an SM's shared memory that the next launch asks for, percent
     Stream(cudaStream_t st, bool chained = true) : s(st), chain(chained) {}
     operator cudaStream_t() const { return s; }
 };
@@ -138,8 +139,12 @@ inline cudaError_t launch_dependent_cluster(void (*kernel)(P...), int cluster, d
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     int n = 0;
+    if (st.carveout >= 0) {
+        attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[n++].val.sharedMemCarveout = st.carveout;
+    }
     if (st.chain) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
@@ -266,6 +271,7 @@ struct CompactJob {
     int64_t *offsets_out[kMaxBatch];        // nullable: the kernel forms the running sum of the budgets itself
     int32_t *kept_out[kMaxBatch];           // nullable, position ranges: the kernel writes the index list
     char *k_out[kMaxBatch], *v_out[kMaxBatch];      // either null: those rows are not moved
+    bool after_rule;                        // behind a launch that chose the budgets from the scores (position ranking)
 };
 
 // The stopping rule of every unit from the records that the scoring left (position ranking per head).

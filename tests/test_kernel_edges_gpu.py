@@ -39,6 +39,17 @@ def test_short_units_from_keys_to_budgets(dtype, d, hq, hkv, w, lens):
         parity.run_fused_and_check(cfg, lay, rank_mode=rank_mode, scope=scope, threshold=0.05)
 
 
+@pytest.mark.parametrize("dtype,d", [("fp32", 64), ("fp32", 128), ("bf16", 64)])
+@pytest.mark.parametrize("lens", [[544], [577, 1], [33, 640, 0]])
+@pytest.mark.parametrize("extent", ["known", 0, 1 << 40])
+def test_rows_and_list_whatever_extent_the_caller_gives(dtype, d, lens, extent):
+    """The copy's grid follows the cache's extent: rows that end with a block's pieces and one more, an extent that is not given
+    and one far beyond."""
+    cfg = cfg_like(num_q_heads=4, num_kv_heads=2, head_dim=d, dtype=dtype, window=24)
+    lay = workloads.make_layer(cfg, 0, seq_lens=lens)
+    parity.run_fused_and_check(cfg, lay, rank_mode=0, threshold=0.05, **({} if extent == "known" else {"kv_tokens": extent}))
+
+
 @pytest.mark.parametrize("dtype,d,hq,hkv,w", [("fp32", 64, 8, 2, 16), ("fp32", 128, 3, 1, 11), ("bf16", 64, 4, 4, 1), ("bf16", 64, 2, 1, 32)])
 @pytest.mark.parametrize("layout", ["head_major", "token_major"])
 @pytest.mark.parametrize("q_offset", [0, 1])
