@@ -272,7 +272,9 @@ __device__ inline uint4 ld_row16(const char *p)
 // Bound by the stream over K.  The warps of one wave of blocks walk the spans of all layers of the group, and a warp asks for
 // the next 16 rows (of its next span too) before it works on those it has: a block per layer and piece of the grid, with the
 // rows of a step loaded and used in turn, kept HBM at 4.8 TB/s (eight layers of 32K positions x 8 heads, 107 us).
-template <int D, int NT>
+// AHEAD: the loads ahead.  Not with two column tiles of 128-element rows, whose registers they overflow (124 bytes of spills
+// inside the stream; two layers of 16000 and 15000 positions x 2 heads, groups of 16, 85.6 us with, 81.8 without).
+template <int D, int NT, bool AHEAD>
 __global__ void __launch_bounds__(kThreadsW1, 2)
 w1_logits_mma_kernel(const __grid_constant__ W1Args a)
 {
@@ -294,7 +296,7 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
     struct Span { W1Item it; int layer, end; const char *base; };
     auto span_of = [&](int64_t item) {
         Span sp;
-        sp.layer = (int)(item / per_layer);
+        sp.layer = a.layers > 1 ? (int)(item / per_layer) : 0;
         sp.it = decode_w1(tb, tb.spans, a.span, B, Hkv, (int)(item - (int64_t)sp.layer * per_layer));
         sp.end = min(sp.it.n, sp.it.pos0 + a.span);
         sp.base = static_cast<const char *>(a.k[sp.layer]) +
@@ -314,7 +316,7 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
     int64_t item = (int64_t)blockIdx.x * kWarpsW1 + warp;
     if (item >= items) return;
     Span sp = span_of(item);
-    load(sp, sp.it.pos0);
+    if (AHEAD) load(sp, sp.it.pos0);
     int cur_u = -1;
     uint4 qf[NT][CH];
     for (;;) {
@@ -340,21 +342,25 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
         float *unit_logits = logits + (int64_t)(it.g * G) * a.total_tokens + tb.pack[it.s];
         item += step;
         const bool more = item < items;
-        if (more) sp = span_of(item);                // the next span: its first rows are asked for under this one's last
+        if (AHEAD && more) sp = span_of(item);       // the next span: its first rows are asked for under this one's last
         float m[NT][2], z[NT][2];
 #pragma unroll
         for (int t = 0; t < NT; ++t) { m[t][0] = m[t][1] = -INFINITY; z[t][0] = z[t][1] = 0.f; }
         const char *const base = static_cast<const char *>(a.k[layer]) +
                                  ((int64_t)it.s * p.k_stride_seq + (int64_t)a.seq_start[it.s] * p.k_stride_tok + (int64_t)it.g * p.k_stride_head) * 2;
         const Span cur = {it, layer, end, base};
+#pragma unroll(AHEAD ? 1 : 2)
         for (int row0 = it.pos0; row0 < end; row0 += 16) {
             const int i0 = row0 + r, i1 = i0 + 8;
             const bool v0 = i0 < end, v1 = i1 < end;
             uint4 xa[CH], xb[CH];
+            if (!AHEAD) load(cur, row0);
 #pragma unroll
             for (int j = 0; j < CH; ++j) { xa[j] = ka[j]; xb[j] = kb[j]; }
-            if (row0 + 16 < end) load(cur, row0 + 16);
-            else if (more) load(sp, sp.it.pos0);
+            if (AHEAD) {
+                if (row0 + 16 < end) load(cur, row0 + 16);
+                else if (more) load(sp, sp.it.pos0);
+            }
             float acc[NT][4];
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
@@ -401,6 +407,7 @@ w1_logits_mma_kernel(const __grid_constant__ W1Args a)
                              it.chunk) * G + head] = make_float2(m[t][e], z[t][e]);
             }
         if (!more) break;
+        if (!AHEAD) sp = span_of(item);
     }
 }
 
@@ -585,8 +592,9 @@ w1_unit_kernel(const __grid_constant__ W1Args a, int stride)
     block_unit_rule<kThreadsUnit>(ur, rule, a.sel_lengths[layer] + u, a.sel_cuts + layer * p.num_seqs * Hkv + u);
 }
 
-template <int GMAX>
-__global__ void __launch_bounds__(kThreadsW1, GMAX <= 8 ? 4 : 2)
+// kAhead chunks of a block have their logits in flight together.
+template <int GMAX, int kAhead>
+__global__ void __launch_bounds__(kThreadsW1, GMAX > 8 ? 2 : GMAX <= 4 && kAhead == 1 ? 5 : 4)
 w1_scores_kernel(const __grid_constant__ W1Args a)
 {
     constexpr int kWarpsW1 = kThreadsW1 / 32;
@@ -644,19 +652,20 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
             __syncthreads();
         }
         // the run of this block's chunks inside the unit, kAhead of them at a time: their logits are in flight together
-        constexpr int kAhead = GMAX <= 4 ? 4 : 2;
         const int run = min(last - item, ceil_div(it.n, kChunk) - it.chunk);
         const float *const y = logits + (int64_t)(it.g * G) * a.total_tokens + tb.pack[it.s];
         float *const dst = scores + (int64_t)it.g * a.total_tokens + tb.pack[it.s];
         GroupPartial *const grp = groups ? groups + ((int64_t)tb.tiles[it.s] * Hkv + (int64_t)it.g * ceil_div(it.n, kTile)) * 4 : nullptr;
         for (int j0 = 0; j0 < run; j0 += kAhead) {
             float yl[kAhead][GMAX];
+            if constexpr (kAhead > 1) {
 #pragma unroll
-            for (int j = 0; j < kAhead; ++j) {
-                const int i = it.pos0 + (j0 + j) * kChunk + threadIdx.x;
+                for (int j = 0; j < kAhead; ++j) {
+                    const int i = it.pos0 + (j0 + j) * kChunk + threadIdx.x;
 #pragma unroll
-                for (int h = 0; h < GMAX; ++h)
-                    if (h < G) yl[j][h] = j0 + j < run && i < it.n ? y[(int64_t)h * a.total_tokens + i] : 0.f;
+                    for (int h = 0; h < GMAX; ++h)
+                        if (h < G) yl[j][h] = j0 + j < run && i < it.n ? y[(int64_t)h * a.total_tokens + i] : 0.f;
+                }
             }
 #pragma unroll
             for (int j = 0; j < kAhead; ++j) {
@@ -666,9 +675,13 @@ w1_scores_kernel(const __grid_constant__ W1Args a)
                 float sc = 0.f;
                 if (valid) {
                     float tot = 0.f;
+                    if constexpr (kAhead > 1) {
 #pragma unroll
-                    for (int h = 0; h < GMAX; ++h)
-                        if (h < G) tot += ex2(yl[j][h] - lse[h]);
+                        for (int h = 0; h < GMAX; ++h)
+                            if (h < G) tot += ex2(yl[j][h] - lse[h]);
+                    } else {
+                        for (int h = 0; h < G; ++h) tot += ex2(y[(int64_t)h * a.total_tokens + i] - lse[h]);
+                    }
                     sc = tot / (float)G;
                     if (!isfinite(sc) && a.dev_status) atomicOr(a.dev_status, REFREE_DEV_NONFINITE);
                     dst[i] = sc;
@@ -695,9 +708,14 @@ template <int GMAX>
 cudaError_t run_w1_scores(W1Args &a, int layers, int64_t chunk_items, Stream st)
 {
     // One wave of blocks over all layers: a block reads the unit's records (some 300 per head) before its first chunk.  (A grid
-    // of four blocks an SM for every layer: 55 us for eight layers of 32K positions, 12 this way.)
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * 4 / layers));
-    const cudaError_t e = launch_dependent(w1_scores_kernel<GMAX>, dim3(grid, layers), dim3(kThreadsW1), 0, st, a);
+    // of four blocks an SM for every layer: 55 us for eight layers of 32K positions, 12 this way; of four blocks of 16 heads, two of
+    // which an SM holds: four layers of 32K positions x 2 heads 176 us with the rest of the run, 136 this way.)
+    constexpr int kPerSm = GMAX > 8 ? 2 : 4;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunk_items, sm_count() * kPerSm / layers));
+    // Where a block has one chunk, and with 16 heads' logits to a chunk, one is enough, in a short body (fp32 d 64, 3000 positions
+    // x 2 heads, a layer 21.2 us with four, 20.7 with one; scoring of 9000 x 2, groups of 16, 23.2 and 21.1).
+    auto *kern = GMAX > 8 || chunk_items <= grid ? w1_scores_kernel<GMAX, 1> : w1_scores_kernel<GMAX, GMAX <= 4 ? 4 : GMAX <= 8 ? 2 : 1>;
+    const cudaError_t e = launch_dependent(kern, dim3(grid, layers), dim3(kThreadsW1), 0, st, a);
     count_launches(1);
     return e;
 }
@@ -721,7 +739,7 @@ cudaError_t run_w1_lanes(W1Args &a, int layers, int grid, Stream st, int G)
 template <int D>
 cudaError_t run_w1_mma(W1Args &a, int grid, Stream st, int G)
 {
-    auto *kern = G <= 8 ? w1_logits_mma_kernel<D, 1> : w1_logits_mma_kernel<D, 2>;
+    auto *kern = G <= 8 ? w1_logits_mma_kernel<D, 1, true> : w1_logits_mma_kernel<D, 2, D == 64>;
     const cudaError_t e = launch_dependent(kern, dim3(grid), dim3(kThreadsW1), 0, st, a);
     count_launches(1);
     return e;

@@ -96,6 +96,14 @@ def test_single_query_row_beyond_the_short_calls(hq, hkv, d, lens):
     parity.run_fused_and_check(cfg, lay, rank_mode=0)
 
 
+@pytest.mark.parametrize("hq,hkv,d,lens", [(16, 4, 128, [37_000, 200, 1]), (10, 2, 64, [76_000]), (24, 2, 128, [38_100, 90]), (32, 2, 64, [9000])])
+def test_single_query_row_of_more_chunks_than_blocks(hq, hkv, d, lens):
+    """A chunk to a block, several chunks of a unit and of two units to a block, with up to 4, 8 and 16 heads a group."""
+    cfg = cfg_like(num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype="bf16", window=1)
+    lay = workloads.make_layer(cfg, 1, seq_lens=lens)
+    parity.run_fused_and_check(cfg, lay, rank_mode=0)
+
+
 def _exact_rule(a, lead, w_eff, threshold):
     """Budget and kept positions of one unit ranked by score, by the documented integers (squares in fixed point, C_n in
     [2^60, 2^61))."""
