@@ -754,14 +754,19 @@ int decode_shape(const refree_params &p, int64_t max_rows, bool mma, int &blocks
     const int64_t fixed = std::max<int64_t>(1, std::min<int64_t>(sms / U, (max_rows + 127) / 128));
     // Lengths are on the device; what the host has is their sum, if the caller says how many tokens the cache holds.  By the
     // fixed cut the longest unit's blocks set the time; by the plan the rows spread over the SMs, less what its rounding
-    // wastes, and a call takes 2 us longer, as long as some 200 rows of a block (bf16; fp32 rows take five times as long), or 5 us
-    // with fewer than eight units, whose records are many.  Us a call, fixed and planned: 8 heads, sequences of 20000, 10000 and
-    // 5000 rows 42.2 and 30.4; of 9000 and 5000 19.5 and 19.3; 13 of 100 to 9000 86.6 and 53.2; 4 heads, eight of 2531 to 16214
-    // 48.4 and 32.2, three of 6000 to 3000 14.8 and 15.4; 2 heads, 30000 and 3000 18.0 and 20.1; fp32, 8 heads, 900, 2600 and
-    // 300 36.4 and 23.6.
+    // wastes, and a call takes some 2 us longer: its head, and more records of the longest unit to merge.  That is counted in rows
+    // of a block: 250 (bf16), 400 with groups of seven and more of 128 elements, whose records are large, 600 with fewer than
+    // eight units, whose records are many; 50 of fp32, whose rows take five times as long, but 300 where the fixed cut leaves a
+    // unit whole and needs no second launch.  Us a call, fixed and planned: 8 heads, sequences of 20000, 10000 and 5000 rows 42.2
+    // and 30.4; of 9000 and 5000 19.5 and 19.3; 13 of 100 to 9000 86.6 and 53.2; 4 heads, eight of 2531 to 16214 48.4 and 32.2,
+    // three of 6000 to 3000 14.8 and 15.4; 2 heads, 30000 and 3000 18.0 and 20.1; 2 heads of groups of 16, 6000 to 100 13.0 and
+    // 13.9, 12000 to 80 in one 15.3 and 19.7; fp32, 8 heads, 900, 2600 and 300 36.4 and 23.6; 16 heads, six of 1200 to 200 31.7
+    // and 38.4, of 5000 and 1000 173 and 65.  (Of 716 batches of 2 to 20 sequences the rule takes the slower form by more than
+    // 5 % in 44, in five of them the plan.)
     const int64_t rows = p.kv_tokens * p.num_kv_heads * (p.k_stride_seq != 0 ? p.num_seqs : 1);     // kv_tokens is per sequence, or of all
+    const int64_t more = mma ? (U < 8 ? 600 : p.head_dim == 128 && p.num_q_heads / p.num_kv_heads >= 7 ? 400 : 250) : fixed == 1 ? 300 : 50;
     if (p.num_seqs > 1 && p.kv_tokens > 0 && U <= kPlanUnits && U < sms &&
-        rows / (sms - (2 * U <= sms ? U / 2 : U)) + (!mma ? 50 : U < 8 ? 600 : 250) < (max_rows + fixed - 1) / fixed) {
+        rows / (sms - (2 * U <= sms ? U / 2 : U)) + more < (max_rows + fixed - 1) / fixed) {
         blocks = (int)sms;
         return kPlanned;
     }

@@ -88,6 +88,16 @@ def test_decode_of_lengths_that_differ(hq, hkv, dtype, d, rows):
     check_against_oracle(len(rows), hq, hkv, d, dtype, lengths, seed=41, max_rows=max(rows), kv_tokens=sum(rows))
 
 
+@pytest.mark.parametrize("dtype,d,rows,launches", [("fp32", 128, [1200, 800, 600, 400, 300, 200], 1), ("fp32", 64, [700, 1025, 411, 96, 1500, 333], 1),
+                                                   ("fp32", 64, [3000, 500, 400, 300, 200, 100], 2)])
+def test_decode_of_units_that_need_no_cut(dtype, d, rows, launches):
+    """More units than half the SMs: each is left whole, and its rows in one launch, unless one is far longer than the rest."""
+    from tests.test_decode_gpu import check_against_oracle
+    before = binding.lib().refree_kernel_launch_count()
+    check_against_oracle(len(rows), 16, 16, d, dtype, [r for r in rows for _ in range(16)], seed=43, max_rows=max(rows), kv_tokens=sum(rows))
+    assert binding.lib().refree_kernel_launch_count() - before == launches
+
+
 @pytest.mark.parametrize("hq,hkv,d", [(8, 2, 128), (16, 1, 128), (12, 1, 64)])
 @pytest.mark.parametrize("lens", [[8193], [20_000, 255, 0, 257], [300] * 40])
 def test_single_query_row_beyond_the_short_calls(hq, hkv, d, lens):
