@@ -238,15 +238,41 @@ __device__ __host__ inline int native_col(int idx, int native)
 }
 
 // Merge the warps' (max, sum, O) through shared memory in warp order and store the block's
-// result: the final output when the unit has one block, a record otherwise.  What a warp counts is worked out once per head.
-// sm: [NW][GP][D + 2] floats, then the block's own record [GP][D + 2] (cluster), then the factors [GP][NW + 1].
-template <int D, int NW>
+// result: the final output when the unit has one block, a record otherwise.  sm: [NW][GP][D + 2] floats, then the
+// block's own record [GP][D + 2] (cluster), then the factors [GP][NW + 1].
+// Two ways to the same bits: every thread works out what the warps count for its element, or that is done once per head and
+// shared, with a barrier more.  The first is faster while a thread has one element, the second beyond (bf16 d 64, groups of one,
+// 300 rows 4.23 and 4.33 us; fp32 d 64, groups of sixteen, five sequences of 1651 to 84 18.9 and 17.4).  fp32 rows of 64 in
+// groups of up to four have the first alone: beside the second their loop over the rows got slower (16 heads, eight sequences of
+// 2435 to 95 rows 40.0 and 41.7).
+enum Merge { kPerElement, kPerHead, kBySize };
+template <int D, int NW, Merge FORM>
 __device__ inline void merge_and_store(const DecArgs &a, float *sm, int GP, int G, const Piece &pc)
 {
     float *const fac = sm + (NW + 1) * GP * (D + 2);
     __syncthreads();
     const int Hkv = a.p.num_kv_heads, s = pc.u / Hkv, g = pc.u - s * Hkv;
     float *recs = a.mode == kCluster ? sm + NW * GP * (D + 2) : a.part + (int64_t)pc.rec * G * (D + 2);
+    if (FORM == kPerElement || (FORM == kBySize && G * (D + 2) <= 32 * NW)) {
+        for (int e = threadIdx.x; e < G * (D + 2); e += 32 * NW) {
+            const int h = e / (D + 2), idx = e % (D + 2);
+            float M = -INFINITY, L = 0.f, val = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) M = fmaxf(M, sm[(w * GP + h) * (D + 2) + D]);
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const float *rec = sm + (w * GP + h) * (D + 2);
+                const float f = rec[D] == -INFINITY ? 0.f : dec_ex2(rec[D] - M);
+                val += rec[idx < D ? idx : 0] * f;
+                L += rec[D + 1] * f;
+            }
+            if (pc.nblocks > 1)
+                recs[e] = idx < D ? val : (idx == D ? M : L);
+            else if (idx < D)
+                a.out[((int64_t)s * a.p.num_q_heads + g * G + h) * D + native_col(idx, a.native)] = L > 0.f ? val / L : 0.f;
+        }
+        return;
+    }
     if (threadIdx.x < G) {
         const int h = threadIdx.x;
         float m[NW], l[NW], M = -INFINITY, L = 0.f;
@@ -495,7 +521,7 @@ __device__ inline void decode_mma(const DecArgs &a, const Piece &pc, float *dec_
         }
         if (c == 0) { rec[D] = m[hh]; rec[D + 1] = l[hh]; }
     }
-    merge_and_store<D, NW>(a, dec_sm, GP, G, pc);
+    merge_and_store<D, NW, kBySize>(a, dec_sm, GP, G, pc);
 }
 
 // fp32 caches and unaligned bf16 pointers: a warp takes rows round-robin, every lane owns
@@ -582,7 +608,7 @@ __device__ inline void decode_lanes(const DecArgs &a, const Piece &pc, float *de
         for (int e = 0; e < E; ++e) rec[lane * E + e] = o[h][e];
         if (lane == 0) { rec[D] = m[h]; rec[D + 1] = l[h]; }
     }
-    merge_and_store<D, NW>(a, dec_sm, GMAX, G, pc);
+    merge_and_store<D, NW, (D == 64 && GMAX == 4 ? kPerElement : kPerHead)>(a, dec_sm, GMAX, G, pc);
 }
 
 // Every thread of the grid waits for what is ahead on the stream before it reads anything.  CLUSTER: a unit's blocks are a
