@@ -211,7 +211,6 @@ compact_inplace_back_kernel(refree_params p, char *k, char *v, const int32_t *se
     // Behind the selection of the same call everything but the budgets was complete before that began: tables and leading rows
     // are read while it drains (a thread has one piece of K and of V where they are few).
     if (!lengths) dependency_wait();
-    trigger_dependents();
     const int n = max(seq_len[s], 0), lead = min(p.sink, n);
     const int64_t tok0 = seq_start[s];
     char *kb = k + ((int64_t)s * p.k_stride_seq + tok0 * p.k_stride_tok + (int64_t)g * p.k_stride_head) * esz;
@@ -226,6 +225,9 @@ compact_inplace_back_kernel(refree_params p, char *k, char *v, const int32_t *se
     };
     if (mine) load(threadIdx.x);
     if (lengths) dependency_wait();
+    // (after the wait: blocks of the next call that came earlier would sit on SMs that the selection still needs; fp32 d 64, six
+    // sequences of 80 to 641 positions x 8 heads 30.5 us, 27.3 this way)
+    trigger_dependents();
     int64_t off, b64;
     if (lengths) {
         // fused pass: budgets come straight from the selection, and the running sum is formed here
