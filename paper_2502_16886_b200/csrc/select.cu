@@ -1105,15 +1105,20 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
             else
                 nblk = avg < 2048 ? 1 : avg < 8192 ? 4 : kMaxCluster;
             // One wave: a block takes an SM, and clusters leave some SMs of a group of them unused (16 units of 32K positions:
-            // 61 us in clusters of eight, which came in two waves, 38 in clusters of four).
-            // (But not where that takes a sequence out of the register-resident kernel's reach: the general kernel needs some
-            // 100 us for it: eleven sequences of 69 to 29809 positions, 8 heads, four layers 1428 -> 1015.)
+            // 61 us in clusters of eight, which came in two waves, 38 in clusters of four; nine sequences of 13095 to 147, 8 heads,
+            // 78 in fours, 60 in twos; sixteen of 2500, 8 heads, 118 and 92).
+            // (But clusters of two, and of one for every 4096 positions of the mean, stay where fewer blocks take a sequence out of
+            // the register-resident kernel's reach: the general kernel needs some 100 us for it: eleven sequences of 69 to 29809
+            // positions, 8 heads, four layers 1428 -> 1015; nine of 20000 to 50, 8 heads, two layers 245 one by one, 172 in twos.)
             const bool resident = p.scope == REFREE_SCOPE_HEAD;
+            int least = 2;
+            while (least < kMaxCluster && avg >= (int64_t)least * 4096) least *= 2;
             for (; nblk > 1; nblk /= 2) {
                 shape(nblk);
                 const int room = cluster_room(0, nblk, select_budget_kernel, cfg);
                 if (room == 0) continue;
-                if ((int64_t)sel_units * layers <= room || (resident && (int64_t)(nblk / 2) * kThreads * 16 < total_tokens)) break;
+                if ((int64_t)sel_units * layers <= room ||
+                    (resident && nblk <= least && (int64_t)(nblk / 2) * kThreads * 16 < total_tokens)) break;
             }
         }
         shape(nblk);
