@@ -486,7 +486,7 @@ template <int E>
 __global__ void __launch_bounds__(kThreads)
 select_score_resident_kernel(refree_params p, const float *scores, const int32_t *seq_len,
                              int64_t total_tokens, const __grid_constant__ SelectOut out, Cut *cuts, int32_t *dev_status,
-                             int2 *chunk_counts, int chunk_stride)
+                             int2 *chunk_counts, int chunk_stride, int from)
 {
     extern __shared__ __align__(16) unsigned char select_smem_raw[];
     SelectSmem &sm = *reinterpret_cast<SelectSmem *>(select_smem_raw);
@@ -506,10 +506,14 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
             (&sm.wsum[0][0])[t] = 0ull;
         }
     };
-    clear_hist();                                    // (before the wait for the scores)
+    if (from == 0) clear_hist();                     // (before the wait for the scores)
     if (threadIdx.x == 0) sm.z_key = 0u;
     dependency_wait();
     trigger_dependents();
+    if (from > 0) {                                  // units up to that length are not this launch's
+        if (max(seq_len[s], 0) <= from) return;
+        clear_hist();
+    }
     if (warp == 0) {
         int a = 0;
         for (int t = lane; t < s; t += 32) a += max(seq_len[t], 0);
@@ -518,7 +522,7 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
     }
     __syncthreads();
     const int n = max(seq_len[s], 0);
-    if (n > nblk * kThreads * E) return;             // too long to hold: select_budget_kernel takes it
+    if (n > nblk * kThreads * E) return;             // too long to hold: a launch of larger clusters or select_budget_kernel takes it
     // elements of this block that lie inside the sequence: a batch sized for its longest sequence leaves most of
     // a short one's element slots empty, and the loops below skip them (the same for every thread of the block)
     const int e_lim = min(E, ceil_div(max(n - rank * kThreads, 0), nblk * kThreads));
@@ -1106,19 +1110,10 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
                 nblk = avg < 2048 ? 1 : avg < 8192 ? 4 : kMaxCluster;
             // One wave: a block takes an SM, and clusters leave some SMs of a group of them unused (16 units of 32K positions:
             // 61 us in clusters of eight, which came in two waves, 38 in clusters of four; nine sequences of 13095 to 147, 8 heads,
-            // 78 in fours, 60 in twos; sixteen of 2500, 8 heads, 118 and 92).
-            // (But clusters of two, and of one for every 4096 positions of the mean, stay where fewer blocks take a sequence out of
-            // the register-resident kernel's reach: the general kernel needs some 100 us for it: eleven sequences of 69 to 29809
-            // positions, 8 heads, four layers 1428 -> 1015; nine of 20000 to 50, 8 heads, two layers 245 one by one, 172 in twos.)
-            const bool resident = p.scope == REFREE_SCOPE_HEAD;
-            int least = 2;
-            while (least < kMaxCluster && avg >= (int64_t)least * 4096) least *= 2;
+            // 78 in fours, 41 one by one, as below; sixteen of 2500, 8 heads, 118 and 36).
             for (; nblk > 1; nblk /= 2) {
                 shape(nblk);
-                const int room = cluster_room(0, nblk, select_budget_kernel, cfg);
-                if (room == 0) continue;
-                if ((int64_t)sel_units * layers <= room ||
-                    (resident && nblk <= least && (int64_t)(nblk / 2) * kThreads * 16 < total_tokens)) break;
+                if (const int room = cluster_room(0, nblk, select_budget_kernel, cfg); room > 0 && (int64_t)sel_units * layers <= room) break;
             }
         }
         shape(nblk);
@@ -1133,27 +1128,31 @@ cudaError_t launch_select(const refree_params &p, const float *scores, const int
             while (E < 16 && (int64_t)rb * kThreads * E < want) E *= 2;
             cudaLaunchConfig_t rc = cfg;
             cudaLaunchAttribute rattr[2] = {attr[0], attr[1]};
-            rattr[0].val.clusterDim.x = rb;
             rc.attrs = rattr;
-            rc.gridDim = dim3(sel_units * rb, layers);
-            cudaError_t re = cudaErrorInvalidValue;
-            auto fits = [&](auto kern) { return rb == 1 || cluster_room(E, rb, kern, rc) > 0; };
             // counts per run of kThreads positions for the index list, where the caller's workspace has room for them
             if (emit && kept_idx && lay.part_bytes >= (size_t)U * layers * (size_t)chunk_stride * sizeof(int2))
                 chunk_counts = reinterpret_cast<int2 *>(ws + lay.part_off);
-            if (E == 4 && fits(select_score_resident_kernel<4>))
-                re = cudaLaunchKernelEx(&rc, select_score_resident_kernel<4>, p, scores, seq_len, total_tokens, out, cuts, dev_status, chunk_counts, chunk_stride);
-            else if (E == 8 && fits(select_score_resident_kernel<8>))
-                re = cudaLaunchKernelEx(&rc, select_score_resident_kernel<8>, p, scores, seq_len, total_tokens, out, cuts, dev_status, chunk_counts, chunk_stride);
-            else if (E == 16 && fits(select_score_resident_kernel<16>))
-                re = cudaLaunchKernelEx(&rc, select_score_resident_kernel<16>, p, scores, seq_len, total_tokens, out, cuts, dev_status, chunk_counts, chunk_stride);
-            if (re == cudaSuccess) {
-                skip_upto = rb * kThreads * E;
+            // units longer than skip_upto, up to what clusters of `blocks` hold
+            auto hold = [&](auto kern, int blocks, int elems) {
+                rattr[0].val.clusterDim.x = blocks;
+                rc.gridDim = dim3(sel_units * blocks, layers);
+                if (blocks > 1 && cluster_room(elems, blocks, kern, rc) < 1) return false;
+                if (cudaLaunchKernelEx(&rc, kern, p, scores, seq_len, total_tokens, out, cuts, dev_status, chunk_counts, chunk_stride,
+                                       skip_upto) != cudaSuccess) {
+                    (void)cudaGetLastError();
+                    return false;
+                }
+                skip_upto = blocks * kThreads * elems;
                 count_launches(1);
-            } else {
-                (void)cudaGetLastError();
-                chunk_counts = nullptr;
-            }
+                return true;
+            };
+            const bool held = E == 4 ? hold(select_score_resident_kernel<4>, rb, 4) : E == 8 ? hold(select_score_resident_kernel<8>, rb, 8)
+                                                                                        : hold(select_score_resident_kernel<16>, rb, 16);
+            if (!held) chunk_counts = nullptr;
+            // Longer ones by the same kernel in clusters of four: the others leave it at once (2 us), and the general kernel takes
+            // some 100 us for a unit (selection, 8 heads, us with it and this way: sequences of 17386 to 64 84 and 59, of 25000 and
+            // twelve of 1000 83 and 63).
+            if (held && rb < 4 && skip_upto < total_tokens) hold(select_score_resident_kernel<16>, 4, 16);
         }
         if (skip_upto == 0 || (int64_t)skip_upto < total_tokens) {
             const cudaError_t le = cudaLaunchKernelEx(&cfg, select_budget_kernel, p, scores, seq_len, total_tokens, out,

@@ -187,6 +187,14 @@ def test_index_list_of_units_without_counts(lens, levels):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("lens", [[16_384] + [100] * 9, [90] * 8 + [16_385, 3000], [66_000] + [70] * 40, [0, 65_536] + [64] * 39])
+def test_score_ranking_of_a_long_unit_among_many_short_ones(lens):
+    """Units that one block holds, the next longer, the longest that four hold and one beyond: three kernels share a call."""
+    cfg = cfg_like(num_q_heads=2, num_kv_heads=2, head_dim=64, dtype="bf16", window=1)
+    lay = workloads.make_layer(cfg, 0, seq_lens=lens)
+    parity.run_fused_and_check(cfg, lay, rank_mode=1, threshold=0.1)
+
+
 @pytest.mark.parametrize("lens", [[2048], [2049, 3000], [4097]])
 def test_index_list_of_a_layer_ranked_across_its_heads(lens):
     cfg = cfg_like(num_q_heads=4, num_kv_heads=2, head_dim=64, dtype="fp32", window=8)
