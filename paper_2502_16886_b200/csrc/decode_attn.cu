@@ -521,7 +521,7 @@ __device__ inline void decode_mma(const DecArgs &a, const Piece &pc, float *dec_
         }
         if (c == 0) { rec[D] = m[hh]; rec[D + 1] = l[hh]; }
     }
-    merge_and_store<D, NW, kBySize>(a, dec_sm, GP, G, pc);
+    merge_and_store<D, NW, (D == 64 ? kBySize : kPerHead)>(a, dec_sm, GP, G, pc);
 }
 
 // fp32 caches and unaligned bf16 pointers: a warp takes rows round-robin, every lane owns
