@@ -742,8 +742,8 @@ refree_status refree_compress_layers(const refree_params *p, int32_t num_layers,
             }
             return t;
         };
-        // the first launch of the run is an ordinary one: its warps read Q and K before they wait for what is ahead of it
-        // on the stream, which may still be writing them
+        // The first launch of the run is chained to what is ahead of it on the stream, which may still be writing Q and K: it
+        // waits before it reads anything.  The launches behind it read Q and K before their wait.
         for (int j = 0; j <= ngroups; ++j) {
             TcGroup beg, fin;
             TcCopyJob job = {};

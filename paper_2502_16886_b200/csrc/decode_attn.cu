@@ -617,7 +617,7 @@ template <int D, int GP, int NW, bool CLUSTER, typename Body>
 __device__ inline void decode_block(const DecArgs &a, float *dec_sm, Body body)
 {
     dependency_wait();
-    trigger_dependents();
+    trigger_dependents();                            // behind the wait: the merge reads the lengths before its own
     Piece pc;
     int64_t lo_k = 0, lo_v = 0, len64 = 0;
     if (a.mode == kPlanned) {

@@ -113,10 +113,14 @@ template <typename Tv> __device__ inline Tv warp_incl_scan(Tv x)
 // ---- dependent launches ------------------------------------------------------
 // Every kernel of a call may be launched while the kernel before it on the stream drains (programmatic dependent
 // launch), which takes the launch latency out of a chain of short kernels.  Rules that keep this safe:
-//   - every thread that touches memory calls dependency_wait() first (at least one thread of the grid must, on every
-//     path, so that the end of a kernel means the end of all before it);
-//   - the first kernel of a call triggers its dependents after that wait, later ones may do so at once: what a kernel
-//     reads before its wait (sequence tables, queries, keys: inputs of the call) was complete before the first one.
+//   - nothing is written to global memory before dependency_wait(), and at least one thread of the grid waits on every path,
+//     so that the end of a kernel means the end of all before it;
+//   - the first kernel of a call triggers its dependents after its wait, later ones may do so at once: the inputs of the call
+//     (sequence tables, queries, keys, values) were complete before the first one and may be read before any wait;
+//   - a result of an earlier kernel of the call may be read before the wait only behind a kernel that triggers after its own:
+//     what was ahead of that one is complete then.  (The index list reads scores this way, behind the two kernels of score
+//     ranking, the merge of the decode step the lengths, behind its attention kernel; the triggers that must stay behind their
+//     waits say so.)
 // A stream, and whether the next launch on it may be chained this way.  Also where a second stream works beside it (a run
 // of layers on two streams, us, chained and not: fp32 d 64, eight layers of 3000 positions, 32 rows, 208 and 287; bf16 d 64,
 // four of 32K 325 and 370; windows in chunks, six layers of 2000 positions, 1200 rows, 766 and 841).

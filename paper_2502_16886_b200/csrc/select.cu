@@ -305,7 +305,7 @@ select_budget_kernel(refree_params p, const float *scores, const int32_t *seq_le
     cuts += blockIdx.y * p.num_seqs * Hkv;
     int32_t *const lengths = out.lengths[blockIdx.y];
     dependency_wait();
-    trigger_dependents();
+    trigger_dependents();                            // behind the wait: emit_kernel reads the scores before its own
     if (skip_upto > 0 && max(seq_len[s], 0) <= skip_upto) return;      // the register-resident kernel takes these (the whole cluster leaves)
     if (threadIdx.x == 0) {
         int a = 0;
@@ -509,7 +509,7 @@ select_score_resident_kernel(refree_params p, const float *scores, const int32_t
     if (from == 0) clear_hist();                     // (before the wait for the scores)
     if (threadIdx.x == 0) sm.z_key = 0u;
     dependency_wait();
-    trigger_dependents();
+    trigger_dependents();                            // behind the wait: emit_kernel reads the scores before its own
     if (from > 0) {                                  // units up to that length are not this launch's
         if (max(seq_len[s], 0) <= from) return;
         clear_hist();
@@ -878,8 +878,8 @@ emit_kernel(refree_params p, const float *scores, const int32_t *seq_len, int64_
     int64_t *const offsets = out.offsets[blockIdx.z];
     int32_t *const kept_idx = out.kept[blockIdx.z];
     trigger_dependents();
-    // The selection before this launch triggered it after its own wait: lengths and scores were complete by then, and are read
-    // before the wait for the selection.
+    // The selection before this launch triggered it after its own wait: tables and scores were complete by then, and are read
+    // before the wait for the selection (the scores from L2).
     const int n = max(seq_len[s], 0), chunk = blockIdx.x * kThreads;
     const bool ranges = p.rank_mode == REFREE_RANK_POSITION || p.force_full;
     // score ranking: a block beyond the end of its sequence has nothing to do (the grid is sized for the longest

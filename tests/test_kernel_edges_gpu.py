@@ -114,6 +114,15 @@ def test_single_query_row_of_more_chunks_than_blocks(hq, hkv, d, lens):
     parity.run_fused_and_check(cfg, lay, rank_mode=0)
 
 
+@pytest.mark.parametrize("group,w", [(1, 257), (4, 65), (4, 75), (3, 110), (2, 192), (4, 100), (7, 64), (1, 449), (7, 73), (2, 17), (5, 13), (1, 130)])
+def test_query_rows_that_do_not_fill_their_products(group, w):
+    """Row blocks of 128 and column products of 256 with rows to spare: warps of the row pass without rows, chunks of the column
+    pass without rows, a second product that is padded; a tile before the window, tiles inside it, one position."""
+    cfg = cfg_like(num_q_heads=2 * group, num_kv_heads=2, head_dim=128, dtype="bf16", window=w)
+    lay = workloads.make_layer(cfg, 2, seq_lens=[700, 129, 1])
+    parity.run_fused_and_check(cfg, lay, rank_mode=0, threshold=0.05)
+
+
 def _exact_rule(a, lead, w_eff, threshold):
     """Budget and kept positions of one unit ranked by score, by the documented integers (squares in fixed point, C_n in
     [2^60, 2^61))."""
