@@ -363,17 +363,19 @@ cudaError_t launch_compact(const refree_params &p, const CompactJob &job, const 
     Stream cs = copy_stream(p, st, job.layers);
     const int per_sm = !cs.chain && (job.layers > 1 || p.num_seqs > 2) ? 32 : 8;
     int gx = max(1, (sm_count() * per_sm) / (U * job.layers));
-    // Position ranges: no more blocks than the longest unit there can be has rows for, two pieces to a thread; a block without
-    // rows waits, reads tables and budgets and holds the next launch up like the others.  And a copy of up to 32 MB behind a launch
-    // of the stopping rule, which fills an SM's shared memory, asks for the same split of it: an SM changes its split only when it
-    // is empty, so blocks that wait there for the rule to end kept the next call's scoring away.  (A layer with its list, us,
-    // without either, with the first, with both: bf16 d 64, 600 positions x 2 heads 24.5, 17.2, 17.2, 2000 x 4 34.7, 33.8, 28.9;
-    // six sequences of 69 to 2141 x 2 25.6, 22.4, 22.0; fp32 d 128, 1500 x 2 31.0, 30.4, 22.3; of 46 MB, 2800 x 16, 59.9, 60.3,
-    // 61.7.  Behind launches with little shared memory the split costs: a single query row, 20000 x 8 51.4 and 57.5.  Ranked by
-    // score, where few rows are kept, fewer blocks gain nothing: bf16 d 64, 1500 x 2 42.1 and 45.2.)
+    // Position ranges: no more blocks than the longest unit there can be has rows for, two pieces to a thread, four behind a launch
+    // of the stopping rule; a block without rows waits, reads tables and budgets and holds the next launch up like the others.  And
+    // a copy of up to 32 MB behind such a launch, which fills an SM's shared memory, asks for the same split of it: an SM changes
+    // its split only when it is empty, so blocks that wait there for the rule to end kept the next call's scoring away.  (A layer
+    // with its list, us, without either, with the first, with both: bf16 d 64, 600 positions x 2 heads 24.5, 17.5, 17.5, 2000 x 4
+    // 34.7, 35.4, 31.2; fp32 d 128, 1500 x 2 31.0, 22.7, 22.4; of 46 MB, 2800 x 16, 59.9, 60.3, 61.7; 112 such calls on average 8.7 %
+    // less.  Behind launches with little shared memory the split costs: a single query row, 20000 x 8 51.4 and 57.5; two pieces and
+    // four there: 700 x 4 of it 9.9 and 10.6.  Ranked by score, where few rows are kept, fewer blocks gain nothing: bf16 d 64,
+    // 1500 x 2 42.1 and 45.2.)
     if (position_ranges && p.kv_tokens > 0) {
         const int64_t pieces = std::min<int64_t>(p.kv_tokens, INT32_MAX) * p.head_dim * (p.dtype == REFREE_DTYPE_F32 ? 4 : 2) / 16;
-        gx = (int)std::min<int64_t>(gx, (pieces + 2 * kThreads - 1) / (2 * kThreads));
+        const int64_t per_block = (int64_t)kThreads * (job.after_rule ? 4 : 2);
+        gx = (int)std::min<int64_t>(gx, (pieces + per_block - 1) / per_block);
     }
     if (job.after_rule && cs.chain && cache_bytes(p, job.layers) <= (int64_t)32 << 20) cs.carveout = 100;
     const cudaError_t e = launch_dependent(compact_kernel, dim3(gx, U, job.layers), dim3(kThreads), 0,
